@@ -803,23 +803,38 @@ __device__ __forceinline__ void issue_land(T *land, const T *__restrict__ src, c
         }
         return;
     }
+    // a warp takes whole rows, all planes of one row at a time; the closing column apart
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nzp = min(NPL, f.n[0] - s.g0[0] - Z0);
     const int nyr = min(EY, f.n[1] - s.g0[1]);
     const int nxc = min(EX, f.n[2] - s.g0[2]);
-    for (int r = warp; r < nzp * EY; r += NWARP) {
-        const int pz = r / EY, y = r % EY;
-        if (y >= nyr) continue;
-        const T *row = src + ((size_t)(s.g0[0] + Z0 + pz) * f.n[1] + s.g0[1] + y) * f.n[2] + s.g0[2];
-        T *dst = land + r * P;
-        if (sizeof(T) == 4) {
-            if (lane < nxc) cp_async4(dst + lane, row + lane);
-            if (lane == 0 && nxc > 32) cp_async4(dst + 32, row + 32);
-        } else {
-            if (lane < nxc) dst[lane] = row[lane];
-            if (lane == 0 && nxc > 32) dst[32] = row[32];
+    const size_t plane = (size_t)f.n[1] * f.n[2];
+    const T *src0 = src + ((size_t)(s.g0[0] + Z0) * f.n[1] + s.g0[1]) * f.n[2] + s.g0[2];
+    for (int y = warp; y < nyr; y += NWARP) {
+        const T *row = src0 + (size_t)y * f.n[2] + lane;
+        T *dst = land + y * P + lane;
+        if (lane < nxc) {
+            if constexpr (sizeof(T) == 4) {
+#pragma unroll
+                for (int pz = 0; pz < NPL; ++pz)
+                    if (pz < nzp) cp_async4(dst + pz * EY * P, row + pz * plane);
+            } else {
+                T v[NPL];
+#pragma unroll
+                for (int pz = 0; pz < NPL; ++pz) v[pz] = pz < nzp ? __ldg(row + pz * plane) : (T)0;
+#pragma unroll
+                for (int pz = 0; pz < NPL; ++pz) dst[pz * EY * P] = v[pz];
+            }
         }
     }
+    if (nxc > OX)
+        for (int r = NT - 1 - (int)threadIdx.x; r < NPL * EY; r += NT) {
+            const int pz = r / EY, y = r - pz * EY;
+            if (pz >= nzp || y >= nyr) continue;
+            const T *one = src0 + pz * plane + (size_t)y * f.n[2] + OX;
+            if constexpr (sizeof(T) == 4) cp_async4(land + r * P + OX, one);
+            else land[r * P + OX] = __ldg(one);
+        }
     cp_async_commit();
 }
 
@@ -916,7 +931,49 @@ __device__ __forceinline__ void write_slab_fast(const CField &F, const CWrite &c
     if ((int)threadIdx.x < rows / 4) reinterpret_cast<uint4 *>(wb)[threadIdx.x] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-// Any other slab: codes stored as alignment allows, anchors, and the exact
+// Rows that are not 16-byte aligned: a warp stores one row per step, one code per lane
+// (consecutive addresses, whatever their alignment; 4 lanes x 8 codes per row had made
+// every 2-byte store touch 32 sectors); the row's outlier word is a ballot.
+// Out of line: inlined, it made the aligned fields' loop 1% slower.
+__device__ __noinline__ void write_slab_rows(const CField &F, const CWrite cw, int z0, int y0, int x0, int col,
+                                             int own_lo, int planes)
+{
+    const uint16_t *stage = reinterpret_cast<const uint16_t *>(g_smem + C_STAGE);
+    const float *box = reinterpret_cast<const float *>(g_smem + C_BOX);
+    const Field &f = F.f;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const size_t plane = (size_t)f.n[1] * f.n[2];
+    const int nx = f.n[2] - x0, ny = min(OY, f.n[1] - y0);
+    const bool in = lane < nx;
+    for (int y = warp; y < ny; y += NWARP) {
+        const size_t grow = (size_t)(z0 + own_lo) * f.n[1] + y0 + y;
+        uint16_t *gp = F.a.codes + grow * f.n[2] + x0 + lane;
+        uint32_t *wb = F.a.bitmap + ((size_t)col * f.n[0] + z0 + own_lo) * OY + y;
+        const uint16_t *sp = stage + own_lo * STAGE_PLANE + y * CP + lane;
+        const bool anchor = in && ((y | lane) & 7) == 0;
+#pragma unroll 2
+        for (int i = 0; i < planes; ++i, gp += plane, wb += OY, sp += STAGE_PLANE) {
+            uint32_t code = *sp;
+            const int pz = own_lo + i;
+            if (anchor && (pz & 7) == 0) {  // anchor (Sec. IV-A): lossless, code R
+                code = (uint32_t)cw.R;
+                F.a.anchors[((size_t)((z0 + pz) / 8) * cw.Ay + (y0 + y) / 8) * cw.Ax +
+                            (x0 + lane) / 8] = box[pz * PLANE + y * EX + lane];
+            }
+            if (in) *gp = (uint16_t)code;
+            const uint32_t word = __ballot_sync(0xffffffffu, in && code == 0u);
+            if (lane == 0) {
+                *wb = word;
+                if (word) {
+                    const size_t gw = (grow + (size_t)i * f.n[1]) * cw.WX + x0 / 32;
+                    atomicAdd(&F.a.blockcnt[gw / BITMAP_BLOCK_WORDS], (uint32_t)__popc(word));
+                }
+            }
+        }
+    }
+}
+
+// Any other slab with 16-byte aligned code rows: codes, anchors, and the exact
 // outlier-bitmap words with their block counts.  A warp takes 8 consecutive
 // rows of one plane, 4 lanes x 8 codes per row.
 __device__ __forceinline__ void write_slab_general(const CField &F, const CWrite &cw, const Slab &sl, int rows,
@@ -943,14 +1000,8 @@ __device__ __forceinline__ void write_slab_general(const CField &F, const CWrite
             w[0] = (w[0] & 0xffff0000u) | (uint32_t)cw.R;
             F.a.anchors[((size_t)(gz / 8) * cw.Ay + gy / 8) * cw.Ax + gx / 8] = box[pz * PLANE + y * EX + 8 * sub];
         }
-        if (nvalid == 8 && cw.code_store == 8) {
+        if (nvalid == 8) {
             *reinterpret_cast<uint4 *>(F.a.codes + gi) = make_uint4(w[0], w[1], w[2], w[3]);
-        } else if (nvalid == 8 && cw.code_store == 4) {
-            reinterpret_cast<uint2 *>(F.a.codes + gi)[0] = make_uint2(w[0], w[1]);
-            reinterpret_cast<uint2 *>(F.a.codes + gi)[1] = make_uint2(w[2], w[3]);
-        } else if (nvalid == 8 && cw.code_store == 2) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) reinterpret_cast<uint32_t *>(F.a.codes + gi)[j] = w[j];
         } else {
 #pragma unroll
             for (int j = 0; j < 8; ++j)
@@ -1010,6 +1061,7 @@ __global__ void __launch_bounds__(NT, kCompressCtas) k_compress(const __grid_con
     __syncthreads();
 
     uint32_t phase = 0;
+    uint32_t out_seen = 0;  // outliers in the shared histogram before the current slab
 
     Cursor cu;
     if (!cursor_start<MULTI>(cu, bv, blockIdx.x)) return;
@@ -1056,7 +1108,6 @@ __global__ void __launch_bounds__(NT, kCompressCtas) k_compress(const __grid_con
         }
         __syncthreads();  // box and levels ready; the landing buffer now stages codes
         if (abort_flag) break;
-        const uint32_t out0 = hist_s[0];  // outliers counted before this slab
 
         run_slab<true>(box, sk, sl, f, lv);  // ends with a barrier
 
@@ -1065,11 +1116,15 @@ __global__ void __launch_bounds__(NT, kCompressCtas) k_compress(const __grid_con
         const int nzp = min(EZ, f.n[0] - sl.g0[0]);
         const int hi = min(sl.own_hi, nzp - 1);
         const int rows = (hi - sl.own_lo + 1) * OY;
-        const bool outliers = hist_s[0] != out0;
+        const uint32_t out_now = hist_s[0];  // no code is counted before the next slab's first barrier
+        const bool outliers = out_now != out_seen;
+        out_seen = out_now;
         if (!outliers && cw.code_store == 8 && sl.g0[1] + OY <= f.n[1] && sl.g0[2] + OX <= f.n[2])
             write_slab_fast(F, cw, sl, rows, stage, box);
-        else
+        else if (cw.code_store == 8)
             write_slab_general(F, cw, sl, rows, stage, box);
+        else
+            write_slab_rows(F, cw, sl.g0[0], sl.g0[1], sl.g0[2], sl.col, sl.own_lo, hi - sl.own_lo + 1);
         // ---- next slab's input into the landing buffer (staged codes written out),
         // and plane 8 carried into plane 0 when the next slab continues this run
         __syncthreads();
@@ -1081,7 +1136,10 @@ __global__ void __launch_bounds__(NT, kCompressCtas) k_compress(const __grid_con
                 for (int i = threadIdx.x; i < PLANE; i += NT) box[i] = box[8 * PLANE + i];
         }
         __syncthreads();  // box free for the next slab
-        if (!has_next || (MULTI && nx.fi != cu.fi)) flush_hist(F, hist_s);  // field done
+        if (!has_next || (MULTI && nx.fi != cu.fi)) {  // field done
+            flush_hist(F, hist_s);
+            out_seen = 0;
+        }
         if (!has_next) break;
         cu = nx;
         sl = sn;
@@ -1297,6 +1355,19 @@ __global__ void __launch_bounds__(NT, kDecompressCtas) k_decompress(const __grid
                 reinterpret_cast<float4 *>(gp)[0] = make_float4(sp[0], sp[1], sp[2], sp[3]);
                 reinterpret_cast<float4 *>(gp)[1] = make_float4(sp[4], sp[5], sp[6], sp[7]);
             }
+        } else if (!F.a.vec_xrec) {
+            // rows that are not 16-byte aligned: a warp stores one row per step, one value per
+            // lane (consecutive addresses)
+            const size_t plane = (size_t)f.n[1] * f.n[2];
+            const int ny = min(OY, f.n[1] - sl.g0[1]);
+            if (lane < f.n[2] - sl.g0[2])
+                for (int y = warp; y < ny; y += NWARP) {
+                    const float *sp = box + sl.own_lo * PLANE + y * EX + lane;
+                    float *gp = F.a.xrec + ((size_t)(sl.g0[0] + sl.own_lo) * f.n[1] + sl.g0[1] + y) * f.n[2] +
+                                sl.g0[2] + lane;
+#pragma unroll 2
+                    for (int i = 0; i < rows / OY; ++i, sp += PLANE, gp += plane) *gp = *sp;
+                }
         } else {
             // 8 lanes x 4 values per row, 4 rows per warp
             const int sub = lane & 7;
@@ -1307,11 +1378,8 @@ __global__ void __launch_bounds__(NT, kDecompressCtas) k_decompress(const __grid
                 if (gy >= f.n[1] || gx >= f.n[2]) continue;
                 const float *s4 = box + pz * PLANE + y * EX + 4 * sub;
                 float *dst = F.a.xrec + ((size_t)gz * f.n[1] + gy) * f.n[2] + gx;
-                if (F.a.vec_xrec && gx + 3 < f.n[2]) {
-                    *reinterpret_cast<float4 *>(dst) = make_float4(s4[0], s4[1], s4[2], s4[3]);
-                } else {
-                    for (int j = 0; j < 4 && gx + j < f.n[2]; ++j) dst[j] = s4[j];
-                }
+                // vec_xrec: rows are whole groups of 4 values
+                *reinterpret_cast<float4 *>(dst) = make_float4(s4[0], s4[1], s4[2], s4[3]);
             }
         }
         __syncthreads();  // every thread is done reading the box
