@@ -209,9 +209,9 @@ int compress_nd(const interp_compress_item &it, interp_stream_t stream)
         timing_mark(0, 1, s);
     }
     if (e == cudaSuccess) {
-        // row-major bitmap (nd.cu); the 1-D / 2-D kernels count every bin themselves
+        // row-major bitmap; the 2-D kernel counts every bin itself, the 1-D one leaves bin R
         const gi::CompactItem ci{bitmap, blockcnt, L.words, d, it.d_x, it.d_out_idx, it.d_out_val,
-                                 it.out_capacity, it.d_hdr, true, nullptr, c.radius};
+                                 it.out_capacity, it.d_hdr, true, c.ndim == 2 ? nullptr : it.d_hist, c.radius};
         e = gi::launch_outlier_compaction(&ci, 1, s);
     }
     return cuda_status(e);
@@ -269,15 +269,15 @@ int interp_compress_batched_scheduled(const interp_compress_item *items, int n, 
         timing_mark(0, 1, s);
     }
     if (e == cudaSuccess) {
-        // ordered compaction of every field in two launches; the 3-D tile kernel leaves bin R
-        // to the scan, the 1-D / 2-D kernels count every bin and write row-major bitmaps
+        // ordered compaction of every field in two launches; the 3-D and 1-D kernels leave
+        // bin R to the scan, the 2-D one counts it; 1-D / 2-D bitmaps are row-major
         gi::CompactItem ci[gi::kMaxBatch];
         for (int i = 0; i < n; ++i) {
             const interp_compress_item &it = items[i];
             const bool nd = is_nd(it.cfg.ndim);
             ci[i] = gi::CompactItem{args[i].bitmap, args[i].blockcnt, L[i].words, args[i].dims, it.d_x,
                                     it.d_out_idx, it.d_out_val, it.out_capacity, it.d_hdr, nd,
-                                    nd ? nullptr : it.d_hist, it.cfg.radius};
+                                    it.cfg.ndim == 2 ? nullptr : it.d_hist, it.cfg.radius};
         }
         e = gi::launch_outlier_compaction(ci, n, s);
     }

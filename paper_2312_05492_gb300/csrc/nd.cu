@@ -1039,28 +1039,24 @@ int nd_tiles_host(int ndim, Dims d)
 
 cudaError_t launch_nd_compress(int ndim, const CompressArgs &a, cudaStream_t s)
 {
-    if (ndim != 1 && ndim != 2) return cudaErrorInvalidValue;
+    if (ndim == 1) return launch_row_compress(a, s);
+    if (ndim != 2) return cudaErrorInvalidValue;
     const int tiles = nd_tiles_host(ndim, a.dims);
     if (tiles == 0) return cudaSuccess;
     const size_t hist_smem = (a.hist && 2 * a.radius <= ND_HIST_SMEM_BINS) ? sizeof(uint32_t) * 2 * a.radius : 0;
-    const int grid = min(tiles, sm_count() * (ndim == 2 ? nd_ctas_per_sm<2>() : nd_ctas_per_sm<1>()));
-    if (ndim == 2)
-        k_nd_compress<2><<<grid, ND_THREADS, hist_smem, s>>>(a);
-    else
-        k_nd_compress<1><<<grid, ND_THREADS, hist_smem, s>>>(a);
+    const int grid = min(tiles, sm_count() * nd_ctas_per_sm<2>());
+    k_nd_compress<2><<<grid, ND_THREADS, hist_smem, s>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_nd_decompress(int ndim, const DecompressArgs &a, cudaStream_t s)
 {
-    if (ndim != 1 && ndim != 2) return cudaErrorInvalidValue;
+    if (ndim == 1) return launch_row_decompress(a, s);
+    if (ndim != 2) return cudaErrorInvalidValue;
     const int tiles = nd_tiles_host(ndim, a.dims);
     if (tiles == 0) return cudaSuccess;
-    const int grid = min(tiles, sm_count() * (ndim == 2 ? nd_ctas_per_sm<2>() : nd_ctas_per_sm<1>()));
-    if (ndim == 2)
-        k_nd_decompress<2><<<grid, ND_THREADS, 0, s>>>(a);
-    else
-        k_nd_decompress<1><<<grid, ND_THREADS, 0, s>>>(a);
+    const int grid = min(tiles, sm_count() * nd_ctas_per_sm<2>());
+    k_nd_decompress<2><<<grid, ND_THREADS, 0, s>>>(a);
     return cudaGetLastError();
 }
 
