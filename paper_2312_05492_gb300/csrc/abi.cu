@@ -160,6 +160,15 @@ size_t interp_workspace_bytes(const int64_t dims[3], const interp_config *cfg)
 // The 1-D / 2-D chunk geometries (interp_config.ndim 1 or 2); 0 and 3 are 3-D.
 bool is_nd(int32_t ndim) { return ndim == 1 || ndim == 2; }
 
+cudaError_t launch_nd_compress(int32_t ndim, const gi::CompressArgs &a, cudaStream_t s)
+{
+    return ndim == 1 ? gi::launch_row_compress(a, s) : gi::launch_plane_compress(a, s);
+}
+cudaError_t launch_nd_decompress(int32_t ndim, const gi::DecompressArgs &a, cudaStream_t s)
+{
+    return ndim == 1 ? gi::launch_row_decompress(a, s) : gi::launch_plane_decompress(a, s);
+}
+
 gi::PrologueItem prologue_item(const interp_compress_item &it, const WsLayout &L)
 {
     unsigned char *ws = static_cast<unsigned char *>(it.d_ws);
@@ -180,7 +189,7 @@ gi::PrologueItem prologue_item(const interp_compress_item &it, const WsLayout &L
 }
 
 // One field in the 1-D or 2-D geometry: the same setup and compaction as the 3-D
-// path around the per-tile kernel of nd.cu.
+// path around the kernels of nd1.cu / nd2.cu.
 int compress_nd(const interp_compress_item &it, interp_stream_t stream)
 {
     const interp_config &c = it.cfg;
@@ -205,13 +214,13 @@ int compress_nd(const interp_compress_item &it, interp_stream_t stream)
                                 it.d_hdr, false, false, 1};
     if (e == cudaSuccess) {
         timing_mark(0, 0, s);
-        e = gi::launch_nd_compress(c.ndim, args, s);
+        e = launch_nd_compress(c.ndim, args, s);
         timing_mark(0, 1, s);
     }
     if (e == cudaSuccess) {
-        // row-major bitmap; the 2-D kernel counts every bin itself, the 1-D one leaves bin R
+        // row-major bitmap; the tile kernels leave bin R to the scan
         const gi::CompactItem ci{bitmap, blockcnt, L.words, d, it.d_x, it.d_out_idx, it.d_out_val,
-                                 it.out_capacity, it.d_hdr, true, c.ndim == 2 ? nullptr : it.d_hist, c.radius};
+                                 it.out_capacity, it.d_hdr, true, it.d_hist, c.radius};
         e = gi::launch_outlier_compaction(&ci, 1, s);
     }
     return cuda_status(e);
@@ -265,19 +274,19 @@ int interp_compress_batched_scheduled(const interp_compress_item *items, int n, 
         const gi::TileSchedule ts{sched ? sched->run : 0, sched ? sched->ctas_per_sm : 0};
         if (n3 > 0) e = gi::launch_compress_tiles(args3, n3, s, &ts);  // one persistent launch for every 3-D field
         for (int i = 0; i < n && e == cudaSuccess; ++i)                // one launch per 1-D / 2-D field
-            if (is_nd(items[i].cfg.ndim)) e = gi::launch_nd_compress(items[i].cfg.ndim, args[i], s);
+            if (is_nd(items[i].cfg.ndim)) e = launch_nd_compress(items[i].cfg.ndim, args[i], s);
         timing_mark(0, 1, s);
     }
     if (e == cudaSuccess) {
-        // ordered compaction of every field in two launches; the 3-D and 1-D kernels leave
-        // bin R to the scan, the 2-D one counts it; 1-D / 2-D bitmaps are row-major
+        // ordered compaction of every field in two launches; the tile kernels leave bin R of
+        // the histogram to the scan; 1-D / 2-D bitmaps are row-major
         gi::CompactItem ci[gi::kMaxBatch];
         for (int i = 0; i < n; ++i) {
             const interp_compress_item &it = items[i];
             const bool nd = is_nd(it.cfg.ndim);
             ci[i] = gi::CompactItem{args[i].bitmap, args[i].blockcnt, L[i].words, args[i].dims, it.d_x,
                                     it.d_out_idx, it.d_out_val, it.out_capacity, it.d_hdr, nd,
-                                    it.cfg.ndim == 2 ? nullptr : it.d_hist, it.cfg.radius};
+                                    it.d_hist, it.cfg.radius};
         }
         e = gi::launch_outlier_compaction(ci, n, s);
     }
@@ -348,7 +357,7 @@ int interp_decompress_batched_scheduled(const interp_decompress_item *items, int
         const gi::TileSchedule ts{sched ? sched->run : 0, sched ? sched->ctas_per_sm : 0};
         if (n3 > 0) e = gi::launch_decompress_tiles(args3, n3, s, &ts);
         for (int i = 0; i < n && e == cudaSuccess; ++i)
-            if (is_nd(items[i].ndim)) e = gi::launch_nd_decompress(items[i].ndim, args[i], s);
+            if (is_nd(items[i].ndim)) e = launch_nd_decompress(items[i].ndim, args[i], s);
         timing_mark(1, 1, s);
     }
     return cuda_status(e);
@@ -393,7 +402,7 @@ int interp_decompress_nd(int32_t ndim, const int64_t dims[3], const interp_heade
     const gi::DecompressArgs args{d, d_anchors, d_codes, d_xrec, d_hdr, false};
     if (e == cudaSuccess) {
         timing_mark(1, 0, s);
-        e = gi::launch_nd_decompress(ndim, args, s);
+        e = launch_nd_decompress(ndim, args, s);
         timing_mark(1, 1, s);
     }
     return cuda_status(e);

@@ -24,6 +24,9 @@ namespace gi {
 #ifndef GI_TILE_THREADS
 #define GI_TILE_THREADS 192
 #endif
+#ifndef GI_PLANE_CTAS
+#define GI_PLANE_CTAS 2
+#endif
 #ifndef GI_ROW_CTAS
 #define GI_ROW_CTAS 3
 #endif
@@ -241,10 +244,9 @@ cudaError_t launch_compress_tiles(const CompressArgs *args, int n, cudaStream_t 
 cudaError_t launch_decompress_tiles(const DecompressArgs *args, int n, cudaStream_t s,
                                     const TileSchedule *sched = nullptr);
 size_t bitmap_words_tiled(Dims d);
-// 1-D (512-point chunks) and 2-D (16^2 chunks) variants (nd.cu); ndim 1 or 2
-cudaError_t launch_nd_compress(int ndim, const CompressArgs &a, cudaStream_t s);
-cudaError_t launch_nd_decompress(int ndim, const DecompressArgs &a, cudaStream_t s);
-// the 1-D kernels (nd1.cu)
+// the 2-D kernels (nd2.cu) and the 1-D kernels (nd1.cu)
+cudaError_t launch_plane_compress(const CompressArgs &a, cudaStream_t s);
+cudaError_t launch_plane_decompress(const DecompressArgs &a, cudaStream_t s);
 cudaError_t launch_row_compress(const CompressArgs &a, cudaStream_t s);
 cudaError_t launch_row_decompress(const DecompressArgs &a, cudaStream_t s);
 // ordered outlier compaction of n fields (one scan launch, one write launch)
