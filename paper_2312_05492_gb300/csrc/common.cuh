@@ -24,12 +24,6 @@ namespace gi {
 #ifndef GI_TILE_THREADS
 #define GI_TILE_THREADS 192
 #endif
-#ifndef GI_PLANE_CTAS
-#define GI_PLANE_CTAS 2
-#endif
-#ifndef GI_ROW_CTAS
-#define GI_ROW_CTAS 3
-#endif
 #ifndef GI_TILE_ROWS
 #define GI_TILE_ROWS 16
 #endif
@@ -113,6 +107,16 @@ __device__ __forceinline__ float sp_cubic_nat(float m3, float m1, float p1, floa
 {
     return div40_rn(23.0f * (m1 + p1) - 3.0f * (m3 + p3));
 }
+// the same with the rare path out of line: inlined at every stencil of a kernel whose
+// passes are unrolled, it pushes the code out of the instruction cache (1-D kernels 6 - 10%
+// slower, 2-D ones 4 - 6%); the 3-D kernels, whose passes are short loops, are 2 - 8% slower
+// with the call (registers kept for it)
+static __device__ __noinline__ float div40_tiny_call(float n) { return div40_tiny(n); }
+__device__ __forceinline__ float sp_cubic_nat_call(float m3, float m1, float p1, float p3)
+{
+    const float n = 23.0f * (m1 + p1) - 3.0f * (m3 + p3), a = fabsf(n);
+    return (a >= 8.07793567e-28f && a <= 3.402823466e38f) ? div40_markstein(n) : div40_tiny_call(n);
+}
 // the cubic kind chosen at run time (0 = not-a-knot, 1 = natural)
 struct Cubic {
     int natural;
@@ -147,11 +151,17 @@ __device__ __forceinline__ uint32_t quantize(float x, float p, const LevelQ &L, 
     const float v = d * L.inv2e;
     const float y = v + kMagic;
     const float q = y - kMagic;
-    bool ok = fabsf(q) < Rf;
     const float r = p + q * L.twoe;
-    ok = ok && (fabsf(x - r) <= L.e);
-    xr = ok ? r : x;
-    return ok ? __float_as_uint(y) - cbias : 0u;
+    const float err = x - r;
+    const uint32_t c = __float_as_uint(y) - cbias;
+    uint32_t code;
+    // both tests and both selections without a branch (written as C++ they became
+    // divergent branches around single moves)
+    asm("{\n .reg .pred ok;\n setp.lt.f32 ok, %2, %3;\n setp.le.and.f32 ok, %4, %5, ok;\n"
+        " selp.f32 %0, %6, %7, ok;\n selp.u32 %1, %8, 0, ok;\n}\n"
+        : "=f"(xr), "=r"(code)
+        : "f"(fabsf(q)), "f"(Rf), "f"(fabsf(err)), "f"(L.e), "f"(r), "f"(x), "r"(c));
+    return code;
 }
 
 // (code - R) as a float, exactly (|code - R| < 2^22): the float whose bits are

@@ -21,9 +21,13 @@
 namespace gi {
 namespace {
 
-constexpr int RW = 8;                 // warps per CTA, each on its own segments
-constexpr int R_THREADS = 32 * RW;
-constexpr int R_CTAS = GI_ROW_CTAS;   // CTAs per SM
+// warps per CTA (each on its own segments) and CTAs per SM: 20 warps of 96 registers for
+// compression (229 us against 252 with 24 warps of 80 on 64 x 2^21 points), 24 of 80 for
+// decompression (171 us against 181)
+struct Shape {
+    int warps, ctas;
+};
+constexpr Shape RC{4, 5}, RD{8, 3};
 constexpr int RUN = 32;               // points per lane
 constexpr int SEG = 32 * RUN;         // points per warp
 constexpr int CHUNK = 512, CLANES = CHUNK / RUN;  // lanes per chunk
@@ -32,14 +36,18 @@ constexpr int VP = 36;                // floats per landed run (32 and 4 of padd
 constexpr int KP = 40;                // codes per landed run
 constexpr int R_HIST_BINS = 8192;     // bins kept in shared memory
 constexpr size_t R_V = sizeof(float) * 32 * VP, R_K = sizeof(uint16_t) * 32 * KP;
-constexpr size_t R_WARP = R_V + R_K;  // per warp: value runs, code runs
-constexpr size_t R_LQ = R_WARP * RW;  // level constants
-constexpr size_t R_SPARE = R_LQ + 16 * LEVELS;  // one word per lane for updates that count nothing
-constexpr size_t R_HIST = R_SPARE + 4 * 32;
-static_assert(R_LQ % 16 == 0 && R_HIST % 16 == 0, "shared layout alignment");
+constexpr size_t R_LQ = 0;                       // level constants
+constexpr size_t R_SPARE = R_LQ + 16 * LEVELS;   // one word per lane for updates that count nothing
+constexpr size_t R_WARPS = R_SPARE + 4 * 32;     // then per warp: value runs, code runs
+constexpr size_t R_WARP = R_V + R_K;
+constexpr size_t R_HIST = R_WARPS + R_WARP * RC.warps;  // compression: the bins
+static_assert(R_WARPS % 16 == 0 && R_HIST % 16 == 0, "shared layout alignment");
 
 extern __shared__ __align__(128) unsigned char r_smem[];
 
+// What a kernel does with the points: apply the stored codes; quantize and count in shared
+// or in global bins.
+enum { DECODE = 0, ENCODE = 1, ENCODE_GBINS = 2 };
 enum { K_LINEAR = 0, K_NAK = 1, K_NATURAL = 2 };
 
 // Level constants, one thread per level, with the header's own arithmetic (alpha^l by
@@ -70,18 +78,20 @@ struct Ctx {
     uint32_t cbias, R;
     float Rf;
     uint32_t hist, spare;  // shared addresses of the bins and of this lane's spare word
-    bool global_bins;      // more than R_HIST_BINS bins: counted in global memory
-    uint32_t *hist_g;      // those bins, may be null
+    uint32_t *hist_g;      // more than R_HIST_BINS bins: those in global memory, may be null
     int lane, cl;          // lane, lane within its chunk
     float closing;         // the point after the segment (an anchor), in every lane
     int last;              // last in-field offset from the segment's start (SEG when it is whole)
 };
 
 // Count a code other than R (whose bin is filled in afterwards as N minus the others).
+// ENCODE_GBINS: more bins than shared memory keeps, counted in global memory (a branch per
+// point when it was decided at run time).
+template <int MODE>
 __device__ __forceinline__ void count(const Ctx &c, uint32_t code, bool counts)
 {
     const bool yes = counts && code != c.R;
-    if (c.global_bins) {
+    if constexpr (MODE == ENCODE_GBINS) {
         if (yes && c.hist_g) atomicAdd(c.hist_g + code, 1u);
     } else {
         asm volatile("red.shared.add.u32 [%0], 1;\n" ::"r"(yes ? c.hist + 4u * code : c.spare));
@@ -91,7 +101,7 @@ __device__ __forceinline__ void count(const Ctx &c, uint32_t code, bool counts)
 template <int KIND>
 __device__ __forceinline__ float cubic_of(float m3, float m1, float p1, float p3)
 {
-    return KIND == K_NATURAL ? sp_cubic_nat(m3, m1, p1, p3) : sp_cubic_nak(m3, m1, p1, p3);
+    return KIND == K_NATURAL ? sp_cubic_nat_call(m3, m1, p1, p3) : sp_cubic_nak(m3, m1, p1, p3);
 }
 
 // Neighbour-count rule (Sec. IV-B.1).
@@ -107,12 +117,12 @@ __device__ __forceinline__ float predict(float m3, float m1, float p1, float p3,
 }
 
 // One point: value v (compression: the original on entry, x' on return) and its code.
-template <bool COMPRESS, bool OUTL>
+template <int MODE, bool OUTL>
 __device__ __forceinline__ uint32_t point(const Ctx &c, const LevelQ &q, float &v, float p, uint32_t code, bool counts)
 {
-    if (COMPRESS) {
+    if (MODE != DECODE) {
         code = quantize(v, p, q, c.cbias, c.Rf, v);
-        count(c, code, counts);
+        count<MODE>(c, code, counts);
     } else {
         const float xq = p + code_to_q(code, c.cbias) * q.twoe;
         v = OUTL && code == 0u ? v : xq;  // an outlier's stored value is there already
@@ -121,7 +131,7 @@ __device__ __forceinline__ uint32_t point(const Ctx &c, const LevelQ &q, float &
 }
 
 // Stride 32 T: only the lanes' first points, through shuffles.
-template <bool COMPRESS, bool OUTL, bool FULL, int T, int KIND>
+template <int MODE, bool OUTL, bool FULL, int T, int KIND>
 __device__ __forceinline__ void coarse_level(Lane &L, const Ctx &c)
 {
     constexpr int l = T == 8 ? 8 : (T == 4 ? 7 : (T == 2 ? 6 : 5));
@@ -137,16 +147,16 @@ __device__ __forceinline__ void coarse_level(Lane &L, const Ctx &c)
     const float p = predict<KIND>(m3, m1, p1, p3, hm3, hp1, hp3);
     const bool mine = (c.cl & (2 * T - 1)) == T;
     float v = a;
-    const uint32_t code = point<COMPRESS, OUTL>(c, q, v, p, L.cw[0] & 0xffffu,
+    const uint32_t code = point<MODE, OUTL>(c, q, v, p, L.cw[0] & 0xffffu,
                                                 mine && (FULL || RUN * c.lane <= c.last));
     if (mine) {
         L.v[0] = v;
-        if (COMPRESS) L.cw[0] = code;
+        if (MODE != DECODE) L.cw[0] = code;
     }
 }
 
 // Stride S <= 16: P = 16 / S points of the lane.
-template <bool COMPRESS, bool OUTL, bool FULL, int S, int KIND>
+template <int MODE, bool OUTL, bool FULL, int S, int KIND>
 __device__ __forceinline__ void lane_level(Lane &L, const Ctx &c, float next0)
 {
     constexpr int l = S == 16 ? 4 : (S == 8 ? 3 : (S == 4 ? 2 : (S == 2 ? 1 : 0)));
@@ -183,19 +193,19 @@ __device__ __forceinline__ void lane_level(Lane &L, const Ctx &c, float next0)
         }
         const uint32_t w = L.cw[o / 2];
         const uint32_t code =
-            point<COMPRESS, OUTL>(c, q, L.v[o], p, S == 1 ? w >> 16 : w & 0xffffu, in);
-        if (COMPRESS) L.cw[o / 2] = S == 1 ? w + (code << 16) : code;
+            point<MODE, OUTL>(c, q, L.v[o], p, S == 1 ? w >> 16 : w & 0xffffu, in);
+        if (MODE != DECODE) L.cw[o / 2] = S == 1 ? w + (code << 16) : code;
     }
 }
 
-template <bool COMPRESS, bool OUTL, bool FULL, int S, int KIND>
+template <int MODE, bool OUTL, bool FULL, int S, int KIND>
 __device__ __forceinline__ void any_level(Lane &L, const Ctx &c, float next0)
 {
-    if constexpr (S >= RUN) coarse_level<COMPRESS, OUTL, FULL, S / RUN, KIND>(L, c);
-    else lane_level<COMPRESS, OUTL, FULL, S, KIND>(L, c, next0);
+    if constexpr (S >= RUN) coarse_level<MODE, OUTL, FULL, S / RUN, KIND>(L, c);
+    else lane_level<MODE, OUTL, FULL, S, KIND>(L, c, next0);
 }
 
-template <bool COMPRESS, bool OUTL, bool FULL, int S>
+template <int MODE, bool OUTL, bool FULL, int S>
 __device__ __forceinline__ void levels_from(Lane &L, const Ctx &c, int kind0, int kind1, int kind2, float next0)
 {
     if (S == 16) {  // the lanes' first points are final: the next lane's serves all finer strides
@@ -203,10 +213,10 @@ __device__ __forceinline__ void levels_from(Lane &L, const Ctx &c, int kind0, in
         if (c.lane == 31) next0 = c.closing;
     }
     const int kind = S == 1 ? kind0 : (S == 2 ? kind1 : kind2);  // coarser levels than 4 follow stride 4
-    if (kind == K_LINEAR) any_level<COMPRESS, OUTL, FULL, S, K_LINEAR>(L, c, next0);
-    else if (kind == K_NAK) any_level<COMPRESS, OUTL, FULL, S, K_NAK>(L, c, next0);
-    else any_level<COMPRESS, OUTL, FULL, S, K_NATURAL>(L, c, next0);
-    if constexpr (S > 1) levels_from<COMPRESS, OUTL, FULL, S / 2>(L, c, kind0, kind1, kind2, next0);
+    if (kind == K_LINEAR) any_level<MODE, OUTL, FULL, S, K_LINEAR>(L, c, next0);
+    else if (kind == K_NAK) any_level<MODE, OUTL, FULL, S, K_NAK>(L, c, next0);
+    else any_level<MODE, OUTL, FULL, S, K_NATURAL>(L, c, next0);
+    if constexpr (S > 1) levels_from<MODE, OUTL, FULL, S / 2>(L, c, kind0, kind1, kind2, next0);
 }
 
 // Kinds of the three level classes (strides 1, 2, 4 and more).
@@ -254,19 +264,20 @@ __device__ __forceinline__ void land_values(float *land, const float *x, const S
     cp_async_commit();
 }
 
-__global__ void __launch_bounds__(R_THREADS, R_CTAS) k_row_compress(const CompressArgs a, uint32_t per_row,
+template <int MODE>
+__global__ void __launch_bounds__(32 * RC.warps, RC.ctas) k_row_compress(const CompressArgs a, uint32_t per_row,
                                                                    uint32_t segs)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nx = a.dims.nx, bins = 2 * a.radius;
-    const bool smem_hist = bins <= R_HIST_BINS;
+    constexpr bool smem_hist = MODE == ENCODE;
     uint32_t *hs = reinterpret_cast<uint32_t *>(r_smem + R_HIST);
     row_levels(a.hdr);
     if (smem_hist)
-        for (int i = threadIdx.x; i < bins; i += R_THREADS) hs[i] = 0u;
+        for (int i = threadIdx.x; i < bins; i += 32 * RC.warps) hs[i] = 0u;
     __syncthreads();
-    float *land = reinterpret_cast<float *>(r_smem + R_WARP * warp);
-    uint16_t *stage = reinterpret_cast<uint16_t *>(r_smem + R_WARP * warp + R_V);
+    float *land = reinterpret_cast<float *>(r_smem + R_WARPS + R_WARP * warp);
+    uint16_t *stage = reinterpret_cast<uint16_t *>(r_smem + R_WARPS + R_WARP * warp + R_V);
     const bool vec = (nx & 3) == 0 && (reinterpret_cast<uintptr_t>(a.x) & 15u) == 0;
     const bool vec_codes = (nx & 7) == 0 && (reinterpret_cast<uintptr_t>(a.codes) & 15u) == 0;
     const Kinds kd = kinds_of(a.hdr);
@@ -277,14 +288,13 @@ __global__ void __launch_bounds__(R_THREADS, R_CTAS) k_row_compress(const Compre
     c.Rf = (float)a.radius;
     c.hist = smem_u32(hs);
     c.spare = smem_u32(r_smem + R_SPARE) + 4u * lane;
-    c.global_bins = !smem_hist;
     c.hist_g = a.hist;
     c.lane = lane;
     c.cl = lane & (CLANES - 1);
 
     // segments go to CTAs first, then to their warps: few segments spread over the SMs
     uint32_t s = blockIdx.x + gridDim.x * (uint32_t)warp;
-    const uint32_t step = gridDim.x * RW;
+    const uint32_t step = gridDim.x * RC.warps;
     float closing = 0.0f;
     if (s < segs) {
         const Seg g = seg_of(s, per_row, nx);
@@ -314,8 +324,8 @@ __global__ void __launch_bounds__(R_THREADS, R_CTAS) k_row_compress(const Compre
         const bool full = g.x0 + SEG < nx;  // both chunks and the closing point inside the row
         c.last = full ? SEG : nx - 1 - g.x0;
         L.cw[0] = c.R;  // the anchors' code
-        if (full) levels_from<true, false, true, 256>(L, c, kd.k0, kd.k1, kd.k2, 0.0f);
-        else levels_from<true, false, false, 256>(L, c, kd.k0, kd.k1, kd.k2, 0.0f);
+        if (full) levels_from<MODE, false, true, 256>(L, c, kd.k0, kd.k1, kd.k2, 0.0f);
+        else levels_from<MODE, false, false, 256>(L, c, kd.k0, kd.k1, kd.k2, 0.0f);
         const int p0 = g.x0 + RUN * lane;  // the lane's first point in the row
         if (c.cl == 0 && p0 < nx) a.anchors[(size_t)g.row * apr + (uint32_t)p0 / CHUNK] = L.v[0];
         // outlier word of the lane's 32 points (row-major bitmap) and its block count
@@ -356,7 +366,7 @@ __global__ void __launch_bounds__(R_THREADS, R_CTAS) k_row_compress(const Compre
     }
     if (a.hist && smem_hist) {
         __syncthreads();
-        for (int i = threadIdx.x; i < bins; i += R_THREADS)
+        for (int i = threadIdx.x; i < bins; i += 32 * RC.warps)
             if (hs[i]) atomicAdd(&a.hist[i], hs[i]);
     }
 }
@@ -385,15 +395,15 @@ __device__ __forceinline__ void land_codes(uint16_t *land, const uint16_t *codes
     cp_async_commit();
 }
 
-__global__ void __launch_bounds__(R_THREADS, R_CTAS) k_row_decompress(const DecompressArgs a, uint32_t per_row,
+__global__ void __launch_bounds__(32 * RD.warps, RD.ctas) k_row_decompress(const DecompressArgs a, uint32_t per_row,
                                                                      uint32_t segs)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nx = a.dims.nx;
     row_levels(a.hdr);
     __syncthreads();
-    float *stage = reinterpret_cast<float *>(r_smem + R_WARP * warp);
-    uint16_t *land = reinterpret_cast<uint16_t *>(r_smem + R_WARP * warp + R_V);
+    float *stage = reinterpret_cast<float *>(r_smem + R_WARPS + R_WARP * warp);
+    uint16_t *land = reinterpret_cast<uint16_t *>(r_smem + R_WARPS + R_WARP * warp + R_V);
     const bool vec = (nx & 3) == 0 && (reinterpret_cast<uintptr_t>(a.xrec) & 15u) == 0;
     const uintptr_t ca = reinterpret_cast<uintptr_t>(a.codes);
     const int width = (nx & 7) == 0 && (ca & 15u) == 0 ? 8 : ((nx & 1) == 0 && (ca & 3u) == 0 ? 2 : 1);
@@ -404,7 +414,6 @@ __global__ void __launch_bounds__(R_THREADS, R_CTAS) k_row_decompress(const Deco
     c.cbias = kMagicBits - c.R;
     c.Rf = 0.0f;
     c.hist = c.spare = 0u;
-    c.global_bins = false;
     c.hist_g = nullptr;
     c.lane = lane;
     c.cl = lane & (CLANES - 1);
@@ -417,7 +426,7 @@ __global__ void __launch_bounds__(R_THREADS, R_CTAS) k_row_decompress(const Deco
                    ? __ldg(a.anchors + (size_t)g.row * apr + (uint32_t)g.x0 / CHUNK + i) : 0.0f;
     };
     uint32_t s = blockIdx.x + gridDim.x * (uint32_t)warp;
-    const uint32_t step = gridDim.x * RW;
+    const uint32_t step = gridDim.x * RD.warps;
     float anc = 0.0f;
     if (s < segs) {
         const Seg g = seg_of(s, per_row, nx);
@@ -458,11 +467,11 @@ __global__ void __launch_bounds__(R_THREADS, R_CTAS) k_row_decompress(const Deco
 #pragma unroll
             for (int i = 0; i < RUN; ++i)
                 if (i < in && ((i & 1) ? L.cw[i / 2] >> 16 : L.cw[i / 2] & 0xffffu) == 0u) L.v[i] = xr[i];
-            levels_from<false, true, false, 256>(L, c, kd.k0, kd.k1, kd.k2, 0.0f);
+            levels_from<DECODE, true, false, 256>(L, c, kd.k0, kd.k1, kd.k2, 0.0f);
         } else if (full) {
-            levels_from<false, false, true, 256>(L, c, kd.k0, kd.k1, kd.k2, 0.0f);
+            levels_from<DECODE, false, true, 256>(L, c, kd.k0, kd.k1, kd.k2, 0.0f);
         } else {
-            levels_from<false, false, false, 256>(L, c, kd.k0, kd.k1, kd.k2, 0.0f);
+            levels_from<DECODE, false, false, 256>(L, c, kd.k0, kd.k1, kd.k2, 0.0f);
         }
         __syncwarp();  // the stage's previous contents are written out
 #pragma unroll
@@ -490,15 +499,15 @@ __global__ void __launch_bounds__(R_THREADS, R_CTAS) k_row_decompress(const Deco
 uint32_t segments_per_row(Dims d) { return (uint32_t)(((long long)d.nx + SEG - 1) / SEG); }
 
 template <typename K, typename A>
-cudaError_t launch_rows(K kernel, const A &a, size_t smem, cudaStream_t s)
+cudaError_t launch_rows(K kernel, Shape shape, const A &a, size_t smem, cudaStream_t s)
 {
     // segments are fewer than 2^32 (N is), and a grid of one wave takes them in turn
     const uint32_t per_row = segments_per_row(a.dims);
     const unsigned long long segs = (unsigned long long)a.dims.nz * a.dims.ny * per_row;
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const unsigned long long wave = (unsigned long long)sm_count() * R_CTAS;
-    kernel<<<(unsigned)(segs < wave ? segs : wave), R_THREADS, smem, s>>>(a, per_row, (uint32_t)segs);
+    const unsigned long long wave = (unsigned long long)sm_count() * shape.ctas;
+    kernel<<<(unsigned)(segs < wave ? segs : wave), 32 * shape.warps, smem, s>>>(a, per_row, (uint32_t)segs);
     return cudaGetLastError();
 }
 
@@ -506,13 +515,13 @@ cudaError_t launch_rows(K kernel, const A &a, size_t smem, cudaStream_t s)
 
 cudaError_t launch_row_compress(const CompressArgs &a, cudaStream_t s)
 {
-    const size_t hist = 2 * a.radius <= R_HIST_BINS ? sizeof(uint32_t) * 2 * (size_t)a.radius : 0;
-    return launch_rows(k_row_compress, a, R_HIST + hist, s);
+    if (2 * a.radius > R_HIST_BINS) return launch_rows(k_row_compress<ENCODE_GBINS>, RC, a, R_HIST, s);
+    return launch_rows(k_row_compress<ENCODE>, RC, a, R_HIST + sizeof(uint32_t) * 2 * (size_t)a.radius, s);
 }
 
 cudaError_t launch_row_decompress(const DecompressArgs &a, cudaStream_t s)
 {
-    return launch_rows(k_row_decompress, a, R_HIST, s);
+    return launch_rows(k_row_decompress, RD, a, R_WARPS + R_WARP * RD.warps, s);
 }
 
 }  // namespace gi

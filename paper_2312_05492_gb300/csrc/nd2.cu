@@ -28,7 +28,7 @@ namespace {
 
 constexpr int PW = 8;                     // warps per CTA, each on its own strips
 constexpr int P_THREADS = 32 * PW;
-constexpr int P_CTAS = GI_PLANE_CTAS;     // CTAs per SM
+constexpr int P_CTAS = 2;                 // CTAs per SM: 16 warps of 128 registers (20 of 96 spill: 25% slower)
 constexpr int A = 16;                     // chunk edge
 constexpr int SX = 64;                    // columns of a strip
 constexpr int LEVELS = 4;
@@ -46,6 +46,9 @@ static_assert(P_WARP % 16 == 0 && P_HIST % 16 == 0, "shared layout alignment");
 
 extern __shared__ __align__(128) unsigned char p_smem[];
 
+// What a kernel does with the points: apply the stored codes; quantize and count in shared
+// or in global bins.
+enum { DECODE = 0, ENCODE = 1, ENCODE_GBINS = 2 };
 enum { K_LINEAR = 0, K_NAK = 1, K_NATURAL = 2 };
 enum { ROW0 = 0, ROW1 = 1, ROW2 = 2, ROW3 = 3 };
 
@@ -73,8 +76,7 @@ struct Ctx {
     uint32_t cbias, R;
     float Rf;
     uint32_t hist, spare;  // shared addresses of the bins and of this lane's spare word
-    bool global_bins;      // more than P_HIST_BINS bins: counted in global memory
-    uint32_t *hist_g;      // those bins, may be null
+    uint32_t *hist_g;      // more than P_HIST_BINS bins: those in global memory, may be null
     int lane, px, py;
     int lx, ly;            // last in-field column from the lane's first one, and row from the
                            // chunk's first one
@@ -83,10 +85,13 @@ struct Ctx {
 };
 
 // Count a code other than R (whose bin is filled in afterwards as N minus the others).
+// ENCODE_GBINS: more bins than shared memory keeps, counted in global memory (a branch per
+// point when it was decided at run time).
+template <int MODE>
 __device__ __forceinline__ void count(const Ctx &c, uint32_t code, bool counts)
 {
     const bool yes = counts && code != c.R;
-    if (c.global_bins) {
+    if constexpr (MODE == ENCODE_GBINS) {
         if (yes && c.hist_g) atomicAdd(c.hist_g + code, 1u);
     } else {
         asm volatile("red.shared.add.u32 [%0], 1;\n" ::"r"(yes ? c.hist + 4u * code : c.spare));
@@ -96,7 +101,7 @@ __device__ __forceinline__ void count(const Ctx &c, uint32_t code, bool counts)
 template <int KIND>
 __device__ __forceinline__ float cubic_of(float m3, float m1, float p1, float p3)
 {
-    return KIND == K_NATURAL ? sp_cubic_nat(m3, m1, p1, p3) : sp_cubic_nak(m3, m1, p1, p3);
+    return KIND == K_NATURAL ? sp_cubic_nat_call(m3, m1, p1, p3) : sp_cubic_nak(m3, m1, p1, p3);
 }
 
 // Neighbour-count rule (Sec. IV-B.1).  MAYBE3: bit 0 / 1 set if x_{n-3s} / x_{n+3s} may
@@ -115,14 +120,14 @@ __device__ __forceinline__ float predict(float m3, float m1, float p1, float p3,
 
 // The point in column e of row j: quantize and count (compression), or apply its code.
 // active: this lane's point belongs to the pass; in: it lies in the field.
-template <bool COMPRESS, bool OUTL, int J, int E>
+template <int MODE, bool OUTL, int J, int E>
 __device__ __forceinline__ void point(Patch &P, const Ctx &c, float p, bool active, bool in)
 {
     float v = P.v[J][E];
-    if (COMPRESS) {
+    if (MODE != DECODE) {
         const uint32_t code = quantize(v, p, c.q, c.cbias, c.Rf, v);
         if constexpr (E < 8) {
-            count(c, code, active && in && (J != ROW0 || c.count0));
+            count<MODE>(c, code, active && in && (J != ROW0 || c.count0));
             uint32_t &w = P.c[J][E / 2];
             if constexpr (E % 2 == 0) w = active ? code : w;
             else w += code << 16;  // odd columns: every lane's, after the even ones
@@ -139,7 +144,7 @@ __device__ __forceinline__ float from(float v, int lane) { return __shfl_sync(0x
 
 // x pass of stride S on row J.  Lanes to the right: px = 7 reads px = 0, which gives its
 // closing column.
-template <bool COMPRESS, bool OUTL, bool FULL, int S, int KIND, int J>
+template <int MODE, bool OUTL, bool FULL, int S, int KIND, int J>
 __device__ __forceinline__ void x_row(Patch &P, const Ctx &c, bool active)
 {
     float *v = P.v[J];
@@ -152,7 +157,7 @@ __device__ __forceinline__ void x_row(Patch &P, const Ctx &c, bool active)
     if constexpr (S == 8) {
         const float prev0 = from(v[0], rowbase | ((c.px - 1) & 7));
         const float p = predict<K_LINEAR, FULL, 0>(0.0f, prev0, next0, 0.0f, false, c.lx >= 8, false);
-        point<COMPRESS, OUTL, J, 0>(P, c, p, active && odd, iny && (FULL || c.lx >= 0));
+        point<MODE, OUTL, J, 0>(P, c, p, active && odd, iny && (FULL || c.lx >= 0));
     } else if constexpr (S == 4) {
         float m3 = 0.0f, p3 = 0.0f;
         if (KIND != K_LINEAR) {
@@ -160,7 +165,7 @@ __device__ __forceinline__ void x_row(Patch &P, const Ctx &c, bool active)
             p3 = from(give0, rowbase | ((c.px + 2) & 7));
         }
         const float p = predict<KIND, FULL, 3>(m3, v[0], next0, p3, odd, c.lx >= 8, !odd && (FULL || c.lx >= 16));
-        point<COMPRESS, OUTL, J, 4>(P, c, p, active, iny && (FULL || c.lx >= 4));
+        point<MODE, OUTL, J, 4>(P, c, p, active, iny && (FULL || c.lx >= 4));
     } else if constexpr (S == 2) {
         float m3 = 0.0f, p3 = 0.0f;
         if (KIND != K_LINEAR) {
@@ -168,9 +173,9 @@ __device__ __forceinline__ void x_row(Patch &P, const Ctx &c, bool active)
             p3 = from(v[4], rowbase | ((c.px + 1) & 7));
         }
         const float k0 = v[0], k4 = v[4];
-        point<COMPRESS, OUTL, J, 2>(P, c, predict<KIND, FULL, 7>(m3, k0, k4, next0, odd, c.lx >= 4, FULL || c.lx >= 8),
+        point<MODE, OUTL, J, 2>(P, c, predict<KIND, FULL, 7>(m3, k0, k4, next0, odd, c.lx >= 4, FULL || c.lx >= 8),
                                     active, iny && (FULL || c.lx >= 2));
-        point<COMPRESS, OUTL, J, 6>(
+        point<MODE, OUTL, J, 6>(
             P, c, predict<KIND, FULL, 7>(k0, k4, next0, p3, true, c.lx >= 8, !odd && (FULL || c.lx >= 12)), active,
             iny && (FULL || c.lx >= 6));
     } else {
@@ -180,34 +185,34 @@ __device__ __forceinline__ void x_row(Patch &P, const Ctx &c, bool active)
             p3 = from(v[2], rowbase | ((c.px + 1) & 7));
         }
         const float k0 = v[0], k2 = v[2], k4 = v[4], k6 = v[6];
-        point<COMPRESS, OUTL, J, 1>(P, c, predict<KIND, FULL, 7>(m3, k0, k2, k4, odd, c.lx >= 2, FULL || c.lx >= 4),
+        point<MODE, OUTL, J, 1>(P, c, predict<KIND, FULL, 7>(m3, k0, k2, k4, odd, c.lx >= 2, FULL || c.lx >= 4),
                                     active, iny && (FULL || c.lx >= 1));
-        point<COMPRESS, OUTL, J, 3>(P, c, predict<KIND, FULL, FULL ? 4 : 7>(k0, k2, k4, k6, true, c.lx >= 4, FULL || c.lx >= 6),
+        point<MODE, OUTL, J, 3>(P, c, predict<KIND, FULL, FULL ? 4 : 7>(k0, k2, k4, k6, true, c.lx >= 4, FULL || c.lx >= 6),
                                     active, iny && (FULL || c.lx >= 3));
-        point<COMPRESS, OUTL, J, 5>(P, c, predict<KIND, FULL, FULL ? 4 : 7>(k2, k4, k6, next0, true, c.lx >= 6, FULL || c.lx >= 8),
+        point<MODE, OUTL, J, 5>(P, c, predict<KIND, FULL, FULL ? 4 : 7>(k2, k4, k6, next0, true, c.lx >= 6, FULL || c.lx >= 8),
                                     active, iny && (FULL || c.lx >= 5));
-        point<COMPRESS, OUTL, J, 7>(
+        point<MODE, OUTL, J, 7>(
             P, c, predict<KIND, FULL, 7>(k4, k6, next0, p3, true, c.lx >= 8, !odd && (FULL || c.lx >= 10)), active,
             iny && (FULL || c.lx >= 7));
     }
 }
 
 // The x pass of stride S on the rows that are multiples of M.
-template <bool COMPRESS, bool OUTL, bool FULL, int S, int KIND, int M>
+template <int MODE, bool OUTL, bool FULL, int S, int KIND, int M>
 __device__ __forceinline__ void x_pass(Patch &P, const Ctx &c)
 {
     const bool row0 = M == 16 ? c.py == 0 : (M == 8 ? (c.py & 1) == 0 : true);
-    x_row<COMPRESS, OUTL, FULL, S, KIND, ROW0>(P, c, row0);
-    if constexpr (M <= 2) x_row<COMPRESS, OUTL, FULL, S, KIND, ROW2>(P, c, true);
+    x_row<MODE, OUTL, FULL, S, KIND, ROW0>(P, c, row0);
+    if constexpr (M <= 2) x_row<MODE, OUTL, FULL, S, KIND, ROW2>(P, c, true);
     if constexpr (M == 1) {
-        x_row<COMPRESS, OUTL, FULL, S, KIND, ROW1>(P, c, true);
-        x_row<COMPRESS, OUTL, FULL, S, KIND, ROW3>(P, c, true);
+        x_row<MODE, OUTL, FULL, S, KIND, ROW1>(P, c, true);
+        x_row<MODE, OUTL, FULL, S, KIND, ROW3>(P, c, true);
     }
 }
 
 // y pass of stride S in column E.  Lanes below: py = 3 reads py = 0, whose row 0 is the
 // closing row.
-template <bool COMPRESS, bool OUTL, bool FULL, int S, int KIND, int E>
+template <int MODE, bool OUTL, bool FULL, int S, int KIND, int E>
 __device__ __forceinline__ void y_col(Patch &P, const Ctx &c, bool active)
 {
     const bool inx = FULL || E <= c.lx;
@@ -216,7 +221,7 @@ __device__ __forceinline__ void y_col(Patch &P, const Ctx &c, bool active)
     if constexpr (S == 8) {
         const float m1 = from(own0, c.lane - 16), p1 = from(x0, c.lane + 16);
         const float p = predict<K_LINEAR, FULL, 0>(0.0f, m1, p1, 0.0f, false, c.ly >= 16, false);
-        point<COMPRESS, OUTL, ROW0, E>(P, c, p, active && c.py == 2, inx && (FULL || c.ly >= 8));
+        point<MODE, OUTL, ROW0, E>(P, c, p, active && c.py == 2, inx && (FULL || c.ly >= 8));
     } else if constexpr (S == 4) {
         const float m1 = from(own0, c.lane - 8), p1 = from(x0, c.lane + 8);
         float m3 = 0.0f, p3 = 0.0f;
@@ -226,7 +231,7 @@ __device__ __forceinline__ void y_col(Patch &P, const Ctx &c, bool active)
         }
         const float p = predict<KIND, FULL, 3>(m3, m1, p1, p3, c.py == 3, 4 * c.py + 4 <= c.ly,
                                                c.py == 1 && (FULL || c.ly >= 16));
-        point<COMPRESS, OUTL, ROW0, E>(P, c, p, active && (c.py & 1), inx && (FULL || 4 * c.py <= c.ly));
+        point<MODE, OUTL, ROW0, E>(P, c, p, active && (c.py & 1), inx && (FULL || 4 * c.py <= c.ly));
     } else {
         const float below0 = from(x0, c.lane + 8);  // row 4 py + 4
         if constexpr (S == 2) {
@@ -238,7 +243,7 @@ __device__ __forceinline__ void y_col(Patch &P, const Ctx &c, bool active)
             const int y = 4 * c.py + 2;
             const float p = predict<KIND, FULL, 7>(m3, own0, below0, p3, c.py > 0, y + 2 <= c.ly,
                                                    c.py < 3 && (FULL || y + 6 <= c.ly));
-            point<COMPRESS, OUTL, ROW2, E>(P, c, p, active, inx && (FULL || y <= c.ly));
+            point<MODE, OUTL, ROW2, E>(P, c, p, active, inx && (FULL || y <= c.ly));
         } else {
             const float r2 = P.v[ROW2][E];
             float m3 = 0.0f, p3 = 0.0f;
@@ -247,10 +252,10 @@ __device__ __forceinline__ void y_col(Patch &P, const Ctx &c, bool active)
                 p3 = from(r2, c.lane + 8);
             }
             const int y = 4 * c.py;
-            point<COMPRESS, OUTL, ROW1, E>(P, c, predict<KIND, FULL, 7>(m3, own0, r2, below0, c.py > 0, y + 2 <= c.ly,
+            point<MODE, OUTL, ROW1, E>(P, c, predict<KIND, FULL, 7>(m3, own0, r2, below0, c.py > 0, y + 2 <= c.ly,
                                                                      FULL || y + 4 <= c.ly),
                                            active, inx && (FULL || y + 1 <= c.ly));
-            point<COMPRESS, OUTL, ROW3, E>(P, c, predict<KIND, FULL, 7>(own0, r2, below0, p3, true, y + 4 <= c.ly,
+            point<MODE, OUTL, ROW3, E>(P, c, predict<KIND, FULL, 7>(own0, r2, below0, p3, true, y + 4 <= c.ly,
                                                                      c.py < 3 && (FULL || y + 6 <= c.ly)),
                                            active, inx && (FULL || y + 3 <= c.ly));
         }
@@ -258,22 +263,22 @@ __device__ __forceinline__ void y_col(Patch &P, const Ctx &c, bool active)
 }
 
 // The y pass of stride S in the columns that are multiples of M, and the closing column.
-template <bool COMPRESS, bool OUTL, bool FULL, int S, int KIND, int M>
+template <int MODE, bool OUTL, bool FULL, int S, int KIND, int M>
 __device__ __forceinline__ void y_pass(Patch &P, const Ctx &c)
 {
-    y_col<COMPRESS, OUTL, FULL, S, KIND, 0>(P, c, M == 16 ? (c.px & 1) == 0 : true);
-    if constexpr (M <= 4) y_col<COMPRESS, OUTL, FULL, S, KIND, 4>(P, c, true);
+    y_col<MODE, OUTL, FULL, S, KIND, 0>(P, c, M == 16 ? (c.px & 1) == 0 : true);
+    if constexpr (M <= 4) y_col<MODE, OUTL, FULL, S, KIND, 4>(P, c, true);
     if constexpr (M <= 2) {
-        y_col<COMPRESS, OUTL, FULL, S, KIND, 2>(P, c, true);
-        y_col<COMPRESS, OUTL, FULL, S, KIND, 6>(P, c, true);
+        y_col<MODE, OUTL, FULL, S, KIND, 2>(P, c, true);
+        y_col<MODE, OUTL, FULL, S, KIND, 6>(P, c, true);
     }
     if constexpr (M == 1) {
-        y_col<COMPRESS, OUTL, FULL, S, KIND, 1>(P, c, true);
-        y_col<COMPRESS, OUTL, FULL, S, KIND, 3>(P, c, true);
-        y_col<COMPRESS, OUTL, FULL, S, KIND, 5>(P, c, true);
-        y_col<COMPRESS, OUTL, FULL, S, KIND, 7>(P, c, true);
+        y_col<MODE, OUTL, FULL, S, KIND, 1>(P, c, true);
+        y_col<MODE, OUTL, FULL, S, KIND, 3>(P, c, true);
+        y_col<MODE, OUTL, FULL, S, KIND, 5>(P, c, true);
+        y_col<MODE, OUTL, FULL, S, KIND, 7>(P, c, true);
     }
-    y_col<COMPRESS, OUTL, FULL, S, KIND, 8>(P, c, true);
+    y_col<MODE, OUTL, FULL, S, KIND, 8>(P, c, true);
 }
 
 // Kinds of the level classes (strides 1, 2, 4 and 8) along y and x.
@@ -292,25 +297,25 @@ __device__ __forceinline__ Kinds kinds_of(const interp_header *h)
     return k;
 }
 
-template <bool COMPRESS, bool OUTL, bool FULL, int S, bool XFIRST>
+template <int MODE, bool OUTL, bool FULL, int S, bool XFIRST>
 __device__ __forceinline__ void x_any(Patch &P, const Ctx &c, int kind)
 {
     constexpr int M = XFIRST ? 2 * S : S;
     // inside a chunk stride 8 is always linear, and stride 4 has no cubic stencil
-    if (S == 8 || kind == K_LINEAR) x_pass<COMPRESS, OUTL, FULL, S, K_LINEAR, M>(P, c);
-    else if (S == 4 || kind == K_NAK) x_pass<COMPRESS, OUTL, FULL, S, K_NAK, M>(P, c);
-    else x_pass<COMPRESS, OUTL, FULL, S, S <= 2 ? K_NATURAL : K_LINEAR, M>(P, c);
+    if (S == 8 || kind == K_LINEAR) x_pass<MODE, OUTL, FULL, S, K_LINEAR, M>(P, c);
+    else if (S == 4 || kind == K_NAK) x_pass<MODE, OUTL, FULL, S, K_NAK, M>(P, c);
+    else x_pass<MODE, OUTL, FULL, S, S <= 2 ? K_NATURAL : K_LINEAR, M>(P, c);
 }
-template <bool COMPRESS, bool OUTL, bool FULL, int S, bool XFIRST>
+template <int MODE, bool OUTL, bool FULL, int S, bool XFIRST>
 __device__ __forceinline__ void y_any(Patch &P, const Ctx &c, int kind)
 {
     constexpr int M = XFIRST ? S : 2 * S;
-    if (S == 8 || kind == K_LINEAR) y_pass<COMPRESS, OUTL, FULL, S, K_LINEAR, M>(P, c);
-    else if (S == 4 || kind == K_NAK) y_pass<COMPRESS, OUTL, FULL, S, K_NAK, M>(P, c);
-    else y_pass<COMPRESS, OUTL, FULL, S, S <= 2 ? K_NATURAL : K_LINEAR, M>(P, c);
+    if (S == 8 || kind == K_LINEAR) y_pass<MODE, OUTL, FULL, S, K_LINEAR, M>(P, c);
+    else if (S == 4 || kind == K_NAK) y_pass<MODE, OUTL, FULL, S, K_NAK, M>(P, c);
+    else y_pass<MODE, OUTL, FULL, S, S <= 2 ? K_NATURAL : K_LINEAR, M>(P, c);
 }
 
-template <bool COMPRESS, bool OUTL, bool FULL, int S, bool XFIRST>
+template <int MODE, bool OUTL, bool FULL, int S, bool XFIRST>
 __device__ __forceinline__ void levels_from(Patch &P, Ctx &c, const Kinds &k)
 {
     constexpr int l = S == 8 ? 3 : (S == 4 ? 2 : (S == 2 ? 1 : 0));
@@ -318,28 +323,28 @@ __device__ __forceinline__ void levels_from(Patch &P, Ctx &c, const Kinds &k)
     c.q = LevelQ{q.x, q.y, q.z};
     const int kx = k.x[l < 2 ? l : 2], ky = k.y[l < 2 ? l : 2];  // stride 8 follows stride 4
     if (XFIRST) {
-        x_any<COMPRESS, OUTL, FULL, S, true>(P, c, kx);
-        y_any<COMPRESS, OUTL, FULL, S, true>(P, c, ky);
+        x_any<MODE, OUTL, FULL, S, true>(P, c, kx);
+        y_any<MODE, OUTL, FULL, S, true>(P, c, ky);
     } else {
-        y_any<COMPRESS, OUTL, FULL, S, false>(P, c, ky);
-        x_any<COMPRESS, OUTL, FULL, S, false>(P, c, kx);
+        y_any<MODE, OUTL, FULL, S, false>(P, c, ky);
+        x_any<MODE, OUTL, FULL, S, false>(P, c, kx);
     }
-    if constexpr (S > 1) levels_from<COMPRESS, OUTL, FULL, S / 2, XFIRST>(P, c, k);
+    if constexpr (S > 1) levels_from<MODE, OUTL, FULL, S / 2, XFIRST>(P, c, k);
 }
 
 // A run's first row on its own (it has no step before it): the x passes on row 0 of the
 // lanes py = 0, as the closing row of a chunk row above.
-template <bool COMPRESS, int S>
+template <int MODE, int S>
 __device__ __forceinline__ void first_row_from(Patch &P, Ctx &c, const Kinds &k)
 {
     constexpr int l = S == 8 ? 3 : (S == 4 ? 2 : (S == 2 ? 1 : 0));
     const float4 q = reinterpret_cast<const float4 *>(p_smem + P_LQ)[l];
     c.q = LevelQ{q.x, q.y, q.z};
     const int kx = k.x[l < 2 ? l : 2];
-    if (S == 8 || kx == K_LINEAR) x_pass<COMPRESS, true, false, S, K_LINEAR, 16>(P, c);
-    else if (S == 4 || kx == K_NAK) x_pass<COMPRESS, true, false, S, K_NAK, 16>(P, c);
-    else x_pass<COMPRESS, true, false, S, S <= 2 ? K_NATURAL : K_LINEAR, 16>(P, c);
-    if constexpr (S > 1) first_row_from<COMPRESS, S / 2>(P, c, k);
+    if (S == 8 || kx == K_LINEAR) x_pass<MODE, true, false, S, K_LINEAR, 16>(P, c);
+    else if (S == 4 || kx == K_NAK) x_pass<MODE, true, false, S, K_NAK, 16>(P, c);
+    else x_pass<MODE, true, false, S, S <= 2 ? K_NATURAL : K_LINEAR, 16>(P, c);
+    if constexpr (S > 1) first_row_from<MODE, S / 2>(P, c, k);
 }
 
 // ------------------------------------------------------------ work items
@@ -414,12 +419,13 @@ __device__ __forceinline__ void set_rows_codes(Patch &P, uint32_t R)
     for (int j = 0; j < 4; ++j) P.c[j][0] = R;  // column 0 of even px in row 0: an anchor, code R
 }
 
+template <int MODE>
 __global__ void __launch_bounds__(P_THREADS, P_CTAS) k_plane_compress(const CompressArgs a, const Plan plan)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const Dims d = a.dims;
     const int bins = 2 * a.radius;
-    const bool smem_hist = bins <= P_HIST_BINS;
+    constexpr bool smem_hist = MODE == ENCODE;
     uint32_t *hs = reinterpret_cast<uint32_t *>(p_smem + P_HIST);
     plane_levels(a.hdr);
     if (smem_hist)
@@ -440,7 +446,6 @@ __global__ void __launch_bounds__(P_THREADS, P_CTAS) k_plane_compress(const Comp
     c.Rf = (float)a.radius;
     c.hist = smem_u32(hs);
     c.spare = smem_u32(p_smem + P_SPARE) + 4u * lane;
-    c.global_bins = !smem_hist;
     c.hist_g = a.hist;
     c.lane = lane;
     c.px = lane & 7;
@@ -464,7 +469,7 @@ __global__ void __launch_bounds__(P_THREADS, P_CTAS) k_plane_compress(const Comp
             P.c[ROW0][0] = c.R;
             c.ly = A;  // the row as row 16 of a chunk row that has it
             c.count0 = c.py == 0;
-            first_row_from<true, 8>(P, c, kd);
+            first_row_from<MODE, 8>(P, c, kd);
         }
         for (int r = t.r0; r < t.r1; ++r) {
             const int y0 = A * r;
@@ -486,11 +491,11 @@ __global__ void __launch_bounds__(P_THREADS, P_CTAS) k_plane_compress(const Comp
             c.count0 = c.py != 0 || r + 1 < t.r1;
             const bool full = d.nx - 1 - t.x0 >= SX && c.ly >= A;
             if (full) {
-                if (xfirst) levels_from<true, false, true, 8, true>(P, c, kd);
-                else levels_from<true, false, true, 8, false>(P, c, kd);
+                if (xfirst) levels_from<MODE, false, true, 8, true>(P, c, kd);
+                else levels_from<MODE, false, true, 8, false>(P, c, kd);
             } else {
-                if (xfirst) levels_from<true, false, false, 8, true>(P, c, kd);
-                else levels_from<true, false, false, 8, false>(P, c, kd);
+                if (xfirst) levels_from<MODE, false, false, 8, true>(P, c, kd);
+                else levels_from<MODE, false, false, 8, false>(P, c, kd);
             }
             // owned rows: row 0 of the lanes py = 0 is the one carried in
             uint32_t out[4][4];
@@ -564,8 +569,10 @@ __global__ void __launch_bounds__(P_THREADS, P_CTAS) k_plane_compress(const Comp
 
 // ---------------------------------------------------------- decompression
 // Codes of rows y0 + 1 .. y0 + 16, columns x0 .. x0 + 64.
-__device__ __forceinline__ void land_codes(unsigned char *land, const uint16_t *codes, Dims d, int z, int y0, int x0,
-                                           int width, int lane)
+// Returns the closing column's code of row y0 + 1 + lane (lanes 0 .. 15), a load that is
+// first needed when the landed rows are.
+__device__ __forceinline__ uint32_t land_codes(unsigned char *land, const uint16_t *codes, Dims d, int z, int y0,
+                                               int x0, int width, int lane)
 {
     uint16_t *dst = reinterpret_cast<uint16_t *>(land + P_LAND);
     const uint16_t *src = codes + ((size_t)z * d.ny + y0 + 1) * d.nx + x0;
@@ -587,9 +594,8 @@ __device__ __forceinline__ void land_codes(unsigned char *land, const uint16_t *
             if (r < ny && e < nx) dst[r * SX + e] = __ldg(src + (size_t)r * d.nx + e);
         }
     }
-    if (lane < A && lane < ny && SX < nx)
-        reinterpret_cast<uint16_t *>(land + P_COL)[lane] = __ldg(src + (size_t)lane * d.nx + SX);
     cp_async_commit();
+    return lane < A && lane < ny && SX < nx ? __ldg(src + (size_t)lane * d.nx + SX) : 0u;
 }
 
 __global__ void __launch_bounds__(P_THREADS, P_CTAS) k_plane_decompress(const DecompressArgs a, const Plan plan)
@@ -614,7 +620,6 @@ __global__ void __launch_bounds__(P_THREADS, P_CTAS) k_plane_decompress(const De
     c.cbias = kMagicBits - c.R;
     c.Rf = 0.0f;
     c.hist = c.spare = 0u;
-    c.global_bins = false;
     c.hist_g = nullptr;
     c.count0 = false;
     c.lane = lane;
@@ -641,7 +646,7 @@ __global__ void __launch_bounds__(P_THREADS, P_CTAS) k_plane_decompress(const De
     for (uint32_t it = blockIdx.x + gridDim.x * (uint32_t)warp; it < plan.items; it += step) {
         const Item t = item_of(plan, it);
         __syncwarp();
-        land_codes(land, a.codes, d, t.z, A * t.r0, t.x0, width, lane);
+        uint32_t col = land_codes(land, a.codes, d, t.z, A * t.r0, t.x0, width, lane);
         c.lx = d.nx - 1 - t.x0 - 8 * c.px;
         Patch P;
         {  // the run's first row
@@ -659,7 +664,7 @@ __global__ void __launch_bounds__(P_THREADS, P_CTAS) k_plane_decompress(const De
             for (int e = 1; e < 8; ++e) P.v[ROW0][e] = 0.0f;
             outliers_of(P, ROW0, a.xrec + g, c.py == 0);
             c.ly = A;
-            first_row_from<false, 8>(P, c, kd);
+            first_row_from<DECODE, 8>(P, c, kd);
         }
         float anc0, anc8;
         anchors_of(t.z, t.r0 + 1, t.x0, anc0, anc8);
@@ -678,13 +683,13 @@ __global__ void __launch_bounds__(P_THREADS, P_CTAS) k_plane_decompress(const De
                 P.c[j][1] = w.y;
                 P.c[j][2] = w.z;
                 P.c[j][3] = w.w;
-                P.mc[j] = reinterpret_cast<const uint16_t *>(land + P_COL)[lr];
+                P.mc[j] = __shfl_sync(0xffffffffu, col, lr);
             }
             P.v[ROW0][0] = anc0;  // anchors of the closing row (lanes py = 0)
             P.v[ROW0][8] = anc8;
             __syncwarp();
             if (r + 1 < t.r1) {
-                land_codes(land, a.codes, d, t.z, y0 + A, t.x0, width, lane);
+                col = land_codes(land, a.codes, d, t.z, y0 + A, t.x0, width, lane);
                 anchors_of(t.z, r + 2, t.x0, anc0, anc8);
             }
             c.ly = d.ny - 1 - y0;
@@ -710,14 +715,14 @@ __global__ void __launch_bounds__(P_THREADS, P_CTAS) k_plane_decompress(const De
                     outliers_of(P, j, base + (size_t)y * d.nx + 8 * c.px, in);
                     if (in && colin && P.mc[j] == 0u) P.v[j][8] = base[(size_t)y * d.nx + SX];
                 }
-                if (xfirst) levels_from<false, true, false, 8, true>(P, c, kd);
-                else levels_from<false, true, false, 8, false>(P, c, kd);
+                if (xfirst) levels_from<DECODE, true, false, 8, true>(P, c, kd);
+                else levels_from<DECODE, true, false, 8, false>(P, c, kd);
             } else if (full) {
-                if (xfirst) levels_from<false, false, true, 8, true>(P, c, kd);
-                else levels_from<false, false, true, 8, false>(P, c, kd);
+                if (xfirst) levels_from<DECODE, false, true, 8, true>(P, c, kd);
+                else levels_from<DECODE, false, true, 8, false>(P, c, kd);
             } else {
-                if (xfirst) levels_from<false, false, false, 8, true>(P, c, kd);
-                else levels_from<false, false, false, 8, false>(P, c, kd);
+                if (xfirst) levels_from<DECODE, false, false, 8, true>(P, c, kd);
+                else levels_from<DECODE, false, false, 8, false>(P, c, kd);
             }
             float *dst = a.xrec + ((size_t)t.z * d.ny + y0) * d.nx + t.x0;
             float o[8];
@@ -798,8 +803,8 @@ cudaError_t launch_planes(K kernel, const Args &a, size_t smem, cudaStream_t s)
 
 cudaError_t launch_plane_compress(const CompressArgs &a, cudaStream_t s)
 {
-    const size_t hist = 2 * a.radius <= P_HIST_BINS ? sizeof(uint32_t) * 2 * (size_t)a.radius : 0;
-    return launch_planes(k_plane_compress, a, P_HIST + hist, s);
+    if (2 * a.radius > P_HIST_BINS) return launch_planes(k_plane_compress<ENCODE_GBINS>, a, P_HIST, s);
+    return launch_planes(k_plane_compress<ENCODE>, a, P_HIST + sizeof(uint32_t) * 2 * (size_t)a.radius, s);
 }
 
 cudaError_t launch_plane_decompress(const DecompressArgs &a, cudaStream_t s)
