@@ -12,7 +12,6 @@
 namespace gi {
 namespace {
 
-constexpr int HQ_THREADS = 1024;
 constexpr int EQ_THREADS = 512;
 constexpr int EQ_MAX_BLOCKS = 1024;
 
@@ -22,21 +21,20 @@ struct ErrPartial {
     unsigned long long finite;
 };
 
-// One CTA over the 2R bins: counts, entropy (double, bins in ascending order
+// One block over the 2R bins: counts, entropy (double, bins in ascending order
 // per thread, then a fixed tree), largest |q| among kept codes.
-__global__ void __launch_bounds__(HQ_THREADS) k_hist_stats(const uint32_t *__restrict__ hist, int radius,
-                                                           interp_quality *out, int has_err)
+__device__ void hist_stats(const uint32_t *__restrict__ hist, int radius, interp_quality *out, int has_err)
 {
-    __shared__ double s_plogp[HQ_THREADS / 32];
-    __shared__ unsigned long long s_n[HQ_THREADS / 32], s_nz[HQ_THREADS / 32];
-    __shared__ int s_maxq[HQ_THREADS / 32];
+    __shared__ double s_plogp[EQ_THREADS / 32];
+    __shared__ unsigned long long s_n[EQ_THREADS / 32], s_nz[EQ_THREADS / 32];
+    __shared__ int s_maxq[EQ_THREADS / 32];
     __shared__ unsigned long long n_total;
     const int bins = 2 * radius;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // pass 1: totals
     unsigned long long n = 0, nz = 0;
     int maxq = 0;
-    for (int c = threadIdx.x; c < bins; c += HQ_THREADS) {
+    for (int c = threadIdx.x; c < bins; c += EQ_THREADS) {
         const uint32_t h = hist[c];
         n += h;
         if (c != radius) nz += h;  // nonzero quant-codes, outliers included
@@ -57,7 +55,7 @@ __global__ void __launch_bounds__(HQ_THREADS) k_hist_stats(const uint32_t *__res
     if (threadIdx.x == 0) {
         unsigned long long tn = 0, tz = 0;
         int tq = 0;
-        for (int w = 0; w < HQ_THREADS / 32; ++w) {
+        for (int w = 0; w < EQ_THREADS / 32; ++w) {
             tn += s_n[w];
             tz += s_nz[w];
             tq = max(tq, s_maxq[w]);
@@ -77,7 +75,7 @@ __global__ void __launch_bounds__(HQ_THREADS) k_hist_stats(const uint32_t *__res
     // pass 2: entropy H = -sum p log2 p, p = h / n
     const double inv_n = n_total ? 1.0 / (double)n_total : 0.0;
     double acc = 0.0;
-    for (int c = threadIdx.x; c < bins; c += HQ_THREADS) {
+    for (int c = threadIdx.x; c < bins; c += EQ_THREADS) {
         const uint32_t h = hist[c];
         if (h) {
             const double p = (double)h * inv_n;
@@ -90,71 +88,176 @@ __global__ void __launch_bounds__(HQ_THREADS) k_hist_stats(const uint32_t *__res
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
-        for (int w = 0; w < HQ_THREADS / 32; ++w) t += s_plogp[w];
+        for (int w = 0; w < EQ_THREADS / 32; ++w) t += s_plogp[w];
         out->entropy_bits = t;
     }
 }
 
-// Reconstruction error over the finite points of x: grid-stride partials,
-// the last CTA to finish folds them and writes the report.
-__global__ void __launch_bounds__(EQ_THREADS) k_err_stats(const float *__restrict__ x, const float *__restrict__ xr,
-                                                          unsigned long long n, ErrPartial *partials,
-                                                          unsigned int *counter, interp_quality *out)
+// Sums of (a - b)^2 to the accuracy of double sums without double arithmetic per point
+// (fp64 runs at 1/64 of the fp32 rate here, and five fp64 operations a point bound this
+// kernel at 0.77 ms for 384^3 points): the difference as an exact pair of floats (Knuth's
+// two-sum), its square as an exact pair (fused multiply-add), and a running pair whose
+// low word collects every rounding error; the pair is added to a double every 64 points.
+// A difference whose square would leave the exact range goes straight to the double.  The
+// maximum is kept as a pair too (rounding the pair to double gives what rounding the
+// difference would).
+struct ErrSum {
+    double sse, maxerr;
+    float hi, lo;    // pending part of the sum
+    float mhi, mlo;  // largest |difference| so far as an exact pair
+    float vmin, vmax;
+    unsigned long long bad;  // non-finite points of x (stored exactly, not counted)
+};
+
+__device__ __forceinline__ void err_flush(ErrSum &s)
 {
-    double sse = 0.0, maxerr = 0.0;
-    float lo = INFINITY, hi = -INFINITY;
-    unsigned long long fin = 0;
-    const unsigned long long tid = (unsigned long long)blockIdx.x * EQ_THREADS + threadIdx.x;
-    const unsigned long long nth = (unsigned long long)gridDim.x * EQ_THREADS;
-    for (unsigned long long i = tid; i < n; i += nth) {
-        const float a = __ldg(x + i);
-        if (!(fabsf(a) <= FLT_MAX)) continue;  // non-finite values are stored exactly
-        const float b = __ldg(xr + i);
-        const double d = (double)a - (double)b;
-        sse += d * d;
-        maxerr = fmax(maxerr, fabs(d));
-        lo = fminf(lo, a);
-        hi = fmaxf(hi, a);
-        ++fin;
+    s.sse += (double)s.hi + (double)s.lo;
+    s.hi = s.lo = 0.0f;
+}
+
+// Non-finite points, and differences whose square would leave the exact range.
+__device__ __forceinline__ void err_rare(ErrSum &s, float a, float b)
+{
+    if (!(fabsf(a) <= FLT_MAX)) {
+        ++s.bad;
+        return;
     }
+    s.vmin = fminf(s.vmin, a);
+    s.vmax = fmaxf(s.vmax, a);
+    const double d = (double)a - (double)b;
+    s.sse += d * d;
+    s.maxerr = fmax(s.maxerr, fabs(d));
+}
+
+__device__ __forceinline__ void err_point(ErrSum &s, float a, float b)
+{
+    // a - b = dh + dl exactly
+    const float dh = a - b, bv = a - dh, av = dh + bv;
+    float dl = (bv - b) + (a - av);
+    const float ad = fabsf(dh);
+    // squares of 2^-48 .. 2^55, and of 0, keep every bit of the pair (infinities and NaN fail)
+    if (!((ad >= 3.552713678800501e-15f || ad == 0.0f) && ad <= 3.602879701896397e16f)) {
+        err_rare(s, a, b);
+        return;
+    }
+    s.vmin = fminf(s.vmin, a);
+    s.vmax = fmaxf(s.vmax, a);
+    const float p = dh * dh;
+    const float e = __fmaf_rn(dl, dl, __fmaf_rn(2.0f * dh, dl, __fmaf_rn(dh, dh, -p)));
+    const float t = s.hi + p, q = t - s.hi;
+    const float r = (s.hi - (t - q)) + (p - q);
+    s.hi = t;
+    s.lo += r + e;
+    // |a - b| = ad + dl with dh's sign taken off
+    dl = __uint_as_float(__float_as_uint(dl) ^ (__float_as_uint(dh) & 0x80000000u));
+    const bool more = ad > s.mhi || (ad == s.mhi && dl > s.mlo);
+    s.mhi = more ? ad : s.mhi;
+    s.mlo = more ? dl : s.mlo;
+}
+
+__device__ __forceinline__ ErrPartial fold(ErrPartial a, const ErrPartial &b)
+{
+    a.sse += b.sse;
+    a.maxerr = fmax(a.maxerr, b.maxerr);
+    a.lo = fminf(a.lo, b.lo);
+    a.hi = fmaxf(a.hi, b.hi);
+    a.finite += b.finite;
+    return a;
+}
+
+// Block reduction in a fixed order; thread 0 holds the result.
+__device__ ErrPartial block_fold(ErrPartial p)
+{
+    __shared__ ErrPartial wp[EQ_THREADS / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
-        sse += __shfl_xor_sync(0xffffffffu, sse, off);
-        maxerr = fmax(maxerr, __shfl_xor_sync(0xffffffffu, maxerr, off));
-        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, off));
-        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, off));
-        fin += __shfl_xor_sync(0xffffffffu, fin, off);
+        ErrPartial o;
+        o.sse = __shfl_down_sync(0xffffffffu, p.sse, off);
+        o.maxerr = __shfl_down_sync(0xffffffffu, p.maxerr, off);
+        o.lo = __shfl_down_sync(0xffffffffu, p.lo, off);
+        o.hi = __shfl_down_sync(0xffffffffu, p.hi, off);
+        o.finite = __shfl_down_sync(0xffffffffu, p.finite, off);
+        p = fold(p, o);
     }
-    __shared__ ErrPartial wp[EQ_THREADS / 32];
-    __shared__ bool last;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) wp[warp] = ErrPartial{sse, maxerr, lo, hi, fin};
     __syncthreads();
-    if (threadIdx.x == 0) {
-        ErrPartial p = wp[0];
-        for (int w = 1; w < EQ_THREADS / 32; ++w) {
-            p.sse += wp[w].sse;
-            p.maxerr = fmax(p.maxerr, wp[w].maxerr);
-            p.lo = fminf(p.lo, wp[w].lo);
-            p.hi = fmaxf(p.hi, wp[w].hi);
-            p.finite += wp[w].finite;
+    if (lane == 0) wp[warp] = p;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int w = 1; w < EQ_THREADS / 32; ++w) p = fold(p, wp[w]);
+    return p;
+}
+
+// The report: block 0 takes the histogram, the others the reconstruction error over the
+// finite points of x (grid-stride, 16-byte loads where both fields allow them); the last
+// of them folds the partials, in a fixed order, and writes the error statistics.
+__global__ void __launch_bounds__(EQ_THREADS, 2) k_quality(const uint32_t *__restrict__ hist, int radius,
+                                                        const float *__restrict__ x, const float *__restrict__ xr,
+                                                        unsigned long long n, int vec, ErrPartial *partials,
+                                                        unsigned int *counter, interp_quality *out)
+{
+    if (blockIdx.x == 0) {
+        hist_stats(hist, radius, out, x != nullptr);
+        return;
+    }
+    const unsigned b = blockIdx.x - 1, nb = gridDim.x - 1;
+    const unsigned long long tid = (unsigned long long)b * EQ_THREADS + threadIdx.x;
+    const unsigned long long nth = (unsigned long long)nb * EQ_THREADS;
+    ErrSum s{0.0, 0.0, 0.0f, 0.0f, 0.0f, 0.0f, INFINITY, -INFINITY, 0ull};
+    unsigned long long points = 0, done = 0;
+    if (vec) {
+        const float4 *x4 = reinterpret_cast<const float4 *>(x), *r4 = reinterpret_cast<const float4 *>(xr);
+        const unsigned long long n4 = n / 4;
+        int pending = 0;
+        unsigned long long i = tid;
+        auto quad = [&](const float4 &v, const float4 &w) {
+            err_point(s, v.x, w.x);
+            err_point(s, v.y, w.y);
+            err_point(s, v.z, w.z);
+            err_point(s, v.w, w.w);
+        };
+        for (; i + nth < n4; i += 2 * nth) {  // four loads in flight
+            const float4 a = __ldcs(x4 + i), c = __ldcs(x4 + i + nth);
+            const float4 u = __ldcs(r4 + i), w = __ldcs(r4 + i + nth);
+            quad(a, u);
+            quad(c, w);
+            points += 8;
+            if (++pending == 8) {
+                err_flush(s);
+                pending = 0;
+            }
         }
-        partials[blockIdx.x] = p;
+        if (i < n4) {
+            quad(__ldcs(x4 + i), __ldcs(r4 + i));
+            points += 4;
+        }
+        err_flush(s);
+        done = n4 * 4;
+    }
+    int pending = 0;
+    for (unsigned long long i = done + tid; i < n; i += nth) {
+        err_point(s, __ldg(x + i), __ldg(xr + i));
+        ++points;
+        if (++pending == 64) {
+            err_flush(s);
+            pending = 0;
+        }
+    }
+    err_flush(s);
+    __shared__ bool last;
+    const ErrPartial p = block_fold(ErrPartial{s.sse, fmax(s.maxerr, (double)s.mhi + (double)s.mlo), s.vmin, s.vmax, points - s.bad});
+    if (threadIdx.x == 0) {
+        partials[b] = p;
         __threadfence();
-        last = atomicAdd(counter, 1u) == gridDim.x - 1;
+        last = atomicAdd(counter, 1u) == nb - 1;
     }
     __syncthreads();
-    if (!last || threadIdx.x != 0) return;
+    if (!last) return;
     __threadfence();
-    ErrPartial t = partials[0];
-    for (unsigned b = 1; b < gridDim.x; ++b) {  // fixed order: reproducible for a given grid
-        const ErrPartial p = partials[b];
-        t.sse += p.sse;
-        t.maxerr = fmax(t.maxerr, p.maxerr);
-        t.lo = fminf(t.lo, p.lo);
-        t.hi = fmaxf(t.hi, p.hi);
-        t.finite += p.finite;
-    }
+    ErrPartial t{0.0, 0.0, INFINITY, -INFINITY, 0ull};
+    for (unsigned k = threadIdx.x; k < nb; k += EQ_THREADS) t = fold(t, partials[k]);
+    t = block_fold(t);
+    if (threadIdx.x != 0) return;
     out->n_finite = t.finite;
     out->sse = t.sse;
     out->max_abs_err = t.maxerr;
@@ -173,20 +276,21 @@ size_t quality_workspace_bytes() { return 256 + sizeof(ErrPartial) * EQ_MAX_BLOC
 cudaError_t launch_quality(const uint32_t *hist, int radius, const float *x, const float *xr, uint64_t n,
                            interp_quality *out, void *ws, cudaStream_t s)
 {
-    const int has_err = x && xr && n > 0;
-    k_hist_stats<<<1, HQ_THREADS, 0, s>>>(hist, radius, out, has_err);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || !has_err) return e;
+    if (!(x && xr && n > 0)) {  // the histogram alone
+        k_quality<<<1, EQ_THREADS, 0, s>>>(hist, radius, nullptr, nullptr, 0ull, 0, nullptr, nullptr, out);
+        return cudaGetLastError();
+    }
     unsigned char *w = static_cast<unsigned char *>(ws);
     unsigned int *counter = reinterpret_cast<unsigned int *>(w);
-    e = cudaMemsetAsync(counter, 0, sizeof(unsigned int), s);
+    const cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned int), s);
     if (e != cudaSuccess) return e;
+    const int vec = aligned16(x) && aligned16(xr);
     unsigned long long blocks = (n + EQ_THREADS * 16ull - 1) / (EQ_THREADS * 16ull);
-    const unsigned long long cap = (unsigned long long)min(EQ_MAX_BLOCKS, 4 * sm_count());
+    const unsigned long long cap = (unsigned long long)min(EQ_MAX_BLOCKS, 2 * sm_count() - 1);  // one wave with block 0
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    k_err_stats<<<(unsigned)blocks, EQ_THREADS, 0, s>>>(x, xr, (unsigned long long)n,
-                                                        reinterpret_cast<ErrPartial *>(w + 256), counter, out);
+    k_quality<<<(unsigned)blocks + 1, EQ_THREADS, 0, s>>>(hist, radius, x, xr, (unsigned long long)n, vec,
+                                                         reinterpret_cast<ErrPartial *>(w + 256), counter, out);
     return cudaGetLastError();
 }
 
