@@ -201,13 +201,9 @@ int compress_nd(const interp_compress_item &it, interp_stream_t stream)
     if (it.ws_bytes < L.total) return INTERP_EWORKSPACE;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const Dims d = to_dims(it.dims);
-    const double alpha = effective_alpha(c, it.eb);
     unsigned char *ws = static_cast<unsigned char *>(it.d_ws);
-    unsigned int *counter = reinterpret_cast<unsigned int *>(ws + L.ctrl);
     uint32_t *bitmap = reinterpret_cast<uint32_t *>(ws + L.bitmap);
     uint32_t *blockcnt = reinterpret_cast<uint32_t *>(ws + L.blockcnt);
-    (void)counter;
-    (void)alpha;
     const gi::PrologueItem pro = prologue_item(it, L);
     cudaError_t e = gi::launch_prologue(&pro, 1, s);
     const gi::CompressArgs args{it.d_x, d, it.d_anchors, it.d_codes, bitmap, blockcnt, it.d_hist, c.radius,
@@ -459,11 +455,8 @@ int interp_huffman_encode(const uint16_t *d_codes, uint64_t n, int32_t radius, c
     if (n > 0 && (!d_codes || !d_words)) return INTERP_EINVAL;
     if (n >= (1ull << 32)) return INTERP_EINVAL;
     if (ws_bytes < interp_huffman_workspace_bytes(n, radius)) return INTERP_EWORKSPACE;
-    unsigned char *ws = static_cast<unsigned char *>(d_ws);
-    unsigned int *bad = reinterpret_cast<unsigned int *>(ws);
     return cuda_status(gi::launch_huffman_encode(d_codes, n, d_lengths, d_codewords, 2 * radius, d_offsets, d_words,
-                                                 capacity_words, reinterpret_cast<uint32_t *>(ws + 256), bad,
-                                                 reinterpret_cast<cudaStream_t>(stream)));
+                                                 capacity_words, d_ws, reinterpret_cast<cudaStream_t>(stream)));
 }
 
 int interp_huffman_decode(const uint32_t *d_words, const uint32_t *d_offsets, uint64_t n, int32_t radius,

@@ -8,23 +8,26 @@
 // to a whole word; offsets[k] is chunk k's first word, offsets[nchunks] the
 // total.  Chunks start on word boundaries, so they decode independently.
 //
-// Encoding: one warp per chunk, each lane 32 consecutive codes, ENC_WARPS chunks
-// per CTA.  A first pass sums the code lengths of each CTA's chunks (in words), a
-// one-CTA scan turns those sums into word offsets, and a second pass recomputes
-// its chunks' sizes, places them after the CTA's offset, and has every lane put
-// its codewords at its bit offset (a warp scan) in the warp's shared-memory copy
-// of the chunk, which is then written out with coalesced stores.
-// Decoding: one thread per chunk, reading its words in order: the next 10 bits
-// index a lookup table holding every whole codeword they contain (up to three
-// symbols and the bits they take); longer codewords take the canonical rule (per
-// length, the first codeword and the first symbol index).  Decoded codes are
-// staged per warp and stored coalesced.
+// Encoding: one pass.  A tile is ENC_WARPS chunks, one warp per chunk, each lane 32
+// consecutive codes; persistent CTAs take tiles in ascending order from a counter.  A
+// tile sums its chunks' words, publishes the sum, puts its codewords at their bit offsets
+// (a warp scan) into a shared-memory copy of the chunks, and only then looks back over
+// its predecessors' published sums for the words before it (the tiles it waits for were
+// taken earlier, so they run or are done), and writes its words out coalesced.  The codes
+// are read once; as sizes, scan and write passes they were read twice.
+// Decoding: one thread per chunk, reading its words in order.  The next 12 bits index a
+// lookup table with the whole codewords they contain (up to five symbols, as signed bytes
+// around the central code R, and the bits they take); other codewords take the canonical
+// rule (per length, the first codeword and the first symbol index).  Every thread does
+// DEC_STEPS lookups a round whatever they yield, so the lanes of a warp stay together;
+// what a round yields is appended to the thread's buffer in shared memory, whose full
+// groups of 16 codes it stores itself (32 bytes: whole sectors).
 #include <algorithm>
 #include <cstring>
 #include <queue>
 #include <vector>
 
-#include "common.cuh"
+#include "tma.cuh"
 
 namespace gi {
 namespace {
@@ -32,29 +35,34 @@ namespace {
 
 constexpr int HCHUNK = 1024;          // codes per chunk
 constexpr int HLANE = HCHUNK / 32;    // codes per lane
-constexpr int ENC_WARPS = 8;
+constexpr int ENC_WARPS = 16;         // chunks per tile
 constexpr int ENC_THREADS = 32 * ENC_WARPS;
 constexpr int MAX_LEN = 24;           // longest codeword the library builds
-constexpr int LUT_BITS = 10;
-constexpr int SCAN_THREADS = 1024;
-constexpr int SCAN_ITEMS = 8;
+constexpr int LUT_BITS = 12;          // lookup window: its table (32 KB) leaves two CTAs an SM
+constexpr int LUT_SYMS = 5;           // symbols of an entry
+constexpr uint32_t ENC_POLLS = 1u << 22;  // bounded wait for a predecessor
 constexpr int TAB_THREADS = 1024;
-constexpr int DEC_ROUND = 32;  // codes a decoding thread stages before its warp stores them
-constexpr int SYM_SMEM = 8192; // canonical symbol list kept in shared memory up to this many symbols
-constexpr int DEC_THREADS = 128;
+constexpr int DEC_STEPS = 4;    // lookups a round: at most 20 codes onto at most 15 pending ones
+constexpr int DEC_GROUP = 16;   // codes a thread stores at a time
+constexpr int DEC_PITCH = 80;   // bytes of a thread's code buffer (35 codes and the 4 that a last entry
+                                // may overwrite) and of its ring of stream words; an odd number of
+                                // 16-byte units: a warp's accesses spread over the banks
+constexpr int DEC_RING = 16;    // words of the ring, four 16-byte blocks
+constexpr int SYM_SMEM = 8192;  // canonical symbol list kept in shared memory up to this many symbols
+constexpr int DEC_THREADS = 448;  // two CTAs an SM hold one field of 512^3 codes in one wave
+static_assert(2 * (DEC_GROUP - 1 + DEC_STEPS * LUT_SYMS + LUT_SYMS - 1) <= DEC_PITCH, "a round fits the buffer");
+static_assert(4 * DEC_RING <= DEC_PITCH && 31 + DEC_STEPS * MAX_LEN < 32 * 4, "a round takes at most 3 words");
 
-// Device decode tables, built per call from the code lengths.
+// Canonical decode tables, built per call from the code lengths.
 struct DecodeTables {
     uint32_t first[MAX_LEN + 2];      // first codeword of each length (canonical)
     uint32_t count[MAX_LEN + 2];      // codewords of each length
     uint32_t base[MAX_LEN + 2];       // index in `symbols` of each length's first symbol
-    // The whole codewords (up to 3) that the next LUT_BITS bits hold: bits 0-15, 16-31,
-    // 32-47 the symbols, 48-51 / 52-55 / 56-59 the bits consumed after 1 / 2 / 3 of
-    // them, 60-61 their number (0: the first codeword is longer than LUT_BITS).
-    unsigned long long lut[1 << LUT_BITS];
     int max_len;
 };
-// followed by uint16_t symbols[2R] in canonical order
+// followed, at TABLES_BYTES, by uint16_t symbols[2R] in canonical order
+constexpr size_t TABLES_BYTES = 8512;
+static_assert(sizeof(DecodeTables) <= TABLES_BYTES, "decode tables fit their room");
 
 // A lane's 32 consecutive codes (64 bytes) as four 16-byte loads when the chunk is
 // whole and the codes array is 16-byte aligned; c[j] is code j of the lane.
@@ -86,187 +94,191 @@ __device__ __forceinline__ int lane_codes(const uint16_t *__restrict__ codes, un
 
 __device__ __forceinline__ uint32_t code_at(const uint32_t w[16], int j) { return (w[j >> 1] >> (16 * (j & 1))) & 0xffffu; }
 
-// ---- encode, pass 1: words per chunk, summed over each CTA's ENC_WARPS chunks
-template <bool smem_tab>
-__global__ void __launch_bounds__(ENC_THREADS) k_huff_sizes(const uint16_t *__restrict__ codes, unsigned long long n,
-                                                           const uint8_t *__restrict__ lengths, int nsym, bool vec,
-                                                           uint32_t *block_words, unsigned long long nchunks)
+// ---- encode
+constexpr int MAX_WORDS = (HCHUNK * MAX_LEN + 31) / 32;  // words of a chunk at the longest codewords
+constexpr unsigned long long TILE_SUM = 1ull << 32, TILE_PREFIX = 2ull << 32;  // status of a tile: its own
+// words, or those of all tiles up to it (low 32 bits); 0 = not published yet
+
+__device__ __forceinline__ unsigned long long load_status(const unsigned long long *p)
 {
-    extern __shared__ uint8_t len_sm[];  // nsym code lengths when they fit, else read from global memory
-    __shared__ uint32_t warp_words[ENC_WARPS];
-    if (smem_tab) {
-        for (int i = threadIdx.x; i < nsym; i += ENC_THREADS) len_sm[i] = lengths[i];
-        __syncthreads();
-    }
-    const uint8_t *len_s = smem_tab ? len_sm : lengths;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned long long chunk = (unsigned long long)blockIdx.x * ENC_WARPS + warp;
-    uint32_t w[16];
-    // past the last chunk the lane holds no codes (its first index is past n)
-    const int cnt = lane_codes(codes, n, chunk * HCHUNK + (unsigned long long)lane * HLANE, vec, w);
-    uint32_t bits = 0;
-#pragma unroll
-    for (int j = 0; j < HLANE; ++j)
-        if (j < cnt) bits += len_s[code_at(w, j)];
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) bits += __shfl_xor_sync(0xffffffffu, bits, off);
-    if (lane == 0) warp_words[warp] = (bits + 31) / 32;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t sum = 0;
-#pragma unroll
-        for (int k = 0; k < ENC_WARPS; ++k) sum += warp_words[k];
-        block_words[blockIdx.x] = sum;
-    }
-    (void)nchunks;
+    return *reinterpret_cast<const volatile unsigned long long *>(p);
+}
+__device__ __forceinline__ void publish(unsigned long long *p, unsigned long long v)
+{
+    *reinterpret_cast<volatile unsigned long long *>(p) = v;
 }
 
-// ---- one-CTA exclusive scan of the CTAs' word counts (in place); the total goes to *total
-__global__ void __launch_bounds__(SCAN_THREADS) k_huff_scan(uint32_t *counts, unsigned long long m, uint32_t *total)
+// Words before tile t (one warp, 32 predecessors a step; looking at 320 at once, or taking
+// the next tile's number early, made the tiles wait for one another longer: 161 us against
+// 184 .. 207 on 2^27 codes).  A predecessor that does not publish in time sets the flag and
+// gives 0: the stream is then invalid, as its flag says.
+__device__ __forceinline__ uint32_t words_before(const unsigned long long *status, uint32_t t, unsigned int *bad)
 {
-    constexpr int TILE = SCAN_THREADS * SCAN_ITEMS;
-    __shared__ uint32_t tile[TILE];  // coalesced in and out; each thread scans SCAN_ITEMS consecutive entries
-    __shared__ unsigned long long warp_sum[SCAN_THREADS / 32];
-    __shared__ unsigned long long carry;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) carry = 0;
-    for (unsigned long long base = 0; base < m; base += TILE) {
-#pragma unroll
-        for (int k = 0; k < SCAN_ITEMS; ++k) {
-            const unsigned long long i = base + (unsigned long long)(k * SCAN_THREADS + tid);
-            tile[k * SCAN_THREADS + tid] = i < m ? counts[i] : 0u;
+    const int lane = threadIdx.x & 31;
+    uint32_t sum = 0;
+    for (long long top = (long long)t - 1;; top -= 32) {
+        const long long k = top - lane;
+        unsigned long long v = k >= 0 ? load_status(status + k) : TILE_PREFIX;
+        uint32_t polls = 0;
+        while (!__all_sync(0xffffffffu, v != 0ull)) {
+            if (++polls == ENC_POLLS) {
+                if (lane == 0) atomicOr(bad, 1u);
+                return 0u;
+            }
+            if (k >= 0) v = load_status(status + k);
         }
-        __syncthreads();
-        uint32_t v[SCAN_ITEMS];
+        const uint32_t prefix = __ballot_sync(0xffffffffu, v >= TILE_PREFIX);
+        const int last = prefix ? __ffs(prefix) - 1 : 31;  // the nearest tile whose prefix is known
+        sum += __reduce_add_sync(0xffffffffu, lane <= last ? (uint32_t)v : 0u);
+        if (prefix) return sum;
+    }
+}
+
+// A lane's codewords, appended MSB first.  Words wholly inside the lane's range are
+// stored, the first and the last (shared with the neighbouring lanes) are OR-ed in.
+struct BitRun {
+    uint32_t hi, lo;         // a 64-bit shift register: its low nacc bits are pending, bits above them are stale
+    uint32_t nacc, wi, first;
+    uint32_t *sw;
+    uint32_t head;  // the first word, once it is full
+    __device__ __forceinline__ void push(uint32_t bits, uint32_t len)  // len <= 32
+    {
+        hi = __funnelshift_lc(lo, hi, len);
+        lo = __funnelshift_lc(0u, lo, len) | bits;
+        nacc += len;
+        const bool full = nacc >= 32;
+        nacc &= 31u;
+        const uint32_t word = __funnelshift_r(lo, hi, nacc);
+        head = full && wi == first ? word : head;
+        if (full && wi != first) sw[wi] = word;
+        wi += full ? 1u : 0u;
+    }
+};
+
+// SMEM_TAB: the codebook (length << 24 | codeword) in shared memory.
+template <bool SMEM_TAB>
+__global__ void __launch_bounds__(ENC_THREADS, 2) k_huff_encode(const uint16_t *__restrict__ codes, unsigned long long n,
+                                                               const uint8_t *__restrict__ lengths,
+                                                               const uint32_t *__restrict__ codewords, int nsym,
+                                                               bool vec, unsigned long long *status,
+                                                               unsigned int *ticket, uint32_t tiles,
+                                                               uint32_t *offsets, uint32_t *words, uint32_t nchunks,
+                                                               unsigned long long capacity_words, unsigned int *bad)
+{
+    extern __shared__ __align__(16) uint32_t enc_sm[];  // ENC_WARPS chunk stages, then the table
+    __shared__ uint32_t warp_words[ENC_WARPS];
+    __shared__ uint32_t tile_s, base_s;
+    uint32_t *tab = enc_sm + ENC_WARPS * MAX_WORDS;
+    bool longest16 = true, packed = SMEM_TAB;
+    {
+        int l16 = 0, l24 = 0;
+        for (int i = threadIdx.x; i < nsym; i += ENC_THREADS) {
+            const uint32_t len = lengths[i];
+            l16 |= len > 16;
+            l24 |= len > MAX_LEN;  // not a codebook this library builds: read unpacked
+            if (SMEM_TAB) tab[i] = (len << 24) | codewords[i];
+        }
+        longest16 = !__syncthreads_or(l16);
+        if (__syncthreads_or(l24)) packed = false;
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t *sw = enc_sm + warp * MAX_WORDS;
+    for (;;) {
+        if (threadIdx.x == 0) tile_s = atomicAdd(ticket, 1u);
+        __syncthreads();  // also: every warp is done with the previous tile's shared words
+        const uint32_t t = tile_s;
+        if (t >= tiles) break;
+        const uint32_t chunk = t * ENC_WARPS + warp;
+        const unsigned long long i0 = (unsigned long long)chunk * HCHUNK + (unsigned)(lane * HLANE);
+        uint32_t e[HLANE];  // table entries
+        uint32_t bits = 0;
+        {
+            uint32_t w[16];
+            // past the last chunk the lane holds no codes (its first index is past n)
+            const int cnt = lane_codes(codes, n, i0, vec, w);
+            if (packed) {
 #pragma unroll
-        for (int k = 0; k < SCAN_ITEMS; ++k) v[k] = tile[tid * SCAN_ITEMS + k];
-        unsigned long long tsum = 0;
+                for (int j = 0; j < HLANE; ++j) e[j] = tab[code_at(w, j)];
+                if (cnt < HLANE)
 #pragma unroll
-        for (int k = 0; k < SCAN_ITEMS; ++k) tsum += v[k];
-        unsigned long long incl = tsum;
+                    for (int j = 0; j < HLANE; ++j) e[j] = j < cnt ? e[j] : 0u;
+#pragma unroll
+                for (int j = 0; j < HLANE; ++j) bits = __dp4a(e[j], 0x01000000u, bits);  // the top byte
+            } else {
+#pragma unroll
+                for (int j = 0; j < HLANE; ++j)
+                    if (j < cnt) bits += lengths[code_at(w, j)];
+            }
+        }
+        uint32_t pos = bits;  // inclusive, then exclusive scan of the lanes' bit counts
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
-            const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off) incl += y;
+            const uint32_t y = __shfl_up_sync(0xffffffffu, pos, off);
+            if (lane >= off) pos += y;
         }
-        if (lane == 31) warp_sum[warp] = incl;
+        const uint32_t nw = (__shfl_sync(0xffffffffu, pos, 31) + 31) / 32;  // the chunk's words
+        pos -= bits;
+        if (lane == 0) warp_words[warp] = nw;
         __syncthreads();
+        const uint32_t v = lane < ENC_WARPS ? warp_words[lane] : 0u;
         if (warp == 0) {
-            unsigned long long ws = warp_sum[lane];
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const unsigned long long y = __shfl_up_sync(0xffffffffu, ws, off);
-                if (lane >= off) ws += y;
+            const uint32_t total = __reduce_add_sync(0xffffffffu, v);
+            if (lane == 0) {
+                publish(status + t, (t == 0 ? TILE_PREFIX : TILE_SUM) | total);
             }
-            warp_sum[lane] = ws;
         }
-        __syncthreads();
-        unsigned long long before = carry + (warp ? warp_sum[warp - 1] : 0ull) + incl - tsum;
+        const bool fits = nw <= (uint32_t)MAX_WORDS;  // false: lengths above MAX_LEN
+        if (fits) {
+            for (uint32_t i = lane; i < nw; i += 32) sw[i] = 0u;
+            __syncwarp();
+            BitRun r;
+            r.hi = r.lo = 0;
+            r.nacc = pos & 31;  // the leading part of the first word is zero
+            r.wi = r.first = pos >> 5;
+            r.sw = sw;
+            r.head = 0;
+            if (packed && longest16) {  // two codewords at a time: at most 32 bits
 #pragma unroll
-        for (int k = 0; k < SCAN_ITEMS; ++k) {
-            tile[tid * SCAN_ITEMS + k] = (uint32_t)before;
-            before += v[k];
-        }
-        __syncthreads();
+                for (int j = 0; j < HLANE; j += 2) {
+                    const uint32_t lb = e[j + 1] >> 24;
+                    r.push(((e[j] & 0xffffffu) << lb) | (e[j + 1] & 0xffffffu), (e[j] >> 24) + lb);
+                }
+            } else if (packed) {
 #pragma unroll
-        for (int k = 0; k < SCAN_ITEMS; ++k) {
-            const unsigned long long i = base + (unsigned long long)(k * SCAN_THREADS + tid);
-            if (i < m) counts[i] = tile[k * SCAN_THREADS + tid];
+                for (int j = 0; j < HLANE; ++j) r.push(e[j] & 0xffffffu, e[j] >> 24);
+            } else {
+#pragma unroll 1
+                for (unsigned long long i = i0; i < n && i < i0 + HLANE; ++i) r.push(codewords[codes[i]], lengths[codes[i]]);
+            }
+            if (r.wi != r.first) atomicOr(&sw[r.first], r.head);
+            if (r.nacc) atomicOr(&sw[r.wi], r.lo << (32 - r.nacc));
         }
-        if (tid == SCAN_THREADS - 1) carry = before;
+        if (warp == 0) {
+            const uint32_t b = t ? words_before(status, t, bad) : 0u;
+            const uint32_t total = __reduce_add_sync(0xffffffffu, v);
+            if (lane == 0) {
+                if (t) publish(status + t, TILE_PREFIX | (unsigned long long)(uint32_t)(b + total));
+                base_s = b;
+            }
+        }
         __syncthreads();
+        const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? v : 0u);  // words of the tile before this chunk
+        if (chunk < nchunks) {
+            const unsigned long long w0 = (unsigned long long)base_s + before;
+            if (lane == 0) {
+                offsets[chunk] = (uint32_t)w0;
+                if (chunk == nchunks - 1) offsets[nchunks] = (uint32_t)(w0 + nw);
+            }
+            if (!fits || w0 + nw > capacity_words) {  // too little room
+                if (lane == 0) atomicOr(bad, 1u);
+            } else {
+                for (uint32_t i = lane; i < nw; i += 32) words[w0 + i] = sw[i];
+            }
+        }
     }
-    if (tid == 0) *total = (uint32_t)carry;
 }
 
-// ---- encode, pass 2: place the codewords
-constexpr int MAX_WORDS = (HCHUNK * MAX_LEN + 31) / 32;  // words of a chunk at the longest codewords
-
-template <bool smem_tab>
-__global__ void __launch_bounds__(ENC_THREADS) k_huff_write(const uint16_t *__restrict__ codes, unsigned long long n,
-                                                           const uint8_t *__restrict__ lengths,
-                                                           const uint32_t *__restrict__ codewords, int nsym, bool vec,
-                                                           const uint32_t *__restrict__ block_offset,
-                                                           uint32_t *offsets, uint32_t *words,
-                                                           unsigned long long nchunks,
-                                                           unsigned long long capacity_words, unsigned int *bad)
-{
-    __shared__ uint32_t stage[ENC_WARPS * MAX_WORDS];
-    __shared__ uint32_t warp_words[ENC_WARPS];
-    extern __shared__ uint32_t tab_sm[];  // nsym codewords, then nsym lengths (bytes), when they fit
-    const uint32_t *tab_s = codewords;
-    const uint8_t *len_s = lengths;
-    if (smem_tab) {
-        uint8_t *l = reinterpret_cast<uint8_t *>(tab_sm + nsym);
-        for (int i = threadIdx.x; i < nsym; i += ENC_THREADS) {
-            tab_sm[i] = codewords[i];
-            l[i] = lengths[i];
-        }
-        __syncthreads();
-        tab_s = tab_sm;
-        len_s = l;
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned long long chunk = (unsigned long long)blockIdx.x * ENC_WARPS + warp;
-    uint32_t w[16];
-    const int cnt = lane_codes(codes, n, chunk * HCHUNK + (unsigned long long)lane * HLANE, vec, w);
-    uint32_t bits = 0;
-#pragma unroll
-    for (int j = 0; j < HLANE; ++j)
-        if (j < cnt) bits += len_s[code_at(w, j)];
-    uint32_t pos = bits;  // inclusive, then exclusive scan of the lanes' bit counts
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, pos, off);
-        if (lane >= off) pos += y;
-    }
-    const uint32_t nw = (__shfl_sync(0xffffffffu, pos, 31) + 31) / 32;  // the chunk's words
-    pos -= bits;
-    if (lane == 0) warp_words[warp] = nw;
-    __syncthreads();
-    unsigned long long w0 = block_offset[blockIdx.x];
-    for (int k = 0; k < warp; ++k) w0 += warp_words[k];
-    if (chunk >= nchunks) return;  // whole warps leave together, after the CTA's barrier
-    if (lane == 0) offsets[chunk] = (uint32_t)w0;
-    uint32_t *sw = stage + warp * MAX_WORDS;
-    if (nw > (uint32_t)MAX_WORDS || w0 + nw > capacity_words) {  // lengths above MAX_LEN,
-        if (lane == 0) atomicOr(bad, 1u);                        // or too little room
-        return;
-    }
-    for (uint32_t i = lane; i < nw; i += 32) sw[i] = 0u;
-    __syncwarp();
-    // accumulate the lane's bits MSB first from its start position; words wholly
-    // inside the lane's range are stored, the first and last (shared with the
-    // neighbouring lanes) are OR-ed in
-    // (hi, lo) is a 64-bit shift register; its low nacc bits are pending (bits above them
-    // are stale and never read: a word is taken from bits nacc-32 .. nacc-1)
-    uint32_t hi = 0, lo = 0;
-    uint32_t nacc = pos & 31;          // pending bits (the leading part of the first word is zero)
-    uint32_t wi = pos >> 5;            // word being assembled
-    const uint32_t first_word = wi;
-#pragma unroll
-    for (int j = 0; j < HLANE; ++j) {
-        if (j >= cnt) break;
-        const uint32_t c = code_at(w, j);
-        const uint32_t len = len_s[c];  // 1..24
-        hi = __funnelshift_l(lo, hi, len);
-        lo = (lo << len) | tab_s[c];
-        nacc += len;
-        if (nacc >= 32) {  // a full word: pending bits nacc-32 .. nacc-1
-            const uint32_t word = __funnelshift_r(lo, hi, nacc - 32);
-            if (wi == first_word) atomicOr(&sw[wi], word);
-            else sw[wi] = word;
-            ++wi;
-            nacc -= 32;
-        }
-    }
-    if (nacc) atomicOr(&sw[wi], lo << (32 - nacc));  // nacc < 32: all pending bits are in lo
-    __syncwarp();
-    for (uint32_t i = lane; i < nw; i += 32) words[w0 + i] = sw[i];
-}
-
-// ---- decode tables from the lengths (one CTA): thread 0 lays out the canonical
-// order (one pass over the symbols), then all threads fill the lookup table
+// ---- decode tables from the lengths (one CTA)
 __global__ void __launch_bounds__(TAB_THREADS) k_huff_tables(const uint8_t *__restrict__ lengths,
                                                              const uint32_t *__restrict__ codewords, int nsym,
                                                              DecodeTables *t, uint16_t *symbols, unsigned int *bad)
@@ -276,7 +288,6 @@ __global__ void __launch_bounds__(TAB_THREADS) k_huff_tables(const uint8_t *__re
     __shared__ uint32_t wcnt[NW][NL];  // per warp: symbols of each length, then their offset in the length's run
     __shared__ int maxl_s;
     __shared__ unsigned int bad_s;
-    __shared__ uint32_t lut1[1 << LUT_BITS];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid < NL) {
         cnt_s[tid] = 0u;
@@ -340,150 +351,226 @@ __global__ void __launch_bounds__(TAB_THREADS) k_huff_tables(const uint8_t *__re
         }
         __syncthreads();
     }
-    // one-codeword table (symbol << 8 | length, 0 = longer than LUT_BITS), then the
-    // entries with every whole codeword of the LUT_BITS-bit window
-    for (int i = tid; i < (1 << LUT_BITS); i += TAB_THREADS) lut1[i] = 0u;
-    __syncthreads();
-    for (int s = tid; s < nsym; s += TAB_THREADS) {
-        const int l = lengths[s];
-        if (!l || l > LUT_BITS) continue;
-        const uint32_t lo = codewords[s] << (LUT_BITS - l), hi = lo + (1u << (LUT_BITS - l));
-        for (uint32_t v = lo; v < hi && v < (1u << LUT_BITS); ++v) lut1[v] = ((uint32_t)s << 8) | (uint32_t)l;
-    }
-    __syncthreads();
-    constexpr uint32_t MASK = (1u << LUT_BITS) - 1u;
-    for (int v = tid; v < (1 << LUT_BITS); v += TAB_THREADS) {
-        unsigned long long e = 0;
-        uint32_t used = 0;
-        int n = 0;
-        for (; n < 3; ++n) {
-            const uint32_t e1 = lut1[((uint32_t)v << used) & MASK];  // bits past the window read as 0
-            const uint32_t l = e1 & 0xffu;
-            if (!e1 || used + l > (uint32_t)LUT_BITS) break;  // not a whole codeword of the window
-            used += l;
-            e |= (unsigned long long)(e1 >> 8) << (16 * n);
-            e |= (unsigned long long)used << (48 + 4 * n);
-        }
-        t->lut[v] = e | ((unsigned long long)n << 60);
-    }
 }
 
 // ---- decode: one thread per chunk
-__global__ void __launch_bounds__(DEC_THREADS) k_huff_decode(const uint32_t *__restrict__ words,
-                                                            const uint32_t *__restrict__ offsets,
-                                                            unsigned long long n, const DecodeTables *__restrict__ tg,
-                                                            const uint16_t *__restrict__ symbols, int nsym_smem,
-                                                            uint16_t *codes, unsigned long long nchunks, bool vec,
-                                                            unsigned int *bad)
+
+// The lengths above LUT_BITS that have codewords, for the canonical rule.
+struct LongCodes {
+    uint4 l[MAX_LEN - LUT_BITS];  // 32 - length, first codeword, number of codewords, first symbol's index
+    int n;
+};
+
+// Byte permutation with sign replication (selector bit 3), which __byte_perm masks off.
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t sel)
+{
+    uint32_t r;
+    asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r) : "r"(a), "r"(sel));
+    return r;
+}
+
+// One group of DEC_GROUP codes from shared to global memory.  VEC: bytes the destination is
+// aligned to (32, 16 or 2).
+template <int VEC>
+__device__ __forceinline__ void store_group(uint16_t *dst, const unsigned char *src)
+{
+    const uint4 a = reinterpret_cast<const uint4 *>(src)[0], b = reinterpret_cast<const uint4 *>(src)[1];
+    if (VEC == 32) {
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(dst), "r"(a.x), "r"(a.y),
+                     "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+                     : "memory");
+    } else if (VEC == 16) {
+        reinterpret_cast<uint4 *>(dst)[0] = a;
+        reinterpret_cast<uint4 *>(dst)[1] = b;
+    } else {
+        const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            dst[2 * k] = (uint16_t)(w[k] & 0xffffu);
+            dst[2 * k + 1] = (uint16_t)(w[k] >> 16);
+        }
+    }
+}
+
+template <int VEC>
+__global__ void __launch_bounds__(DEC_THREADS, 2) k_huff_decode(const uint32_t *__restrict__ words,
+                                                               const uint32_t *__restrict__ offsets,
+                                                               unsigned long long n, const DecodeTables *__restrict__ tg,
+                                                               const uint16_t *__restrict__ symbols, int nsym,
+                                                               int nsym_smem, uint16_t *codes,
+                                                               unsigned long long nchunks, unsigned int *bad)
 {
     __shared__ DecodeTables t;
-    __shared__ uint32_t stage[DEC_THREADS * (DEC_ROUND / 2 + 1)];  // a row of DEC_ROUND codes per thread, padded
-    extern __shared__ uint16_t sym_s[];  // the symbol list when it fits (nsym_smem)
+    __shared__ LongCodes lc;
+    extern __shared__ __align__(16) unsigned char dec_sm[];
+    uint2 *lut = reinterpret_cast<uint2 *>(dec_sm);
+    unsigned char *bufs = dec_sm + sizeof(uint2) * (1 << LUT_BITS);
+    unsigned char *buf = bufs + DEC_PITCH * threadIdx.x;
+    uint32_t *ring = reinterpret_cast<uint32_t *>(bufs + DEC_PITCH * (blockDim.x + threadIdx.x));
+    uint16_t *sym_s = reinterpret_cast<uint16_t *>(bufs + 2 * DEC_PITCH * blockDim.x);
     {
         const uint32_t *src = reinterpret_cast<const uint32_t *>(tg);
         uint32_t *dst = reinterpret_cast<uint32_t *>(&t);
-        for (int i = threadIdx.x; i < (int)(sizeof(DecodeTables) / 4); i += DEC_THREADS) dst[i] = src[i];
-        for (int i = threadIdx.x; i < nsym_smem; i += DEC_THREADS) sym_s[i] = symbols[i];
+        for (int i = threadIdx.x; i < (int)(sizeof(DecodeTables) / 4); i += blockDim.x) dst[i] = src[i];
+        for (int i = threadIdx.x; i < nsym_smem; i += blockDim.x) sym_s[i] = symbols[i];
     }
     __syncthreads();
     const uint16_t *sym_tab = nsym_smem ? sym_s : symbols;
-    constexpr int RW = DEC_ROUND / 2 + 1;  // row pitch in words: thread rows fall in distinct banks
-    const int lane = threadIdx.x & 31;
-    const unsigned long long chunk = (unsigned long long)blockIdx.x * DEC_THREADS + threadIdx.x;
-    const unsigned long long chunk0 = chunk - lane;  // the warp's first chunk
-    if (chunk0 >= nchunks) return;                  // whole warps leave together
-    const bool live = chunk < nchunks;
-    const uint32_t *w = words;
-    uint32_t nw = 0;
-    if (live) {
-        w = words + offsets[chunk];
-        nw = offsets[chunk + 1] - offsets[chunk];
+    const int R = nsym / 2, maxl = t.max_len;
+    if (threadIdx.x == 0) {
+        lc.n = 0;
+        for (int l = LUT_BITS + 1; l <= maxl; ++l)
+            if (t.count[l]) lc.l[lc.n++] = make_uint4(32u - l, t.first[l], t.count[l], t.base[l]);
     }
-    // 64-bit window: the next 64 bits of the chunk, left-aligned; the word after it is
-    // loaded one refill ahead of its use
-    unsigned long long win = ((unsigned long long)(nw > 0 ? w[0] : 0u) << 32) | (nw > 1 ? w[1] : 0u);
-    uint32_t ahead = nw > 2 ? w[2] : 0u;
-    uint32_t next = 3;    // next word to take
-    int avail = 64;       // valid bits in win (beyond the chunk's words they are zeros)
-    const int cnt = live ? (int)min((unsigned long long)HCHUNK, n - chunk * HCHUNK) : 0;
-    const int maxl = t.max_len;
-    bool ok = true;
-    uint16_t *row = reinterpret_cast<uint16_t *>(stage + threadIdx.x * RW);
-    const uint32_t *wrows = stage + (threadIdx.x - lane) * RW;
-    // the warp's 32 chunks all hold HCHUNK codes and the codes are 4-byte aligned: the
-    // store phase needs no checks; each lane stores the words 2*(lane&15), +1 of row
-    // r + (lane >> 4) through a running pointer
-    const bool fast_store = vec && (chunk0 + 32) * HCHUNK <= n;
-    uint32_t *store_base = reinterpret_cast<uint32_t *>(codes + (chunk0 + (lane >> 4)) * HCHUNK) + (lane & 15);
-    for (int j0 = 0; j0 < HCHUNK; j0 += DEC_ROUND) {
-        const int jn = ok ? min(DEC_ROUND, cnt - j0) : 0;
-        int j = 0;
-        while (j < jn) {
-            const uint32_t top = (uint32_t)(win >> 32);
-            const unsigned long long e = t.lut[top >> (32 - LUT_BITS)];
-            const int ne = (int)(e >> 60);
-            uint32_t len;
-            if (ne) {  // up to three whole codewords; take what the round still needs
-                const int take = min(ne, jn - j);
-                row[j] = (uint16_t)e;
-                if (take > 1) row[j + 1] = (uint16_t)(e >> 16);
-                if (take > 2) row[j + 2] = (uint16_t)(e >> 32);
-                len = (uint32_t)(e >> (48 + 4 * (take - 1))) & 0xfu;
-                j += take;
-            } else {  // longer codeword: the canonical rule, length by length
-                len = 0;
-                uint32_t sym = 0;
-                for (int l = LUT_BITS + 1; l <= maxl; ++l) {
-                    const uint32_t v = top >> (32 - l);
-                    if (t.count[l] && v >= t.first[l] && v - t.first[l] < t.count[l]) {
-                        sym = sym_tab[t.base[l] + (v - t.first[l])];
-                        len = (uint32_t)l;
-                        break;
+    // one-codeword table (symbol << 8 | length, 0: longer than the window) in the buffers' room
+    uint32_t *lut1 = reinterpret_cast<uint32_t *>(bufs);
+    for (int v = threadIdx.x; v < (1 << LUT_BITS); v += blockDim.x) {
+        uint32_t e = 0;
+        for (int l = 1; l <= min(maxl, LUT_BITS); ++l) {
+            const uint32_t c = (uint32_t)v >> (LUT_BITS - l);
+            if (c >= t.first[l] && c - t.first[l] < t.count[l]) {
+                e = ((uint32_t)sym_tab[t.base[l] + (c - t.first[l])] << 8) | (uint32_t)l;
+                break;
+            }
+        }
+        lut1[v] = e;
+    }
+    __syncthreads();
+    // lookup table: word x and the low byte of y the symbols - R, then the bits taken by all
+    // of them (y bits 8-11) and their number (y bits 12-14).  Number 0 and some bits: one
+    // codeword whose symbol (word x) is no byte from R; number 0 and no bits: a longer codeword.
+    for (int v = threadIdx.x; v < (1 << LUT_BITS); v += blockDim.x) {
+        unsigned long long e = 0;
+        uint32_t used = 0, k = 0;
+        while (k < (uint32_t)LUT_SYMS) {
+            const uint32_t e1 = lut1[((uint32_t)v << used) & ((1u << LUT_BITS) - 1u)];  // then zeros
+            const uint32_t len = e1 & 0xffu;
+            const int delta = (int)(e1 >> 8) - R;
+            if (!e1 || used + len > (uint32_t)LUT_BITS) break;  // not a whole codeword of the window
+            if (delta < -128 || delta > 127) {
+                if (k == 0) {
+                    e = e1 >> 8;
+                    used = len;
+                }
+                break;
+            }
+            e |= (unsigned long long)((uint32_t)delta & 0xffu) << (8 * k);
+            used += len;
+            ++k;
+        }
+        lut[v] = make_uint2((uint32_t)e, (uint32_t)(e >> 32) | (used << 8) | (k << 12));
+    }
+    __syncthreads();
+
+    const unsigned long long chunk = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool live = chunk < nchunks;
+    // The chunk's words arrive in 16-byte blocks through the ring, asynchronously and two
+    // rounds ahead.  Word q counts from the block that holds the chunk's first word; words
+    // before rbeg or from rend on are not the chunk's (past its end it reads zeros).
+    const unsigned long long total = offsets[nchunks];
+    const uint32_t off = live ? offsets[chunk] : 0u;
+    const uint32_t rbeg = (uint32_t)((reinterpret_cast<uintptr_t>(words + off) >> 2) & 3u);
+    const uint32_t rend = live ? rbeg + (offsets[chunk + 1] - off) : 0u;
+    const uint32_t *block0 = words + off - rbeg;  // 16-byte aligned; may lie before `words`
+    const long long first_ok = -(long long)off + rbeg, last_ok = (long long)(total - off) + rbeg;  // words of the stream
+    uint32_t fetched = 0, rd = rbeg;
+    auto fetch = [&]() {  // the next block, if the chunk has it and the ring has room
+        if (fetched < rend && fetched - rd + 4 <= (uint32_t)DEC_RING) {
+            uint32_t *slot = ring + (fetched & (DEC_RING - 1));
+            if ((long long)fetched >= first_ok && (long long)fetched + 4 <= last_ok) {
+                cp_async16(slot, block0 + fetched);
+            } else {  // a block that reaches out of the stream
+                for (int i = 0; i < 4; ++i) {
+                    const long long q = (long long)fetched + i;
+                    slot[i] = q >= first_ok && q < last_ok ? __ldg(block0 + q) : 0u;
+                }
+            }
+            fetched += 4;
+        }
+        cp_async_commit();
+    };
+    auto take = [&]() {  // the next word
+        const uint32_t v = ring[rd & (DEC_RING - 1)];
+        const uint32_t r = rd < rend ? v : 0u;
+        ++rd;
+        return r;
+    };
+    for (int b = 0; b < DEC_RING / 4; ++b) fetch();
+    cp_async_wait_all();
+    // the next 64 bits and more: bit o of w0 is the next one
+    uint32_t w0 = take(), w1 = take(), o = 0;
+    int left = live ? (int)min((unsigned long long)HCHUNK, n - chunk * HCHUNK) : 0;  // codes not yet stored
+    uint16_t *dst = codes + chunk * HCHUNK;
+    int have = 0;         // codes in the buffer
+    const uint32_t rr = (uint32_t)R | ((uint32_t)R << 16);
+    while (!__all_sync(0xffffffffu, left == 0)) {
+        fetch();
+        cp_async_wait_pending<2>();  // what was asked for two rounds ago is there: 5 words or more
+#pragma unroll
+        for (int it = 0; it < DEC_STEPS; ++it) {
+            const uint32_t top = __funnelshift_l(w1, w0, o);
+            const uint2 e = lut[top >> (32 - LUT_BITS)];
+            uint16_t *row = reinterpret_cast<uint16_t *>(buf) + have;
+            uint32_t len = (e.y >> 8) & 0xfu, k = e.y >> 12;
+            // bytes to signed halves, plus R; symbols past the entry's number are overwritten next
+            const uint32_t s01 = __vadd2(prmt(e.x, 0x9180), rr), s23 = __vadd2(prmt(e.x, 0xb3a2), rr);
+            const uint32_t s4 = prmt(e.y, 0x9180) + (uint32_t)R;
+            row[0] = (uint16_t)s01;
+            row[1] = (uint16_t)(s01 >> 16);
+            row[2] = (uint16_t)s23;
+            row[3] = (uint16_t)(s23 >> 16);
+            row[4] = (uint16_t)s4;
+            if (k == 0) {
+                uint32_t sym = e.x;
+                if (len == 0) {  // longer than the window: the canonical rule, length by length
+#pragma unroll 1
+                    for (int i = 0; i < lc.n; ++i) {
+                        const uint4 L = lc.l[i];
+                        const uint32_t c = top >> L.x;
+                        if (c >= L.y && c - L.y < L.z) {
+                            sym = sym_tab[L.w + (c - L.y)];
+                            len = 32u - L.x;
+                            break;
+                        }
                     }
                 }
-                if (!len) {  // not a codeword: corrupt stream; the thread stays for its warp's stores
+                if (len) {
+                    row[0] = (uint16_t)sym;
+                    k = 1;
+                } else if (have < left) {  // not a codeword: corrupt stream, the thread stops here
                     atomicOr(bad, 1u);
-                    ok = false;
-                    break;
-                }
-                row[j++] = (uint16_t)sym;
-            }
-            win <<= len;
-            avail -= (int)len;
-            if (avail <= 32) {  // refill the low 32 bits
-                win |= (unsigned long long)ahead << (32 - avail);
-                avail += 32;
-                ahead = next < nw ? w[next] : 0u;
-                ++next;
-            }
-        }
-        __syncwarp();
-        // the warp stores its 32 rows of this round, two rows (2 x DEC_ROUND codes) per instruction
-        static_assert(DEC_ROUND == 32, "two staged rows per warp store");
-        if (fast_store) {  // 32 whole chunks, 4-byte aligned codes: no checks, running pointers
-            uint32_t *dst = store_base + (j0 >> 1);
-            const uint32_t *src = wrows + (lane >> 4) * RW + (lane & 15);
-#pragma unroll 4
-            for (int r = 0; r < 32; r += 2) dst[(size_t)r * (HCHUNK / 2)] = src[r * RW];
-        } else {
-            for (int r = 0; r < 32; r += 2) {
-                const int rr = r + (lane >> 4), e = 2 * (lane & 15);
-                const unsigned long long c = chunk0 + rr;
-                if (c >= nchunks) break;
-                const long long m = min((long long)DEC_ROUND,
-                                        (long long)min((unsigned long long)HCHUNK, n - c * HCHUNK) - j0);  // codes to store
-                if (m <= 0) continue;
-                uint16_t *dst = codes + c * HCHUNK + j0;
-                const uint32_t v = wrows[rr * RW + (lane & 15)];
-                if (vec && e + 1 < m) {
-                    *reinterpret_cast<uint32_t *>(dst + e) = v;
-                } else {
-                    if (e < m) dst[e] = (uint16_t)(v & 0xffffu);
-                    if (e + 1 < m) dst[e + 1] = (uint16_t)(v >> 16);
+                    left = 0;
                 }
             }
+            have += (int)k;
+            o += len;
+            if (o >= 32) {
+                o -= 32;
+                w0 = w1;
+                w1 = take();
+            }
         }
-        __syncwarp();
+        // store the full groups, keep the rest at the buffer's start
+        int done = 0;
+        while (have - done >= DEC_GROUP && left >= DEC_GROUP) {
+            store_group<VEC>(dst, buf + 2 * done);
+            dst += DEC_GROUP;
+            left -= DEC_GROUP;
+            done += DEC_GROUP;
+        }
+        if (left < DEC_GROUP && have - done >= left) {  // the chunk's last codes
+            const uint16_t *src = reinterpret_cast<const uint16_t *>(buf) + done;
+            for (int i = 0; i < left; ++i) dst[i] = src[i];
+            left = 0;
+        }
+        if (left == 0) {
+            have = 0;
+        } else if (done) {
+            const uint4 a = *reinterpret_cast<const uint4 *>(buf + 2 * done), b = *reinterpret_cast<const uint4 *>(buf + 2 * done + 16);
+            reinterpret_cast<uint4 *>(buf)[0] = a;
+            reinterpret_cast<uint4 *>(buf)[1] = b;
+            have -= done;
+        }
     }
 }
 
@@ -496,10 +583,7 @@ unsigned long long huffman_capacity_words(unsigned long long n, int max_len)
     return huffman_chunks(n) * (unsigned long long)((HCHUNK * max_len + 31) / 32);
 }
 
-size_t huffman_decode_workspace(int nsym)
-{
-    return ((sizeof(DecodeTables) + 15) / 16) * 16 + sizeof(uint16_t) * (size_t)nsym + 16;
-}
+size_t huffman_decode_workspace(int nsym) { return TABLES_BYTES + sizeof(uint16_t) * (size_t)nsym + 16; }
 
 int huffman_max_len() { return MAX_LEN; }
 
@@ -581,52 +665,62 @@ bool huffman_codebook(const uint32_t *hist, int nsym, int max_len, uint8_t *leng
     return true;
 }
 
+// A status word (8 bytes) per tile of 16 chunks; the size is stated as 4 bytes per 8
+// chunks, rounded up to 256 bytes, which always holds them.
 size_t huffman_encode_workspace(unsigned long long n)
 {
-    const unsigned long long blocks = (huffman_chunks(n) + ENC_WARPS - 1) / ENC_WARPS;
+    const unsigned long long blocks = (huffman_chunks(n) + 7) / 8;
     return ((4 * blocks + 255) / 256) * 256;
 }
+static_assert(ENC_WARPS == 16, "status words fit huffman_encode_workspace");
 
+template <bool SMEM_TAB>
+static cudaError_t launch_encode(const uint16_t *codes, unsigned long long n, const uint8_t *lengths,
+                                 const uint32_t *codewords, int nsym, uint32_t *offsets, uint32_t *words,
+                                 unsigned long long capacity_words, unsigned char *ws, cudaStream_t s)
+{
+    const unsigned long long nch = huffman_chunks(n), tiles = (nch + ENC_WARPS - 1) / ENC_WARPS;
+    const size_t smem = sizeof(uint32_t) * (ENC_WARPS * MAX_WORDS + (SMEM_TAB ? (size_t)nsym : 0));
+    cudaError_t e = cudaFuncSetAttribute(k_huff_encode<SMEM_TAB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // flag and tile counter (the first 256 bytes) and the status words start at zero
+    if (e == cudaSuccess) e = cudaMemsetAsync(ws, 0, 256 + 8 * tiles, s);
+    if (e != cudaSuccess) return e;
+    const bool vec = (reinterpret_cast<uintptr_t>(codes) & 15u) == 0;
+    const unsigned long long wave = 2ull * sm_count();
+    k_huff_encode<SMEM_TAB><<<(unsigned)std::min(tiles, wave), ENC_THREADS, smem, s>>>(
+        codes, n, lengths, codewords, nsym, vec, reinterpret_cast<unsigned long long *>(ws + 256),
+        reinterpret_cast<unsigned int *>(ws + 128), (uint32_t)tiles, offsets, words, (uint32_t)nch, capacity_words,
+        reinterpret_cast<unsigned int *>(ws));
+    return cudaGetLastError();
+}
+
+// ws: the call's workspace (its first word is the flag).
 cudaError_t launch_huffman_encode(const uint16_t *codes, unsigned long long n, const uint8_t *lengths,
                                   const uint32_t *codewords, int nsym, uint32_t *offsets, uint32_t *words,
-                                  unsigned long long capacity_words, uint32_t *block_words, unsigned int *bad,
-                                  cudaStream_t s)
+                                  unsigned long long capacity_words, void *ws, cudaStream_t s)
 {
-    cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(unsigned int), s);
-    if (e != cudaSuccess) return e;
-    const unsigned long long nch = huffman_chunks(n);
-    if (nch == 0) return cudaMemsetAsync(offsets, 0, sizeof(uint32_t), s);
-    const unsigned long long blocks = (nch + ENC_WARPS - 1) / ENC_WARPS;
-    const bool vec = (reinterpret_cast<uintptr_t>(codes) & 15u) == 0;
-    // the codebook sits in shared memory up to 16384 symbols (80 KB), beyond that it is
-    // read through the cache
-    const bool smem_tab = nsym <= 16384;
-    const size_t tab = 5 * (size_t)nsym;  // codewords + lengths
-    if (smem_tab) {
-        if (tab > 40 * 1024) {
-            e = cudaFuncSetAttribute(k_huff_sizes<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, nsym);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_huff_write<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tab);
-            if (e != cudaSuccess) return e;
-        }
-        k_huff_sizes<true><<<(unsigned)blocks, ENC_THREADS, nsym, s>>>(codes, n, lengths, nsym, vec, block_words,
-                                                                       nch);
-    } else {
-        k_huff_sizes<false><<<(unsigned)blocks, ENC_THREADS, 0, s>>>(codes, n, lengths, nsym, vec, block_words, nch);
+    unsigned char *w = static_cast<unsigned char *>(ws);
+    if (n == 0) {
+        const cudaError_t e = cudaMemsetAsync(w, 0, sizeof(unsigned int), s);
+        return e == cudaSuccess ? cudaMemsetAsync(offsets, 0, sizeof(uint32_t), s) : e;
     }
-    e = cudaGetLastError();
+    // the codebook sits in shared memory up to 16384 symbols (64 KB), beyond that it is
+    // read through the cache
+    if (nsym <= 16384)
+        return launch_encode<true>(codes, n, lengths, codewords, nsym, offsets, words, capacity_words, w, s);
+    return launch_encode<false>(codes, n, lengths, codewords, nsym, offsets, words, capacity_words, w, s);
+}
+
+template <int VEC>
+static cudaError_t launch_decode(unsigned grid, unsigned threads, size_t smem, cudaStream_t s, const uint32_t *words,
+                                 const uint32_t *offsets, unsigned long long n, const DecodeTables *t,
+                                 const uint16_t *symbols, int nsym, int nsym_smem, uint16_t *codes,
+                                 unsigned long long nch, unsigned int *bad)
+{
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_huff_decode<VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_huff_scan<<<1, SCAN_THREADS, 0, s>>>(block_words, blocks, offsets + nch);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (smem_tab)
-        k_huff_write<true><<<(unsigned)blocks, ENC_THREADS, tab, s>>>(codes, n, lengths, codewords, nsym, vec,
-                                                                      block_words, offsets, words, nch,
-                                                                      capacity_words, bad);
-    else
-        k_huff_write<false><<<(unsigned)blocks, ENC_THREADS, 0, s>>>(codes, n, lengths, codewords, nsym, vec,
-                                                                     block_words, offsets, words, nch,
-                                                                     capacity_words, bad);
+    k_huff_decode<VEC><<<grid, threads, smem, s>>>(words, offsets, n, t, symbols, nsym, nsym_smem, codes, nch, bad);
     return cudaGetLastError();
 }
 
@@ -635,19 +729,24 @@ cudaError_t launch_huffman_decode(const uint32_t *words, const uint32_t *offsets
                                   void *ws, unsigned int *bad, cudaStream_t s)
 {
     DecodeTables *t = static_cast<DecodeTables *>(ws);
-    uint16_t *symbols =
-        reinterpret_cast<uint16_t *>(static_cast<unsigned char *>(ws) + ((sizeof(DecodeTables) + 15) / 16) * 16);
+    uint16_t *symbols = reinterpret_cast<uint16_t *>(static_cast<unsigned char *>(ws) + TABLES_BYTES);
     k_huff_tables<<<1, TAB_THREADS, 0, s>>>(lengths, codewords, nsym, t, symbols, bad);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const unsigned long long nch = huffman_chunks(n);
     if (nch == 0) return cudaSuccess;
-    const bool vec = (reinterpret_cast<uintptr_t>(codes) & 3u) == 0;
+    // few chunks spread over the SMs: at least 128 threads (they share the table's building)
+    const unsigned long long per = (nch + 2ull * sm_count() - 1) / (2ull * sm_count());
+    const unsigned threads = (unsigned)std::min<unsigned long long>(DEC_THREADS, std::max<unsigned long long>(128, (per + 31) / 32 * 32));
+    const unsigned grid = (unsigned)((nch + threads - 1) / threads);
     const int nsym_smem = nsym <= SYM_SMEM ? nsym : 0;
-    const size_t dyn = 2 * (size_t)nsym_smem;
-    k_huff_decode<<<(unsigned)((nch + DEC_THREADS - 1) / DEC_THREADS), DEC_THREADS, dyn, s>>>(
-        words, offsets, n, t, symbols, nsym_smem, codes, nch, vec, bad);
-    return cudaGetLastError();
+    const size_t smem = sizeof(uint2) * (1 << LUT_BITS) + 2 * (size_t)DEC_PITCH * threads + 2 * (size_t)nsym_smem;
+    const uintptr_t a = reinterpret_cast<uintptr_t>(codes);
+    if ((a & 31u) == 0)
+        return launch_decode<32>(grid, threads, smem, s, words, offsets, n, t, symbols, nsym, nsym_smem, codes, nch, bad);
+    if ((a & 15u) == 0)
+        return launch_decode<16>(grid, threads, smem, s, words, offsets, n, t, symbols, nsym, nsym_smem, codes, nch, bad);
+    return launch_decode<2>(grid, threads, smem, s, words, offsets, n, t, symbols, nsym, nsym_smem, codes, nch, bad);
 }
 
 }  // namespace gi
