@@ -209,11 +209,10 @@ inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 
 // Bitmap word gw (ascending index order: row = gw / words_per_row of the (z, y)
 // rows, 32 x-positions each) lives at a tile-major address: rows are grouped by
 // OY along y, and a group's words of one 32-column strip are contiguous per z.
-__device__ __forceinline__ size_t tiled_word(long long gw, int words_per_row, int ny, int nz)
+__device__ __forceinline__ size_t tiled_word(uint32_t gw, uint32_t words_per_row, int ny, int nz)
 {
-    const long long row = gw / words_per_row;
-    const int cx = (int)(gw - row * words_per_row);
-    const int gz = (int)(row / ny), gy = (int)(row - (long long)gz * ny);
+    const uint32_t row = gw / words_per_row, cx = gw - row * words_per_row;
+    const uint32_t gz = row / (uint32_t)ny, gy = row - gz * (uint32_t)ny;
     const size_t col = (size_t)(gy / OY) * words_per_row + cx;
     return (col * nz + gz) * OY + (gy % OY);
 }
@@ -259,7 +258,7 @@ cudaError_t launch_plane_compress(const CompressArgs &a, cudaStream_t s);
 cudaError_t launch_plane_decompress(const DecompressArgs &a, cudaStream_t s);
 cudaError_t launch_row_compress(const CompressArgs &a, cudaStream_t s);
 cudaError_t launch_row_decompress(const DecompressArgs &a, cudaStream_t s);
-// ordered outlier compaction of n fields (one scan launch, one write launch)
+// ordered outlier compaction of n fields (one launch, two with a field of many blocks)
 struct CompactItem {
     const uint32_t *bitmap;
     uint32_t *blockcnt;
