@@ -109,6 +109,15 @@ int code_store_width(const void *codes, int nx)
 
 int cuda_status(cudaError_t e) { return e == cudaSuccess ? INTERP_OK : INTERP_ECUDA; }
 
+// whether a call's kernels leave room for the next one's CTAs (gi::small_call)
+template <typename Item>
+bool small_fields(const Item *items, int n)
+{
+    unsigned long long points = 0;
+    for (int i = 0; i < n; ++i) points += (unsigned long long)items[i].dims[0] * items[i].dims[1] * items[i].dims[2];
+    return gi::small_call(points);
+}
+
 // ---- optional event timing around the tile kernels (measurement only)
 constexpr int kTimingPairs = 512;
 struct TimingLog {
@@ -160,13 +169,13 @@ size_t interp_workspace_bytes(const int64_t dims[3], const interp_config *cfg)
 // The 1-D / 2-D chunk geometries (interp_config.ndim 1 or 2); 0 and 3 are 3-D.
 bool is_nd(int32_t ndim) { return ndim == 1 || ndim == 2; }
 
-cudaError_t launch_nd_compress(int32_t ndim, const gi::CompressArgs &a, cudaStream_t s)
+cudaError_t launch_nd_compress(int32_t ndim, const gi::CompressArgs &a, bool early, cudaStream_t s)
 {
-    return ndim == 1 ? gi::launch_row_compress(a, s) : gi::launch_plane_compress(a, s);
+    return ndim == 1 ? gi::launch_row_compress(a, early, s) : gi::launch_plane_compress(a, early, s);
 }
-cudaError_t launch_nd_decompress(int32_t ndim, const gi::DecompressArgs &a, cudaStream_t s)
+cudaError_t launch_nd_decompress(int32_t ndim, const gi::DecompressArgs &a, bool early, cudaStream_t s)
 {
-    return ndim == 1 ? gi::launch_row_decompress(a, s) : gi::launch_plane_decompress(a, s);
+    return ndim == 1 ? gi::launch_row_decompress(a, early, s) : gi::launch_plane_decompress(a, early, s);
 }
 
 gi::PrologueItem prologue_item(const interp_compress_item &it, const WsLayout &L)
@@ -204,20 +213,21 @@ int compress_nd(const interp_compress_item &it, interp_stream_t stream)
     unsigned char *ws = static_cast<unsigned char *>(it.d_ws);
     uint32_t *bitmap = reinterpret_cast<uint32_t *>(ws + L.bitmap);
     uint32_t *blockcnt = reinterpret_cast<uint32_t *>(ws + L.blockcnt);
+    const bool early = small_fields(&it, 1);
     const gi::PrologueItem pro = prologue_item(it, L);
     cudaError_t e = gi::launch_prologue(&pro, 1, s);
     const gi::CompressArgs args{it.d_x, d, it.d_anchors, it.d_codes, bitmap, blockcnt, it.d_hist, c.radius,
                                 it.d_hdr, false, false, 1};
     if (e == cudaSuccess) {
         timing_mark(0, 0, s);
-        e = launch_nd_compress(c.ndim, args, s);
+        e = launch_nd_compress(c.ndim, args, early, s);
         timing_mark(0, 1, s);
     }
     if (e == cudaSuccess) {
         // row-major bitmap; the tile kernels leave bin R to the scan
         const gi::CompactItem ci{bitmap, blockcnt, L.words, d, it.d_x, it.d_out_idx, it.d_out_val,
                                  it.out_capacity, it.d_hdr, true, it.d_hist, c.radius};
-        e = gi::launch_outlier_compaction(&ci, 1, s);
+        e = gi::launch_outlier_compaction(&ci, 1, early, s);
     }
     return cuda_status(e);
 }
@@ -264,13 +274,14 @@ int interp_compress_batched_scheduled(const interp_compress_item *items, int n, 
                                  it.d_hdr, gi::aligned16(it.d_codes) && d.nx % 8 == 0, c.domain_x == 32,
                                  code_store_width(it.d_codes, d.nx)};
     }
+    const bool early = small_fields(items, n);
     cudaError_t e = gi::launch_prologue(pro, n, s);
     if (e == cudaSuccess) {
         timing_mark(0, 0, s);
         const gi::TileSchedule ts{sched ? sched->run : 0, sched ? sched->ctas_per_sm : 0};
-        if (n3 > 0) e = gi::launch_compress_tiles(args3, n3, s, &ts);  // one persistent launch for every 3-D field
+        if (n3 > 0) e = gi::launch_compress_tiles(args3, n3, early, s, &ts);  // one persistent launch for every 3-D field
         for (int i = 0; i < n && e == cudaSuccess; ++i)                // one launch per 1-D / 2-D field
-            if (is_nd(items[i].cfg.ndim)) e = launch_nd_compress(items[i].cfg.ndim, args[i], s);
+            if (is_nd(items[i].cfg.ndim)) e = launch_nd_compress(items[i].cfg.ndim, args[i], early, s);
         timing_mark(0, 1, s);
     }
     if (e == cudaSuccess) {
@@ -284,7 +295,7 @@ int interp_compress_batched_scheduled(const interp_compress_item *items, int n, 
                                     it.d_out_idx, it.d_out_val, it.out_capacity, it.d_hdr, nd,
                                     it.d_hist, it.cfg.radius};
         }
-        e = gi::launch_outlier_compaction(ci, n, s);
+        e = gi::launch_outlier_compaction(ci, n, early, s);
     }
     return cuda_status(e);
 }
@@ -345,15 +356,16 @@ int interp_decompress_batched_scheduled(const interp_decompress_item *items, int
                                                        gi::aligned16(it.d_xrec) && d.nx % 4 == 0, it.d_out_idx,
                                                        it.out_capacity};
     }
+    const bool early = small_fields(items, n);
     // every field's stored outlier values in one launch, then one tile launch for the 3-D
     // fields and one per 1-D / 2-D field
     cudaError_t e = nsc > 0 ? gi::launch_outlier_scatter(sc, nsc, s) : cudaSuccess;
     if (e == cudaSuccess) {
         timing_mark(1, 0, s);
         const gi::TileSchedule ts{sched ? sched->run : 0, sched ? sched->ctas_per_sm : 0};
-        if (n3 > 0) e = gi::launch_decompress_tiles(args3, n3, s, &ts);
+        if (n3 > 0) e = gi::launch_decompress_tiles(args3, n3, early, s, &ts);
         for (int i = 0; i < n && e == cudaSuccess; ++i)
-            if (is_nd(items[i].ndim)) e = launch_nd_decompress(items[i].ndim, args[i], s);
+            if (is_nd(items[i].ndim)) e = launch_nd_decompress(items[i].ndim, args[i], early, s);
         timing_mark(1, 1, s);
     }
     return cuda_status(e);
@@ -395,10 +407,11 @@ int interp_decompress_nd(int32_t ndim, const int64_t dims[3], const interp_heade
         const gi::ScatterItem sc{d_hdr, d_out_idx, d_out_val, out_capacity, d_xrec};
         e = gi::launch_outlier_scatter(&sc, 1, s);
     }
+    const bool early = gi::small_call((unsigned long long)dims[0] * dims[1] * dims[2]);
     const gi::DecompressArgs args{d, d_anchors, d_codes, d_xrec, d_hdr, false};
     if (e == cudaSuccess) {
         timing_mark(1, 0, s);
-        e = launch_nd_decompress(ndim, args, s);
+        e = launch_nd_decompress(ndim, args, early, s);
         timing_mark(1, 1, s);
     }
     return cuda_status(e);

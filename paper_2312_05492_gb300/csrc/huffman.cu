@@ -283,6 +283,7 @@ __global__ void __launch_bounds__(TAB_THREADS) k_huff_tables(const uint8_t *__re
                                                              const uint32_t *__restrict__ codewords, int nsym,
                                                              DecodeTables *t, uint16_t *symbols, unsigned int *bad)
 {
+    wait_for_previous();
     constexpr int NL = MAX_LEN + 2, NW = TAB_THREADS / 32;
     __shared__ uint32_t cnt_s[NL], base_s[NL], run_s[NL];
     __shared__ uint32_t wcnt[NW][NL];  // per warp: symbols of each length, then their offset in the length's run
@@ -400,6 +401,7 @@ __global__ void __launch_bounds__(DEC_THREADS, 2) k_huff_decode(const uint32_t *
                                                                int nsym_smem, uint16_t *codes,
                                                                unsigned long long nchunks, unsigned int *bad)
 {
+    wait_for_previous();
     __shared__ DecodeTables t;
     __shared__ LongCodes lc;
     extern __shared__ __align__(16) unsigned char dec_sm[];
@@ -720,8 +722,9 @@ static cudaError_t launch_decode(unsigned grid, unsigned threads, size_t smem, c
     const cudaError_t e =
         cudaFuncSetAttribute(k_huff_decode<VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_huff_decode<VEC><<<grid, threads, smem, s>>>(words, offsets, n, t, symbols, nsym, nsym_smem, codes, nch, bad);
-    return cudaGetLastError();
+    // the tables kernel is one CTA
+    return launch_after(true, k_huff_decode<VEC>, grid, threads, smem, s, words, offsets, n, t, symbols, nsym, nsym_smem,
+                        codes, nch, bad);
 }
 
 cudaError_t launch_huffman_decode(const uint32_t *words, const uint32_t *offsets, unsigned long long n,

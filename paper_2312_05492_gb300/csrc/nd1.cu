@@ -268,6 +268,7 @@ template <int MODE>
 __global__ void __launch_bounds__(32 * RC.warps, RC.ctas) k_row_compress(const CompressArgs a, uint32_t per_row,
                                                                    uint32_t segs)
 {
+    wait_for_previous();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nx = a.dims.nx, bins = 2 * a.radius;
     constexpr bool smem_hist = MODE == ENCODE;
@@ -398,6 +399,7 @@ __device__ __forceinline__ void land_codes(uint16_t *land, const uint16_t *codes
 __global__ void __launch_bounds__(32 * RD.warps, RD.ctas) k_row_decompress(const DecompressArgs a, uint32_t per_row,
                                                                      uint32_t segs)
 {
+    wait_for_previous();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nx = a.dims.nx;
     row_levels(a.hdr);
@@ -499,7 +501,7 @@ __global__ void __launch_bounds__(32 * RD.warps, RD.ctas) k_row_decompress(const
 uint32_t segments_per_row(Dims d) { return (uint32_t)(((long long)d.nx + SEG - 1) / SEG); }
 
 template <typename K, typename A>
-cudaError_t launch_rows(K kernel, Shape shape, const A &a, size_t smem, cudaStream_t s)
+cudaError_t launch_rows(K kernel, Shape shape, const A &a, size_t smem, bool early, cudaStream_t s)
 {
     // segments are fewer than 2^32 (N is), and a grid of one wave takes them in turn
     const uint32_t per_row = segments_per_row(a.dims);
@@ -507,21 +509,21 @@ cudaError_t launch_rows(K kernel, Shape shape, const A &a, size_t smem, cudaStre
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const unsigned long long wave = (unsigned long long)sm_count() * shape.ctas;
-    kernel<<<(unsigned)(segs < wave ? segs : wave), 32 * shape.warps, smem, s>>>(a, per_row, (uint32_t)segs);
-    return cudaGetLastError();
+    return launch_after(early, kernel, (unsigned)(segs < wave ? segs : wave), 32 * shape.warps, smem, s, a, per_row,
+                        (uint32_t)segs);
 }
 
 }  // namespace
 
-cudaError_t launch_row_compress(const CompressArgs &a, cudaStream_t s)
+cudaError_t launch_row_compress(const CompressArgs &a, bool early, cudaStream_t s)
 {
-    if (2 * a.radius > R_HIST_BINS) return launch_rows(k_row_compress<ENCODE_GBINS>, RC, a, R_HIST, s);
-    return launch_rows(k_row_compress<ENCODE>, RC, a, R_HIST + sizeof(uint32_t) * 2 * (size_t)a.radius, s);
+    if (2 * a.radius > R_HIST_BINS) return launch_rows(k_row_compress<ENCODE_GBINS>, RC, a, R_HIST, early, s);
+    return launch_rows(k_row_compress<ENCODE>, RC, a, R_HIST + sizeof(uint32_t) * 2 * (size_t)a.radius, early, s);
 }
 
-cudaError_t launch_row_decompress(const DecompressArgs &a, cudaStream_t s)
+cudaError_t launch_row_decompress(const DecompressArgs &a, bool early, cudaStream_t s)
 {
-    return launch_rows(k_row_decompress, RD, a, R_WARPS + R_WARP * RD.warps, s);
+    return launch_rows(k_row_decompress, RD, a, R_WARPS + R_WARP * RD.warps, early, s);
 }
 
 }  // namespace gi

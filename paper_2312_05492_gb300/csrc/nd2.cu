@@ -422,6 +422,7 @@ __device__ __forceinline__ void set_rows_codes(Patch &P, uint32_t R)
 template <int MODE>
 __global__ void __launch_bounds__(P_THREADS, P_CTAS) k_plane_compress(const CompressArgs a, const Plan plan)
 {
+    wait_for_previous();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const Dims d = a.dims;
     const int bins = 2 * a.radius;
@@ -600,6 +601,7 @@ __device__ __forceinline__ uint32_t land_codes(unsigned char *land, const uint16
 
 __global__ void __launch_bounds__(P_THREADS, P_CTAS) k_plane_decompress(const DecompressArgs a, const Plan plan)
 {
+    wait_for_previous();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const Dims d = a.dims;
     plane_levels(a.hdr);
@@ -789,27 +791,26 @@ Plan plan_of(Dims d, unsigned long long warps)
 }
 
 template <typename K, typename Args>
-cudaError_t launch_planes(K kernel, const Args &a, size_t smem, cudaStream_t s)
+cudaError_t launch_planes(K kernel, const Args &a, size_t smem, bool early, cudaStream_t s)
 {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const uint32_t wave = (uint32_t)(sm_count() * P_CTAS);
     const Plan p = plan_of(a.dims, (unsigned long long)wave * PW);
-    kernel<<<p.items < wave ? p.items : wave, P_THREADS, smem, s>>>(a, p);
-    return cudaGetLastError();
+    return launch_after(early, kernel, p.items < wave ? p.items : wave, P_THREADS, smem, s, a, p);
 }
 
 }  // namespace
 
-cudaError_t launch_plane_compress(const CompressArgs &a, cudaStream_t s)
+cudaError_t launch_plane_compress(const CompressArgs &a, bool early, cudaStream_t s)
 {
-    if (2 * a.radius > P_HIST_BINS) return launch_planes(k_plane_compress<ENCODE_GBINS>, a, P_HIST, s);
-    return launch_planes(k_plane_compress<ENCODE>, a, P_HIST + sizeof(uint32_t) * 2 * (size_t)a.radius, s);
+    if (2 * a.radius > P_HIST_BINS) return launch_planes(k_plane_compress<ENCODE_GBINS>, a, P_HIST, early, s);
+    return launch_planes(k_plane_compress<ENCODE>, a, P_HIST + sizeof(uint32_t) * 2 * (size_t)a.radius, early, s);
 }
 
-cudaError_t launch_plane_decompress(const DecompressArgs &a, cudaStream_t s)
+cudaError_t launch_plane_decompress(const DecompressArgs &a, bool early, cudaStream_t s)
 {
-    return launch_planes(k_plane_decompress, a, P_HIST, s);
+    return launch_planes(k_plane_decompress, a, P_HIST, early, s);
 }
 
 }  // namespace gi

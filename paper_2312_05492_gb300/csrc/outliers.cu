@@ -182,12 +182,14 @@ struct CompactBatch {
 
 __global__ void __launch_bounds__(SCAN_THREADS) k_outlier_scan(const __grid_constant__ CompactBatch B)
 {
+    wait_for_previous();
     const CompactField &F = B.f[blockIdx.x];
     if (F.scanned) outlier_scan_block(F.blockcnt, F.nblk, F.hdr, F.capacity, F.hist, F.radius, F.n);
 }
 
 __global__ void __launch_bounds__(WRITE_THREADS) k_outlier_write(const __grid_constant__ CompactBatch B)
 {
+    wait_for_previous();
     int fi = 0;
     while (fi + 1 < B.n && B.f[fi + 1].b0 <= (int)blockIdx.x) ++fi;
     const CompactField &F = B.f[fi];
@@ -240,6 +242,7 @@ struct ScatterBatch {
 
 __global__ void k_outlier_scatter(const __grid_constant__ ScatterBatch B)
 {
+    wait_for_previous();
     const ScatterField &F = B.f[blockIdx.x / B.blocks];
     const unsigned long long b = blockIdx.x % B.blocks;
     unsigned long long n = F.hdr->n_outliers;
@@ -319,7 +322,7 @@ __global__ void __launch_bounds__(HIST_THREADS) k_histogram(const uint16_t *__re
 
 }  // namespace
 
-cudaError_t launch_outlier_compaction(const CompactItem *items, int n, cudaStream_t s)
+cudaError_t launch_outlier_compaction(const CompactItem *items, int n, bool early, cudaStream_t s)
 {
     if (n < 1 || n > kMaxBatch) return cudaErrorInvalidValue;
     CompactBatch B;
@@ -353,12 +356,10 @@ cudaError_t launch_outlier_compaction(const CompactItem *items, int n, cudaStrea
     }
     B.n = n;
     if (scan) {
-        k_outlier_scan<<<n, SCAN_THREADS, 0, s>>>(B);
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launch_after(false, k_outlier_scan, n, SCAN_THREADS, 0, s, B);
         if (e != cudaSuccess) return e;
     }
-    k_outlier_write<<<blocks, WRITE_THREADS, 0, s>>>(B);
-    return cudaGetLastError();
+    return launch_after(early, k_outlier_write, blocks, WRITE_THREADS, 0, s, B);
 }
 
 cudaError_t launch_outlier_scatter(const ScatterItem *items, int n, cudaStream_t s)
@@ -369,7 +370,10 @@ cudaError_t launch_outlier_scatter(const ScatterItem *items, int n, cudaStream_t
     for (int i = 0; i < n; ++i) B.f[i] = ScatterField{items[i].hdr, items[i].idx, items[i].val,
                                                       (unsigned long long)items[i].capacity, items[i].xrec};
     B.n = n;
-    B.blocks = std::max(1, 8 * sm_count() / n);  // a full SM of threads: the stores are scattered
+    // a full SM of threads (the stores are scattered), but no more than the lists may need
+    uint64_t most = 1;
+    for (int i = 0; i < n; ++i) most = std::max<uint64_t>(most, items[i].capacity);
+    B.blocks = (int)std::min<uint64_t>(std::max(1, 8 * sm_count() / n), (most + 1023) / 1024);
     k_outlier_scatter<<<B.blocks * n, 256, 0, s>>>(B);
     return cudaGetLastError();
 }

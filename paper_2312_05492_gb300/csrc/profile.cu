@@ -325,6 +325,7 @@ struct PrologueBatch {
 
 __global__ void __launch_bounds__(RANGE_THREADS) k_prologue(const __grid_constant__ PrologueBatch B)
 {
+    wait_for_previous();
     const int b = blockIdx.x;
     int fi = 0;
     while (fi + 1 < B.n && B.f[fi + 1].b0 <= b) ++fi;
@@ -359,6 +360,7 @@ struct ZeroBatch {
 
 __global__ void __launch_bounds__(512) k_zero(const __grid_constant__ ZeroBatch B)
 {
+    wait_for_previous();
     const ZeroField &F = B.f[blockIdx.x];
     for (int i = threadIdx.x; i < F.ctrl_words; i += 512) F.ctrl[i] = 0u;
     for (int i = threadIdx.x; i < F.nblk; i += 512) F.blockcnt[i] = 0u;
@@ -375,6 +377,8 @@ int sm_count()
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return 1;
     return sms;
 }
+
+bool small_call(unsigned long long points) { return points <= 32768ull * (unsigned)sm_count(); }
 
 namespace {
 
@@ -464,8 +468,7 @@ cudaError_t launch_prologue(const PrologueItem *items, int n, cudaStream_t s)
     k_zero<<<n, 512, 0, s>>>(Z);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_prologue<<<blocks, RANGE_THREADS, 0, s>>>(B);
-    return cudaGetLastError();
+    return launch_after(true, k_prologue, blocks, RANGE_THREADS, 0, s, B);  // k_zero is a few CTAs
 }
 
 cudaError_t launch_profile(const float *x, Dims d, interp_header *hdr, int apply_decision, cudaStream_t s, int ndim)

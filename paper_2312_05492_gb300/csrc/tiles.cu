@@ -1056,6 +1056,7 @@ __device__ __forceinline__ void write_slab_general(const CField &F, const CWrite
 template <bool MULTI>
 __global__ void __launch_bounds__(NT, kCompressCtas) k_compress(const __grid_constant__ CBatch B)
 {
+    wait_for_previous();
     unsigned char *smem = g_smem;
     Levels &lv = g_lv;
     __shared__ int abort_flag;
@@ -1247,6 +1248,7 @@ __device__ __forceinline__ void land_outliers(float *box, const uint16_t *land, 
 template <bool MULTI>
 __global__ void __launch_bounds__(NT, kDecompressCtas) k_decompress(const __grid_constant__ DBatch B)
 {
+    wait_for_previous();
     unsigned char *smem = g_smem;
     Levels &lv = g_lv;
     __shared__ int abort_flag;
@@ -1508,7 +1510,7 @@ int scheduled_grid(int grid, const TileSchedule *sched)
     return std::max(grid, 1);
 }
 
-cudaError_t launch_compress_tiles(const CompressArgs *args, int n, cudaStream_t s, const TileSchedule *sched)
+cudaError_t launch_compress_tiles(const CompressArgs *args, int n, bool early, cudaStream_t s, const TileSchedule *sched)
 {
     if (n < 1 || n > kMaxBatch) return cudaErrorInvalidValue;
     int grid = 0;
@@ -1534,11 +1536,11 @@ cudaError_t launch_compress_tiles(const CompressArgs *args, int n, cudaStream_t 
     B.n = n;
     B.items = items;
     if (items < grid) grid = items;
-    kernel<<<grid, NT, kCompressSmem, s>>>(B);
-    return cudaGetLastError();
+    return launch_after(early, kernel, grid, NT, kCompressSmem, s, B);
 }
 
-cudaError_t launch_decompress_tiles(const DecompressArgs *args, int n, cudaStream_t s, const TileSchedule *sched)
+cudaError_t launch_decompress_tiles(const DecompressArgs *args, int n, bool early, cudaStream_t s,
+                                    const TileSchedule *sched)
 {
     if (n < 1 || n > kMaxBatch) return cudaErrorInvalidValue;
     int grid = 0;
@@ -1565,9 +1567,7 @@ cudaError_t launch_decompress_tiles(const DecompressArgs *args, int n, cudaStrea
     B.n = n;
     B.items = items;
     if (items < grid) grid = items;
-    if (n > 1) k_decompress<true><<<grid, NT, kDecompressSmem, s>>>(B);
-    else k_decompress<false><<<grid, NT, kDecompressSmem, s>>>(B);
-    return cudaGetLastError();
+    return launch_after(early, n > 1 ? k_decompress<true> : k_decompress<false>, grid, NT, kDecompressSmem, s, B);
 }
 
 // ------------------------------------------------------------ tensor maps
