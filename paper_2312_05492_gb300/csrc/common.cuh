@@ -21,15 +21,11 @@ namespace gi {
 // chunks, Sec. IV-C), i.e. a (8TZ+1) x (8TY+1) x (8TX+1) box.
 // A CTA marches along z through a column of 2 x 4 chunks of 8^3 points
 // (16 y x 32 x owned points), one slab of 8 planes at a time.
-#ifndef GI_TILE_THREADS
-#define GI_TILE_THREADS 192
-#endif
 #ifndef GI_TILE_ROWS
 #define GI_TILE_ROWS 16
 #endif
 constexpr int OY = GI_TILE_ROWS, OX = 32;  // owned extent of a column
 static_assert(OY % 8 == 0, "columns hold whole chunks");
-constexpr int TILE_THREADS = GI_TILE_THREADS;
 static_assert(OX == 32, "one outlier-bitmap word covers the 32 x-positions of an owned row");
 
 // outlier bitmap: one 32-bit word per 32 x-positions of every (z, y) row

@@ -32,28 +32,38 @@ namespace gi {
 namespace {
 
 // ------------------------------------------------------------ geometry
-constexpr int NT = TILE_THREADS;
-constexpr int NWARP = NT / 32;
+// threads per CTA: with fewer, each warp does more of a pass per fixed cost (dispatch, index
+// set-up, barrier); compression 512^3 382 -> 361 us from 192 to 128 threads, decompression
+// is 2% slower with 128 and 13% with 256
+constexpr int CNT = 128, DNT = 192;
+template <bool COMPRESS>
+constexpr int kThreads = COMPRESS ? CNT : DNT;
 constexpr int EZ = 9, EY = OY + 1, EX = OX + 1;  // slab box extents (z, y, x)
-constexpr int PLANE = EY * EX;                   // 561 floats, odd: conflict-free row walks
-constexpr int BOXF = EZ * PLANE;                 // floats per slab box
+// Floats per box row and plane.  Compression works where the TMA landed the values, so its
+// rows are whole 16-byte groups: an odd number of them, so that a warp's 16-byte reads of
+// rows (x passes) fall in distinct banks.  Nothing lands in decompression's box: odd rows,
+// free of bank conflicts along every axis (512^3 with rows of 36: 260 us, 282 when the passes
+// end along x; with odd rows: 243 and 245).
+constexpr int XP = OX + 4, PLANE = EY * XP;
+constexpr int DP = EX, DPLANE = EY * DP;
 constexpr int CP = OX + 2;                       // u16 pitch of code rows (17 words, odd)
 constexpr int CBOX_PLANE = EY * CP;              // code box (compression staging, decompression input):
 constexpr int CBOX = EZ * CBOX_PLANE;            // every row and column of the slab box
 constexpr int STAGE_PLANE = CBOX_PLANE;
 constexpr int STAGE = CBOX;
-// TMA landing buffers: dense boxes whose rows are a multiple of 16 bytes
-constexpr int XP = 36;                           // floats per landed row (x 0..35)
 constexpr int XPL = 8;                           // landed input planes: 1..8 of a slab (plane 0 is
                                                  // carried, or loaded directly at a run's start)
-constexpr int XLAND = XPL * EY * XP;
 constexpr int KP = 40;                           // codes per landed row (x 0..39)
 constexpr int KLAND = EZ * EY * KP;
 constexpr uint32_t kTmaPolls = 1u << 22;         // bounded wait for one TMA box
 
 __host__ __device__ constexpr int ext_of(int a) { return a == 2 ? EX : (a == 1 ? EY : EZ); }
 __host__ __device__ constexpr int own_of(int a) { return a == 2 ? OX : (a == 1 ? OY : EZ); }
-__host__ __device__ constexpr int bstride(int a) { return a == 2 ? 1 : (a == 1 ? EX : PLANE); }
+template <bool COMPRESS>
+__host__ __device__ constexpr int bstride(int a)
+{
+    return a == 2 ? 1 : (a == 1 ? (COMPRESS ? XP : DP) : (COMPRESS ? PLANE : DPLANE));
+}
 __host__ __device__ constexpr int sstride(int a) { return a == 2 ? 1 : (a == 1 ? CP : STAGE_PLANE); }
 __host__ __device__ constexpr int cstride(int a) { return a == 2 ? 1 : (a == 1 ? CP : CBOX_PLANE); }
 // decompression reads the codes where the TMA landed them: rows of KP codes, planes of EY rows
@@ -72,30 +82,29 @@ __host__ __device__ constexpr uint32_t magic_of(int n)
 // floor(w / n) for 0 <= w < 2^16 and 1 <= n <= 64, given magic_of(n) (0 for n = 1)
 __device__ __forceinline__ int fdiv(int w, uint32_t m) { return m ? (int)__umulhi((uint32_t)w, m) : w; }
 
-// dynamic shared-memory layouts: the TMA landing buffer first (the dynamic
-// shared-memory base is 128-byte aligned), then 16-byte aligned sub-arrays
+// dynamic shared-memory layouts.  Planes 1..8 of the compression box are where the TMA lands
+// the slab (a 128-byte aligned address), plane 0 lies before them: the passes work on the
+// landed values in place.
 __host__ __device__ constexpr size_t al16(size_t v) { return (v + 15) / 16 * 16; }
-// compression: the staged codes reuse the landing buffer (the next slab's load is
-// issued once they are written out)
-constexpr size_t C_LAND = 0;
-constexpr size_t C_STAGE = C_LAND;
-constexpr size_t C_BOX = al16(C_LAND + sizeof(float) * XLAND);
-constexpr size_t C_HIST = al16(C_BOX + sizeof(float) * BOXF);
+__host__ __device__ constexpr size_t al128(size_t v) { return (v + 127) / 128 * 128; }
+constexpr size_t C_LAND = al128(sizeof(float) * PLANE);
+constexpr size_t C_BOX = C_LAND - sizeof(float) * PLANE;
+constexpr size_t C_STAGE = al16(C_BOX + sizeof(float) * EZ * PLANE);
+constexpr size_t C_HIST = al16(C_STAGE + sizeof(uint16_t) * STAGE);
+static_assert(C_BOX % 16 == 0, "box rows 16-byte aligned");
 // histogram bins, then one spare word per lane that takes the updates a point
 // does not count (a predicated update would become a branch per point)
 constexpr int HIST_WORDS = HIST_SMEM_BINS + 32;
 constexpr size_t C_BAR = al16(C_HIST + sizeof(uint32_t) * HIST_WORDS);
 constexpr size_t kCompressSmem = C_BAR + 16;
-static_assert(sizeof(uint16_t) * STAGE <= sizeof(float) * XLAND, "staged codes fit the landing buffer");
 // decompression: one code landing buffer (the next slab's codes land once the
 // current slab's passes are done with theirs), then the value box and its barrier
-__host__ __device__ constexpr size_t al128(size_t v) { return (v + 127) / 128 * 128; }
 constexpr size_t D_LAND = 0;
 constexpr size_t D_BOX = al128(sizeof(uint16_t) * KLAND);
-constexpr size_t D_BAR = al16(D_BOX + sizeof(float) * BOXF);
+constexpr size_t D_BAR = al16(D_BOX + sizeof(float) * EZ * DPLANE);
 constexpr size_t kDecompressSmem = D_BAR + 16;
-// with 16-row columns, 5 compression CTAs fit an SM: dynamic + static (< 512 B) + 1 KB reserved each
-constexpr int kCompressCtas = 5;
+// with 16-row columns, 6 compression CTAs fit an SM: dynamic + static (< 512 B) + 1 KB reserved each
+constexpr int kCompressCtas = 6;
 static_assert(OY != 16 || kCompressCtas * (kCompressSmem + 512 + 1024) <= 228 * 1024, "compression CTAs per SM");
 // the smaller decompression CTA leaves room for six (at 56 registers a thread)
 constexpr int kDecompressCtas = 6;
@@ -121,9 +130,9 @@ struct Slab {
     int g0[3];           // global origin of the slab box (z, y, x)
     int col;             // column index (cy * cols_x + cx)
     bool carried;        // plane 0 carried from the previous slab (not recomputed)
-    int own_lo, own_hi;  // local planes whose outputs this slab writes
+    int own_lo;          // first local plane whose outputs this slab writes
     int lim[3];          // per axis: box positions below lim are owned and inside the field
-                         // (z: planes up to own_hi; y, x: owned rows / columns)
+                         // (z: planes written; y, x: owned rows / columns)
 };
 
 // Per-call constants, one copy in shared memory.
@@ -144,6 +153,15 @@ struct Levels {
     int natural[3];     // per axis: natural cubic (else not-a-knot)
     uint4 k4;           // R, float(R) bits, cbias
     int dense_out;      // decompression: outliers exceed 1/64 of the points
+};
+
+// The slab a CTA works on and the next one, computed by one thread (they are the same
+// for all, and cost every thread divisions and registers across the passes).
+struct SlabState {
+    Slab s;
+    int fi;        // field
+    int item, c, c_first, c_last;
+    bool valid;    // there is such a slab
 };
 
 // Dynamic shared memory of the tile kernels (layouts C_* and D_* above).
@@ -192,19 +210,24 @@ __device__ __forceinline__ void load_levels(Levels &lv, const interp_header *h)
 // planes [8c, 8c+8] except: plane 8c when carried (the previous slab of the
 // run wrote it as its plane 8), and plane 8c+8 when the run ends there and it
 // is not the field's last plane (the next run starts with it).
-__device__ __forceinline__ void slab_setup(Slab &s, const Field &f, int item, int c, int c_first, int c_last)
+__device__ __forceinline__ void slab_planes(Slab &s, const Field &f, int c, int c_last)
 {
-    const int col = item % f.cols;
+    s.own_lo = s.carried ? 1 : 0;
+    const bool field_end = 8 * c + 8 == f.n[0] - 1;
+    const int own_hi = (c != c_last || field_end) ? 8 : 7;
+    s.lim[0] = min(own_hi, f.n[0] - 1 - s.g0[0]) + 1;
+}
+
+// The first slab of a run.
+__device__ __forceinline__ void slab_setup(Slab &s, const Field &f, int col, int c, int c_last)
+{
     const int cx = col % f.cols_x, cy = col / f.cols_x;
     s.g0[0] = 8 * c;
     s.g0[1] = OY * cy;
     s.g0[2] = OX * cx;
     s.col = col;
-    s.carried = c != c_first;
-    s.own_lo = s.carried ? 1 : 0;
-    const bool field_end = 8 * c + 8 == f.n[0] - 1;
-    s.own_hi = (c != c_last || field_end) ? 8 : 7;
-    s.lim[0] = min(s.own_hi, f.n[0] - 1 - s.g0[0]) + 1;
+    s.carried = false;
+    slab_planes(s, f, c, c_last);
     s.lim[1] = min(OY, f.n[1] - s.g0[1]);
     s.lim[2] = min(OX, f.n[2] - s.g0[2]);
 }
@@ -239,7 +262,7 @@ __device__ __forceinline__ void run_pass(float *__restrict__ box, const Sink &sk
     constexpr int U = axis_u(D), V = axis_v(D);
     constexpr int EU = ext_of(U), EV = ext_of(V);
     constexpr int NC = chunks_of(D);
-    constexpr int BD = bstride(D), BU = bstride(U), BV = bstride(V);
+    constexpr int BD = bstride<COMPRESS>(D), BU = bstride<COMPRESS>(U), BV = bstride<COMPRESS>(V);
     constexpr int SD = sstride(D), SU = sstride(U), SV = sstride(V);
     constexpr int KD = lstride(D), KU = lstride(U), KV = lstride(V);
     constexpr int l = S == 1 ? 0 : (S == 2 ? 1 : 2);
@@ -267,7 +290,7 @@ __device__ __forceinline__ void run_pass(float *__restrict__ box, const Sink &sk
     const float Rf = lv.Rf;
     const uint32_t cbias = lv.cbias;
 
-    for (int w = threadIdx.x; w < nseg; w += NT) {
+    for (int w = threadIdx.x; w < nseg; w += kThreads<COMPRESS>) {
         // consecutive threads walk U first, then V, then the chunk along D
         const int q1 = fdiv(w, mU);
         const int iu = w - q1 * nU;
@@ -500,6 +523,32 @@ __device__ __forceinline__ void seg_full(float *L, uint16_t *C, const LevelQ &Lq
                                          const SegOut &so)
 {
     constexpr bool SPLINE = KIND != KIND_LINEAR;
+    if (COMPRESS && BD == 1 && S == 1) {
+        // along x at stride 1 the segment's 8 values are two 16-byte words (and its closing
+        // point one more), read and written back whole; nothing else writes them in this pass
+        const float4 a = *reinterpret_cast<const float4 *>(L), b = *reinterpret_cast<const float4 *>(L + 4);
+        const float k8 = L[8];
+        float4 u = a, v = b;
+        const float p1 = SPLINE ? sp_quad_right(a.x, a.z, b.x) : sp_linear(a.x, a.z);
+        const float p3 = SPLINE ? cubic_of<KIND>(a.x, a.z, b.x, b.z) : sp_linear(a.z, b.x);
+        const float p5 = SPLINE ? cubic_of<KIND>(a.z, b.x, b.z, k8) : sp_linear(b.x, b.z);
+        const float p7 = SPLINE ? sp_quad_left(b.x, b.z, k8) : sp_linear(b.z, k8);
+        const uint32_t c1 = quantize(a.y, p1, Lq, cbias, Rf, u.y), c3 = quantize(a.w, p3, Lq, cbias, Rf, u.w);
+        const uint32_t c5 = quantize(b.y, p5, Lq, cbias, Rf, v.y), c7 = quantize(b.w, p7, Lq, cbias, Rf, v.w);
+        if (so.keep) {
+            *reinterpret_cast<float4 *>(L) = u;
+            *reinterpret_cast<float4 *>(L + 4) = v;
+        }
+        C[1] = (uint16_t)c1;
+        C[3] = (uint16_t)c3;
+        C[5] = (uint16_t)c5;
+        C[7] = (uint16_t)c7;
+        atomicAdd((so.owned && c1 != so.R) ? so.hist + c1 : so.spare, 1u);
+        atomicAdd((so.owned && c3 != so.R) ? so.hist + c3 : so.spare, 1u);
+        atomicAdd((so.owned && c5 != so.R) ? so.hist + c5 : so.spare, 1u);
+        atomicAdd((so.owned && c7 != so.R) ? so.hist + c7 : so.spare, 1u);
+        return;
+    }
     if (!COMPRESS && BD == 1 && KD == 1) {
         // decompression along x: the chunk row's 8 codes are one aligned 16-byte word
         // of the landed codes (rows of 80 bytes), so one load serves the segment
@@ -578,7 +627,7 @@ struct PassK {
 
 // Pass k of the level of stride S for axis order ORD.  Segments are numbered with
 // U (the faster other axis) fastest, then V, then the chunk along D; thread t
-// takes segments t, t + NT, ...  Threads without a segment skip the pass at once.
+// takes segments t, t + threads, ...  Threads without a segment skip the pass at once.
 template <bool COMPRESS, int ORD, bool CARRIED, int S, int K, int KIND>
 __device__ __forceinline__ void fast_pass(const FastCtx &c, const PassK &pk)
 {
@@ -592,7 +641,7 @@ __device__ __forceinline__ void fast_pass(const FastCtx &c, const PassK &pk)
     constexpr int nV = count_on(ext_of(V), stepV) - v0;
     constexpr int NC = chunks_of(D);
     constexpr int NSEG = nU * nV * NC;
-    constexpr int BD = bstride(D), BU = bstride(U), BV = bstride(V);
+    constexpr int BD = bstride<COMPRESS>(D), BU = bstride<COMPRESS>(U), BV = bstride<COMPRESS>(V);
     // codes: compression stages them in the code-box layout, decompression reads them as landed
     constexpr int KD = COMPRESS ? cstride(D) : lstride(D), KU = COMPRESS ? cstride(U) : lstride(U),
                   KV = COMPRESS ? cstride(V) : lstride(V);
@@ -604,7 +653,7 @@ __device__ __forceinline__ void fast_pass(const FastCtx &c, const PassK &pk)
     so.spare = c.hist + HIST_SMEM_BINS + (threadIdx.x & 31);
     so.R = pk.R;
 #pragma unroll 1
-    for (int w = (int)threadIdx.x; w < NSEG; w += NT) {
+    for (int w = (int)threadIdx.x; w < NSEG; w += kThreads<COMPRESS>) {
         const int q1 = w / nU;
         const int iu = w - q1 * nU;
         const int cd = NC == 1 ? 0 : q1 / nV;
@@ -661,7 +710,6 @@ __device__ __forceinline__ void fast_slab(const FastCtx &c, const PassK &pk, boo
     }
 }
 
-// The nine passes of a slab in the default neighbour domain, every order.
 // The nine passes of a slab in the default neighbour domain, every order.
 // rem: last in-field offset per axis from the box origin; lim: Slab::lim.
 template <bool COMPRESS>
@@ -749,49 +797,45 @@ struct BatchView {
     int n, items;
 };
 
-struct Cursor {
-    int item, fi, c, c_first, c_last;
-};
-
-template <bool MULTI, typename FieldT>
-__device__ __forceinline__ bool cursor_start(Cursor &cu, const BatchView<FieldT> &b, int item)
+// The first slab of work item `item` (invalid beyond the last item).
+template <typename FieldT>
+__device__ __forceinline__ void slab_start(SlabState &st, const BatchView<FieldT> &b, int item)
 {
-    cu.item = item;
-    if (item >= b.items) return false;
+    st.item = item;
+    st.valid = item < b.items;
+    if (!st.valid) return;
     int fi = 0;
-    if (MULTI)
-        while (fi + 1 < b.n && b.fld[fi + 1].item0 <= item) ++fi;
-    cu.fi = fi;
+    while (fi + 1 < b.n && b.fld[fi + 1].item0 <= item) ++fi;
+    st.fi = fi;
     const Field &f = b.fld[fi].f;
-    const int run_id = (item - b.fld[fi].item0) / f.cols;
-    cu.c_first = run_id * f.run;
-    cu.c_last = min(cu.c_first + f.run, f.slabs) - 1;
-    cu.c = cu.c_first;
-    return true;
+    const int li = item - b.fld[fi].item0;
+    const int run_id = li / f.cols;
+    st.c_first = run_id * f.run;
+    st.c_last = min(st.c_first + f.run, f.slabs) - 1;
+    st.c = st.c_first;
+    slab_setup(st.s, f, li - run_id * f.cols, st.c, st.c_last);
 }
 
-template <bool MULTI, typename FieldT>
-__device__ __forceinline__ bool cursor_next(Cursor &cu, const BatchView<FieldT> &b)
+// The slab after `st`: the next one of its run, or the first of the CTA's next item.
+template <typename FieldT>
+__device__ __forceinline__ void slab_next(SlabState &nx, const SlabState &st, const BatchView<FieldT> &b)
 {
-    if (cu.c < cu.c_last) {
-        ++cu.c;
-        return true;
+    if (st.c < st.c_last) {
+        nx = st;
+        ++nx.c;
+        nx.s.g0[0] += 8;
+        nx.s.carried = true;
+        slab_planes(nx.s, b.fld[st.fi].f, nx.c, nx.c_last);
+    } else {
+        slab_start(nx, b, st.item + gridDim.x);
     }
-    return cursor_start<MULTI>(cu, b, cu.item + gridDim.x);
 }
 
-template <bool MULTI, typename FieldT>
-__device__ __forceinline__ void slab_of(Slab &s, const Cursor &cu, const BatchView<FieldT> &b)
-{
-    const FieldT &F = b.fld[MULTI ? cu.fi : 0];
-    slab_setup(s, F.f, cu.item - F.item0, cu.c, cu.c_first, cu.c_last);
-}
-
-// Bring the 9 x 17 x XP (or KP) input box of a slab into the landing buffer:
+// Bring the NPL x 17 x XP (or KP) input box of a slab into shared memory:
 // one TMA box (thread 0; out-of-field elements are zero-filled), or, when the
 // field's rows cannot be described by a tensor map, 4-byte cp.async copies
 // of the in-field elements by all threads.
-template <typename T, int P, int NPL, int Z0>
+template <typename T, int P, int NPL, int Z0, int NT>
 __device__ __forceinline__ void issue_land(T *land, const T *__restrict__ src, const CUtensorMap *map, bool use_tma,
                                            uint64_t *bar, const Field &f, const Slab &s)
 {
@@ -810,7 +854,7 @@ __device__ __forceinline__ void issue_land(T *land, const T *__restrict__ src, c
     const int nxc = min(EX, f.n[2] - s.g0[2]);
     const size_t plane = (size_t)f.n[1] * f.n[2];
     const T *src0 = src + ((size_t)(s.g0[0] + Z0) * f.n[1] + s.g0[1]) * f.n[2] + s.g0[2];
-    for (int y = warp; y < nyr; y += NWARP) {
+    for (int y = warp; y < nyr; y += NT / 32) {
         const T *row = src0 + (size_t)y * f.n[2] + lane;
         T *dst = land + y * P + lane;
         if (lane < nxc) {
@@ -890,23 +934,36 @@ __device__ __forceinline__ void flush_hist(const CField &F, uint32_t *hist_s)
     __syncthreads();
     const int bins = min(2 * F.a.radius, HIST_SMEM_BINS);
     if (F.a.hist)
-        for (int i = threadIdx.x; i < bins; i += NT) {
+        for (int i = threadIdx.x; i < bins; i += CNT) {
             const uint32_t h = hist_s[i];
             if (h) atomicAdd(&F.a.hist[i], h);
         }
-    for (int i = threadIdx.x; i < HIST_SMEM_BINS; i += NT) hist_s[i] = 0u;
+    for (int i = threadIdx.x; i < HIST_SMEM_BINS; i += CNT) hist_s[i] = 0u;
     __syncthreads();
+}
+
+// The slab's anchors (planes 0 and 8 as far as the slab owns them), lossless.  They are
+// never modified, so they are stored while the box still holds the input.
+__device__ __forceinline__ void write_anchors(const CField &F, const CWrite &cw, const Slab &sl, const float *box)
+{
+    constexpr int AY = OY / 8, AX = OX / 8;
+    const int t = threadIdx.x;
+    if (t >= 2 * AY * AX) return;
+    const int pz = 8 * (t / (AY * AX)), y = 8 * (t / AX % AY), x = 8 * (t % AX);
+    if (pz < sl.own_lo || pz >= sl.lim[0] || y >= sl.lim[1] || x >= sl.lim[2]) return;
+    const int az = (sl.g0[0] + pz) / 8, ay = (sl.g0[1] + y) / 8, ax = (sl.g0[2] + x) / 8;
+    F.a.anchors[((size_t)az * cw.Ay + ay) * cw.Ax + ax] = box[pz * PLANE + y * XP + x];
 }
 
 // The owned planes of a slab whose rows all lie inside the field, with 16-byte
 // aligned code rows and no outlier: staged codes -> global (8 codes per thread
-// and store, three planes per step), anchors, and all-zero outlier-bitmap words.
-static_assert(NT % 4 == 0 && (NT / 4) % OY == 0, "write-out steps cover whole planes");
+// and store, three planes per step), code R at anchors, and all-zero outlier-bitmap words.
+static_assert(CNT % 4 == 0 && (CNT / 4) % OY == 0, "write-out steps cover whole planes");
 __device__ __forceinline__ void write_slab_fast(const CField &F, const CWrite &cw, const Slab &sl, int rows,
-                                                const uint16_t *stage, const float *box)
+                                                const uint16_t *stage)
 {
     const Field &f = F.f;
-    constexpr int PSTEP = NT / 4 / OY;  // planes per step
+    constexpr int PSTEP = CNT / 4 / OY;  // planes per step
     const int sub = threadIdx.x & 3;
     int r = threadIdx.x >> 2;
     const int y = r % OY;
@@ -915,15 +972,11 @@ __device__ __forceinline__ void write_slab_fast(const CField &F, const CWrite &c
     const uint16_t *sp = stage + pz * STAGE_PLANE + y * CP + 8 * sub;
     uint16_t *gp = F.a.codes + ((size_t)(sl.g0[0] + pz) * f.n[1] + sl.g0[1] + y) * f.n[2] + sl.g0[2] + 8 * sub;
     const bool anchor_row = (y & 7) == 0;
-    for (; r < rows; r += NT / 4, pz += PSTEP, sp += PSTEP * STAGE_PLANE, gp += PSTEP * plane) {
+    for (; r < rows; r += CNT / 4, pz += PSTEP, sp += PSTEP * STAGE_PLANE, gp += PSTEP * plane) {
         const uint32_t *s32 = reinterpret_cast<const uint32_t *>(sp);
         uint32_t w0 = s32[0];
         const uint32_t w1 = s32[1], w2 = s32[2], w3 = s32[3];
-        if (anchor_row && (pz & 7) == 0) {  // anchor at x = 8*sub (Sec. IV-A): lossless, code R
-            w0 = (w0 & 0xffff0000u) | (uint32_t)cw.R;
-            const int gz = sl.g0[0] + pz, gy = sl.g0[1] + y, gx = sl.g0[2] + 8 * sub;
-            F.a.anchors[((size_t)(gz / 8) * cw.Ay + gy / 8) * cw.Ax + gx / 8] = box[pz * PLANE + y * EX + 8 * sub];
-        }
+        if (anchor_row && (pz & 7) == 0) w0 = (w0 & 0xffff0000u) | (uint32_t)cw.R;  // anchor at x = 8*sub
         *reinterpret_cast<uint4 *>(gp) = make_uint4(w0, w1, w2, w3);
     }
     // the slab's bitmap words are contiguous (16 per plane, tile-major layout)
@@ -939,7 +992,6 @@ __device__ __noinline__ void write_slab_rows(const CField &F, const CWrite cw, i
                                              int own_lo, int planes)
 {
     const uint16_t *stage = reinterpret_cast<const uint16_t *>(g_smem + C_STAGE);
-    const float *box = reinterpret_cast<const float *>(g_smem + C_BOX);
     const Field &f = F.f;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const size_t plane = (size_t)f.n[1] * f.n[2];
@@ -954,21 +1006,17 @@ __device__ __noinline__ void write_slab_rows(const CField &F, const CWrite cw, i
     const size_t my_block = block_of(lane < planes ? lane : 0, 0);
     const uint32_t split = __ballot_sync(0xffffffffu, lane < planes && my_block != block_of(lane, ny - 1));
     uint32_t count = 0;
-    for (int y = warp; y < ny; y += NWARP) {
+    for (int y = warp; y < ny; y += (CNT / 32)) {
         const size_t grow = (size_t)(z0 + own_lo) * f.n[1] + y0 + y;
         uint16_t *gp = F.a.codes + grow * f.n[2] + x0 + lane;
         uint32_t *wb = F.a.bitmap + ((size_t)col * f.n[0] + z0 + own_lo) * OY + y;
         const uint16_t *sp = stage + own_lo * STAGE_PLANE + y * CP + lane;
         const bool anchor = in && ((y | lane) & 7) == 0;
-#pragma unroll 2
+#pragma unroll 4
         for (int i = 0; i < planes; ++i, gp += plane, wb += OY, sp += STAGE_PLANE) {
             uint32_t code = *sp;
             const int pz = own_lo + i;
-            if (anchor && (pz & 7) == 0) {  // anchor (Sec. IV-A): lossless, code R
-                code = (uint32_t)cw.R;
-                F.a.anchors[((size_t)((z0 + pz) / 8) * cw.Ay + (y0 + y) / 8) * cw.Ax +
-                            (x0 + lane) / 8] = box[pz * PLANE + y * EX + lane];
-            }
+            if (anchor && (pz & 7) == 0) code = (uint32_t)cw.R;  // anchor (Sec. IV-A)
             if (in) *gp = (uint16_t)code;
             const uint32_t word = __ballot_sync(0xffffffffu, in && code == 0u);
             if (lane == 0) *wb = word;
@@ -987,16 +1035,16 @@ __device__ __noinline__ void write_slab_rows(const CField &F, const CWrite cw, i
     }
 }
 
-// Any other slab with 16-byte aligned code rows: codes, anchors, and the exact
+// Any other slab with 16-byte aligned code rows: codes and the exact
 // outlier-bitmap words with their block counts.  A warp takes 8 consecutive
 // rows of one plane, 4 lanes x 8 codes per row.
 __device__ __forceinline__ void write_slab_general(const CField &F, const CWrite &cw, const Slab &sl, int rows,
-                                                   const uint16_t *stage, const float *box)
+                                                   const uint16_t *stage)
 {
     const Field &f = F.f;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int sub = lane & 3;
-    for (int base = warp * 8; base < rows; base += NWARP * 8) {
+    for (int base = warp * 8; base < rows; base += (CNT / 32) * 8) {
         const int row = base + (lane >> 2);
         const int pz = sl.own_lo + row / OY, y = row % OY;
         const int gz = sl.g0[0] + pz, gy = sl.g0[1] + y;
@@ -1010,10 +1058,7 @@ __device__ __forceinline__ void write_slab_general(const CField &F, const CWrite
             for (int j = 0; j < 4; ++j) w[j] = srow[j];
         }
         const size_t gi = ((size_t)gz * f.n[1] + gy) * f.n[2] + gx;
-        if (nvalid > 0 && ((pz | y) & 7) == 0) {  // anchor at x = 8*sub (Sec. IV-A): lossless, code R
-            w[0] = (w[0] & 0xffff0000u) | (uint32_t)cw.R;
-            F.a.anchors[((size_t)(gz / 8) * cw.Ay + gy / 8) * cw.Ax + gx / 8] = box[pz * PLANE + y * EX + 8 * sub];
-        }
+        if (((pz | y) & 7) == 0) w[0] = (w[0] & 0xffff0000u) | (uint32_t)cw.R;  // anchor at x = 8*sub (Sec. IV-A)
         if (nvalid == 8) {
             *reinterpret_cast<uint4 *>(F.a.codes + gi) = make_uint4(w[0], w[1], w[2], w[3]);
         } else {
@@ -1052,15 +1097,19 @@ __device__ __forceinline__ void write_slab_general(const CField &F, const CWrite
     }
 }
 
-// MULTI = false: a single field (index 0 everywhere, resolved at compile time).
-template <bool MULTI>
-__global__ void __launch_bounds__(NT, kCompressCtas) k_compress(const __grid_constant__ CBatch B)
+// TMA: every field's rows can be described by a tensor map.  Otherwise (copies by all
+// threads for the fields that cannot) one CTA less per SM: the shared memory of six leaves
+// next to no L1 cache, through which those copies go (449x449x235 274 -> 263 us; with TMA
+// the sixth CTA is worth 377 -> 361 us on 512^3).
+template <bool TMA>
+__global__ void __launch_bounds__(CNT, TMA ? kCompressCtas : kCompressCtas - 1) k_compress(const __grid_constant__ CBatch B)
 {
     wait_for_previous();
     unsigned char *smem = g_smem;
     Levels &lv = g_lv;
+    __shared__ SlabState st[3];  // in turn: this slab, the next, the one after it
     __shared__ int abort_flag;
-    float *land = reinterpret_cast<float *>(smem + C_LAND);
+    float *land = reinterpret_cast<float *>(smem + C_LAND);  // planes 1..8 of the box
     float *box = reinterpret_cast<float *>(smem + C_BOX);
     uint16_t *stage = reinterpret_cast<uint16_t *>(smem + C_STAGE);
     uint32_t *hist_s = reinterpret_cast<uint32_t *>(smem + C_HIST);
@@ -1072,95 +1121,81 @@ __global__ void __launch_bounds__(NT, kCompressCtas) k_compress(const __grid_con
         mbar_init(bar, 1);
         fence_barrier_init();
     }
-    for (int i = threadIdx.x; i < HIST_WORDS; i += NT) hist_s[i] = 0u;
+    for (int i = threadIdx.x; i < HIST_WORDS; i += CNT) hist_s[i] = 0u;
     __syncthreads();
 
     uint32_t phase = 0;
-    uint32_t out_seen = 0;  // outliers in the shared histogram before the current slab
-
-    Cursor cu;
-    if (!cursor_start<MULTI>(cu, bv, blockIdx.x)) return;
-    Slab sl;
-    slab_of<MULTI>(sl, cu, bv);
+    int cur = 0;  // st[cur]: this slab
+    if (threadIdx.x == 0) slab_start(st[0], bv, blockIdx.x);
+    __syncthreads();
     int lv_field = -1;
+    uint32_t out_seen = 0;  // outliers in the shared histogram before the current slab
     {
-        const int fi = MULTI ? cu.fi : 0;
-        issue_land<float, XP, XPL, 1>(land, B.fld[fi].a.x, &B.map[fi], B.fld[fi].use_tma, bar, B.fld[fi].f, sl);
+        const CField &F = B.fld[st[0].fi];
+        issue_land<float, XP, XPL, 1, CNT>(land, F.a.x, &B.map[st[0].fi], TMA || F.use_tma, bar, F.f, st[0].s);
     }
     for (;;) {
-        const int fi = MULTI ? cu.fi : 0;
+        const Slab &sl = st[cur].s;
+        const int fi = st[cur].fi;
         const CField &F = B.fld[fi];
         const Field &f = F.f;
-        const Sink sk{stage, nullptr, hist_s, F.a.hist};
-        Cursor nx = cu;
-        const bool has_next = cursor_next<MULTI>(nx, bv);
-        Slab sn = sl;
-        if (has_next) slab_of<MULTI>(sn, nx, bv);
         if (threadIdx.x == 0 && lv_field != fi) load_levels(lv, F.a.hdr);
+        // the next slab (slots in turn by three: a slow thread may still be writing out the
+        // previous slab)
+        const int nxt = cur == 2 ? 0 : cur + 1;
+        if (threadIdx.x == CNT - 1) slab_next(st[nxt], st[cur], bv);
         lv_field = fi;
 
         // ---- input: plane 0 carried, or loaded directly at a run's start; planes 1..8 landed
         if (!sl.carried) {
             const int nyr = min(EY, f.n[1] - sl.g0[1]), nxc = min(EX, f.n[2] - sl.g0[2]);
             const float *src = F.a.x + ((size_t)sl.g0[0] * f.n[1] + sl.g0[1]) * f.n[2] + sl.g0[2];
-            for (int i = threadIdx.x; i < EY * EX; i += NT) {
+            for (int i = threadIdx.x; i < EY * EX; i += CNT) {
                 const int y = i / EX, xx = i - y * EX;
-                if (y < nyr && xx < nxc) box[i] = __ldg(src + (size_t)y * f.n[2] + xx);
+                if (y < nyr && xx < nxc) box[y * XP + xx] = __ldg(src + (size_t)y * f.n[2] + xx);
             }
         }
-        if (!wait_land(F.use_tma, bar, phase)) abort_flag = 1;
-        if (!F.use_tma) __syncthreads();  // cp.async copies of all threads visible
-        for (int i = threadIdx.x; i < XPL * EY * 9; i += NT) {  // 9 groups of 4 floats per row (x 0..35)
-            const int row = i / 9, q = i - 9 * row;
-            const float4 v = *reinterpret_cast<const float4 *>(land + row * XP + 4 * q);
-            float *d = box + (row + EY) * EX + 4 * q;  // landed row r is box row r + EY (plane + 1)
-            d[0] = v.x;
-            if (q < 8) {
-                d[1] = v.y;
-                d[2] = v.z;
-                d[3] = v.w;
-            }
-        }
-        __syncthreads();  // box and levels ready; the landing buffer now stages codes
+        if (!wait_land(TMA || F.use_tma, bar, phase)) abort_flag = 1;
+        __syncthreads();  // box and levels ready; the previous slab's staged codes are written out
         if (abort_flag) break;
-
-        run_slab<true>(box, sk, sl, f, lv);  // ends with a barrier
-
-        // ---- owned planes: codes, anchors, outlier-bitmap words
         const CWrite cw = cwrite_of(F);
-        const int nzp = min(EZ, f.n[0] - sl.g0[0]);
-        const int hi = min(sl.own_hi, nzp - 1);
-        const int rows = (hi - sl.own_lo + 1) * OY;
-        const uint32_t out_now = hist_s[0];  // no code is counted before the next slab's first barrier
+        write_anchors(F, cw, sl, box);
+
+        run_slab<true>(box, Sink{stage, nullptr, hist_s, F.a.hist}, sl, f, lv);  // ends with a barrier
+
+        const uint32_t out_now = hist_s[0];  // no code is counted between here and the next slab's first barrier
         const bool outliers = out_now != out_seen;
         out_seen = out_now;
-        if (!outliers && cw.code_store == 8 && sl.g0[1] + OY <= f.n[1] && sl.g0[2] + OX <= f.n[2])
-            write_slab_fast(F, cw, sl, rows, stage, box);
-        else if (cw.code_store == 8)
-            write_slab_general(F, cw, sl, rows, stage, box);
-        else
-            write_slab_rows(F, cw, sl.g0[0], sl.g0[1], sl.g0[2], sl.col, sl.own_lo, hi - sl.own_lo + 1);
-        // ---- next slab's input into the landing buffer (staged codes written out),
-        // and plane 8 carried into plane 0 when the next slab continues this run
+        const SlabState &nx = st[nxt];
+        const bool has_next = nx.valid;
+        // ---- plane 8 carried into plane 0 when the next slab continues this run; then the
+        // next slab's input, which lands while this slab's codes are written out
+        if (has_next && nx.s.carried)
+            for (int i = threadIdx.x; i < PLANE / 4; i += CNT)
+                reinterpret_cast<float4 *>(box)[i] = reinterpret_cast<const float4 *>(box + 8 * PLANE)[i];
         __syncthreads();
         if (has_next) {
-            const int nfi = MULTI ? nx.fi : 0;
+            const int nfi = nx.fi;
             const CField &N = B.fld[nfi];
-            issue_land<float, XP, XPL, 1>(land, N.a.x, &B.map[nfi], N.use_tma, bar, N.f, sn);
-            if (nx.item == cu.item)
-                for (int i = threadIdx.x; i < PLANE; i += NT) box[i] = box[8 * PLANE + i];
+            issue_land<float, XP, XPL, 1, CNT>(land, N.a.x, &B.map[nfi], TMA || N.use_tma, bar, N.f, nx.s);
         }
-        __syncthreads();  // box free for the next slab
-        if (!has_next || (MULTI && nx.fi != cu.fi)) {  // field done
+        // ---- owned planes: codes and outlier-bitmap words
+        const int planes = sl.lim[0] - sl.own_lo;
+        if (!outliers && cw.code_store == 8 && sl.lim[1] == OY && sl.lim[2] == OX)
+            write_slab_fast(F, cw, sl, planes * OY, stage);
+        else if (cw.code_store == 8)
+            write_slab_general(F, cw, sl, planes * OY, stage);
+        else
+            write_slab_rows(F, cw, sl.g0[0], sl.g0[1], sl.g0[2], sl.col, sl.own_lo, planes);
+        if (!has_next || nx.fi != fi) {  // field done
             flush_hist(F, hist_s);
             out_seen = 0;
         }
         if (!has_next) break;
-        cu = nx;
-        sl = sn;
+        cur = nxt;
     }
     if (abort_flag) {
-        const int fi = MULTI ? cu.fi : 0;
+        const int fi = st[cur].fi;
         if (threadIdx.x == 0) {
             atomicOr(&B.fld[fi].a.hdr->status, INTERP_STATUS_TIMEOUT);
             // the transfer that did not arrive gets a second bounded wait before the
@@ -1204,7 +1239,7 @@ __device__ __forceinline__ void land_outliers(float *box, const uint16_t *land, 
     const int nitem = (EZ - pz0) * EY * 5;  // 5 groups of 8 codes per row (x 0..39)
     // the landed rows are 5 groups each, so the groups of planes pz0.. are one flat run
     const uint4 *l4 = reinterpret_cast<const uint4 *>(land) + pz0 * EY * 5;
-    for (int i = threadIdx.x; i < nitem; i += NT) {
+    for (int i = threadIdx.x; i < nitem; i += DNT) {
         const uint4 v = l4[i];
         if (!(has_zero_half(v.x) | has_zero_half(v.y) | has_zero_half(v.z) | has_zero_half(v.w))) continue;
         const int row = pz0 * EY + i / 5, q = i % 5;
@@ -1215,7 +1250,7 @@ __device__ __forceinline__ void land_outliers(float *box, const uint16_t *land, 
         const int nj = min(8, min(nxc, EX) - 8 * q);  // in-field codes of the group
         if (DENSE) {
             const size_t g = ((size_t)(sl.g0[0] + pz) * f.n[1] + sl.g0[1] + y) * f.n[2] + sl.g0[2] + 8 * q;
-            float *brow = box + row * EX + 8 * q;
+            float *brow = box + row * DP + 8 * q;
             if (F.a.vec_xrec && nj == 8) {
                 const float4 a = __ldg(reinterpret_cast<const float4 *>(F.a.xrec + g));
                 const float4 b = __ldg(reinterpret_cast<const float4 *>(F.a.xrec + g) + 1);
@@ -1232,7 +1267,7 @@ __device__ __forceinline__ void land_outliers(float *box, const uint16_t *land, 
                 if (((wv[j >> 1] >> (16 * (j & 1))) & 0xffffu) == 0u) {
                     const size_t g =
                         ((size_t)(sl.g0[0] + pz) * f.n[1] + sl.g0[1] + y) * f.n[2] + sl.g0[2] + 8 * q + j;
-                    box[row * EX + 8 * q + j] = __ldg(F.a.xrec + g);
+                    box[row * DP + 8 * q + j] = __ldg(F.a.xrec + g);
                 }
             }
         }
@@ -1245,12 +1280,12 @@ __device__ __forceinline__ void land_outliers(float *box, const uint16_t *land, 
 // next slab are fetched into registers before the current slab's passes.  One
 // buffer (rather than two) lets six CTAs share an SM, whose extra warps hide
 // the rest of the latency (measured faster than two buffers at five CTAs).
-template <bool MULTI>
-__global__ void __launch_bounds__(NT, kDecompressCtas) k_decompress(const __grid_constant__ DBatch B)
+__global__ void __launch_bounds__(DNT, kDecompressCtas) k_decompress(const __grid_constant__ DBatch B)
 {
     wait_for_previous();
     unsigned char *smem = g_smem;
     Levels &lv = g_lv;
+    __shared__ SlabState st[3];  // in turn: this slab, the next, the one after it
     __shared__ int abort_flag;
     float *box = reinterpret_cast<float *>(smem + D_BOX);
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + D_BAR);
@@ -1268,7 +1303,7 @@ __global__ void __launch_bounds__(NT, kDecompressCtas) k_decompress(const __grid
     constexpr int AYN = OY / 8 + 1, AXN = OX / 8 + 1;  // anchor rows / columns of the box
     const int ai = threadIdx.x;
     const int a_z = ai / (AYN * AXN), a_y = (ai / AXN) % AYN, a_x = ai % AXN;
-    const int a_off = (8 * a_z) * PLANE + (8 * a_y) * EX + 8 * a_x;
+    const int a_off = (8 * a_z) * DPLANE + (8 * a_y) * DP + 8 * a_x;
     auto anchor_fetch = [&](const DField &F, const Slab &s, float &v) {
         const Field &f = F.f;
         const int pz = 8 * a_z, y = 8 * a_y, x = 8 * a_x;
@@ -1281,19 +1316,18 @@ __global__ void __launch_bounds__(NT, kDecompressCtas) k_decompress(const __grid
         return ok;
     };
 
-    Cursor cu;
-    if (!cursor_start<MULTI>(cu, bv, blockIdx.x)) return;
-    Slab sl;
-    slab_of<MULTI>(sl, cu, bv);
+    int cur = 0;  // st[cur]: this slab
+    if (threadIdx.x == 0) slab_start(st[0], bv, blockIdx.x);
+    __syncthreads();
     // A single field whose outliers are all listed and number at most one per thread:
     // each thread keeps one outlier's coordinates, and a slab runs the outlier scan only
     // when one of them lies in its box (on smooth fields almost none does).
     bool few = false;
     int oz = -1, oy = 0, ox = 0;
-    if (!MULTI) {
+    if (B.n == 1) {
         const DField &F0 = B.fld[0];
         const unsigned long long nout = F0.a.hdr->n_outliers;
-        few = F0.a.out_idx != nullptr && nout <= F0.a.out_capacity && nout <= (unsigned long long)NT;
+        few = F0.a.out_idx != nullptr && nout <= F0.a.out_capacity && nout <= (unsigned long long)DNT;
         if (few && threadIdx.x < nout) {
             const uint32_t g = __ldg(F0.a.out_idx + threadIdx.x);
             const uint32_t plane = (uint32_t)F0.f.n[1] * (uint32_t)F0.f.n[2];
@@ -1307,28 +1341,32 @@ __global__ void __launch_bounds__(NT, kDecompressCtas) k_decompress(const __grid
     float anc = 0.0f;
     bool anc_ok;
     {
-        const int fi = MULTI ? cu.fi : 0;
-        issue_land<uint16_t, KP, EZ, 0>(land, B.fld[fi].a.codes, &B.map[fi], B.fld[fi].use_tma, bar, B.fld[fi].f,
-                                        sl);
-        anc_ok = anchor_fetch(B.fld[fi], sl, anc);
+        const DField &F = B.fld[st[0].fi];
+        issue_land<uint16_t, KP, EZ, 0, DNT>(land, F.a.codes, &B.map[st[0].fi], F.use_tma, bar, F.f, st[0].s);
+        anc_ok = anchor_fetch(F, st[0].s, anc);
+        if (threadIdx.x == DNT - 1) slab_next(st[1], st[0], bv);
+        __syncthreads();
     }
     for (;;) {
-        const int fi = MULTI ? cu.fi : 0;
+        const Slab &sl = st[cur].s;
+        const int nxt = cur == 2 ? 0 : cur + 1;
+        const SlabState &nx = st[nxt];
+        const int fi = st[cur].fi;
         const DField &F = B.fld[fi];
         const Field &f = F.f;
-        Cursor nx = cu;
-        const bool has_next = cursor_next<MULTI>(nx, bv);
-        Slab sn = sl;
-        if (has_next) slab_of<MULTI>(sn, nx, bv);
+        const bool has_next = nx.valid;
         if (threadIdx.x == 0 && lv_field != fi) load_levels(lv, F.a.hdr);
         lv_field = fi;
+
+        // the slab after the next one, read from the next iteration on (its slot held the
+        // slab before this one)
+        if (threadIdx.x == DNT - 1 && has_next) slab_next(st[nxt == 2 ? 0 : nxt + 1], nx, bv);
 
         // ---- this slab's codes
         if (!wait_land(F.use_tma, bar, phase)) abort_flag = 1;
         if (anc_ok) box[a_off] = anc;  // this slab's anchors, fetched a slab ago
         if (has_next) {
-            const int nfi = MULTI ? nx.fi : 0;
-            anc_ok = anchor_fetch(B.fld[nfi], sn, anc);
+            anc_ok = anchor_fetch(B.fld[nx.fi], nx.s, anc);
         }
         const bool mine = oz >= sl.g0[0] && oz < sl.g0[0] + EZ && oy >= sl.g0[1] && oy < sl.g0[1] + EY &&
                           ox >= sl.g0[2] && ox < sl.g0[2] + EX;
@@ -1343,90 +1381,80 @@ __global__ void __launch_bounds__(NT, kDecompressCtas) k_decompress(const __grid
         }
         if (abort_flag) break;
 
-        const Sink sk{nullptr, land, nullptr, nullptr};
-        run_slab<false>(box, sk, sl, f, lv);  // ends with a barrier
+        run_slab<false>(box, Sink{nullptr, land, nullptr, nullptr}, sl, f, lv);  // ends with a barrier
         // ---- the codes are read: the next slab's land during the write-out
         if (has_next) {
-            const int nfi = MULTI ? nx.fi : 0;
+            const int nfi = nx.fi;
             const DField &N = B.fld[nfi];
-            issue_land<uint16_t, KP, EZ, 0>(land, N.a.codes, &B.map[nfi], N.use_tma, bar, N.f, sn);
+            issue_land<uint16_t, KP, EZ, 0, DNT>(land, N.a.codes, &B.map[nfi], N.use_tma, bar, N.f, nx.s);
         }
 
         // ---- write the owned planes
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        const int nzp = min(EZ, f.n[0] - sl.g0[0]);
-        const int hi = min(sl.own_hi, nzp - 1);
-        const int rows = (hi - sl.own_lo + 1) * OY;
-        if (F.a.vec_xrec && sl.g0[1] + OY <= f.n[1] && sl.g0[2] + OX <= f.n[2]) {
-            // whole rows, 16-byte aligned: 8 values per thread, three planes per step
-            constexpr int PSTEP = NT / 4 / OY;
-            const int sub4 = threadIdx.x & 3;
-            int r = threadIdx.x >> 2;
-            const int y = r % OY;
-            const int pz = sl.own_lo + r / OY;
+        const int planes = sl.lim[0] - sl.own_lo, rows = planes * OY;
+        if (F.a.vec_xrec && sl.lim[1] == OY && sl.lim[2] == OX) {
+            // whole rows, 16-byte aligned: 8 lanes x 4 values per row (whole sectors per
+            // store), DNT / 8 rows apart, so that after two steps a thread is back on its row
+            constexpr int RSTEP = DNT / 8, PSTEP = 2 * RSTEP / OY;
+            static_assert(2 * RSTEP % OY == 0, "two write-out steps cover whole planes");
             const size_t plane = (size_t)f.n[1] * f.n[2];
-            const float *sp = box + pz * PLANE + y * EX + 8 * sub4;
-            float *gp = F.a.xrec + ((size_t)(sl.g0[0] + pz) * f.n[1] + sl.g0[1] + y) * f.n[2] + sl.g0[2] + 8 * sub4;
-            for (; r < rows; r += NT / 4, sp += PSTEP * PLANE, gp += PSTEP * plane) {
-                reinterpret_cast<float4 *>(gp)[0] = make_float4(sp[0], sp[1], sp[2], sp[3]);
-                reinterpret_cast<float4 *>(gp)[1] = make_float4(sp[4], sp[5], sp[6], sp[7]);
+            const int x4 = 4 * (threadIdx.x & 7);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                int r = (threadIdx.x >> 3) + h * RSTEP;
+                const int y = r % OY, pz = sl.own_lo + r / OY;
+                const float *sp = box + pz * DPLANE + y * DP + x4;
+                float *gp = F.a.xrec + ((size_t)(sl.g0[0] + pz) * f.n[1] + sl.g0[1] + y) * f.n[2] + sl.g0[2] + x4;
+                for (; r < rows; r += 2 * RSTEP, sp += PSTEP * DPLANE, gp += PSTEP * plane)
+                    *reinterpret_cast<float4 *>(gp) = make_float4(sp[0], sp[1], sp[2], sp[3]);
             }
-        } else if (!F.a.vec_xrec) {
-            // rows that are not 16-byte aligned: a warp stores one row per step, one value per
-            // lane (consecutive addresses)
+        } else if (F.a.vec_xrec) {
+            // 8 lanes x 4 values per row
+            for (int i = threadIdx.x; i < rows * 8; i += DNT) {
+                const int row = i >> 3, pz = sl.own_lo + row / OY, y = row % OY, x4 = 4 * (i & 7);
+                if (y >= sl.lim[1] || x4 >= sl.lim[2]) continue;  // a multiple of 4 columns lies in the field
+                float *dst = F.a.xrec + ((size_t)(sl.g0[0] + pz) * f.n[1] + sl.g0[1] + y) * f.n[2] + sl.g0[2] + x4;
+                const float *sp = box + pz * DPLANE + y * DP + x4;
+                *reinterpret_cast<float4 *>(dst) = make_float4(sp[0], sp[1], sp[2], sp[3]);
+            }
+        } else {
+            // rows that are not 16-byte aligned: a warp stores one row per step, one value per lane
+            const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
             const size_t plane = (size_t)f.n[1] * f.n[2];
-            const int ny = min(OY, f.n[1] - sl.g0[1]);
-            if (lane < f.n[2] - sl.g0[2])
-                for (int y = warp; y < ny; y += NWARP) {
-                    const float *sp = box + sl.own_lo * PLANE + y * EX + lane;
+            if (lane < sl.lim[2])
+                for (int y = warp; y < sl.lim[1]; y += (DNT / 32)) {
+                    const float *sp = box + sl.own_lo * DPLANE + y * DP + lane;
                     float *gp = F.a.xrec + ((size_t)(sl.g0[0] + sl.own_lo) * f.n[1] + sl.g0[1] + y) * f.n[2] +
                                 sl.g0[2] + lane;
-#pragma unroll 2
-                    for (int i = 0; i < rows / OY; ++i, sp += PLANE, gp += plane) *gp = *sp;
+                    for (int i = 0; i < planes; ++i, sp += DPLANE, gp += plane) *gp = *sp;
                 }
-        } else {
-            // 8 lanes x 4 values per row, 4 rows per warp
-            const int sub = lane & 7;
-            for (int base = warp * 4; base < rows; base += NWARP * 4) {
-                const int row = base + (lane >> 3);
-                const int pz = sl.own_lo + row / OY, y = row % OY;
-                const int gz = sl.g0[0] + pz, gy = sl.g0[1] + y, gx = sl.g0[2] + 4 * sub;
-                if (gy >= f.n[1] || gx >= f.n[2]) continue;
-                const float *s4 = box + pz * PLANE + y * EX + 4 * sub;
-                float *dst = F.a.xrec + ((size_t)gz * f.n[1] + gy) * f.n[2] + gx;
-                // vec_xrec: rows are whole groups of 4 values
-                *reinterpret_cast<float4 *>(dst) = make_float4(s4[0], s4[1], s4[2], s4[3]);
-            }
         }
         __syncthreads();  // every thread is done reading the box
         if (!has_next) break;
         // ---- carry plane 8 into plane 0 of the next slab of the same run
-        if (nx.item == cu.item) {
-            for (int i = threadIdx.x; i < PLANE; i += NT) box[i] = box[8 * PLANE + i];
+        if (nx.s.carried) {
+            for (int i = threadIdx.x; i < DPLANE; i += DNT) box[i] = box[8 * DPLANE + i];
             __syncthreads();
         }
-        cu = nx;
-        sl = sn;
+        cur = nxt;
     }
     if (abort_flag && threadIdx.x == 0) {
-        atomicOr(&const_cast<interp_header *>(B.fld[MULTI ? cu.fi : 0].a.hdr)->status, INTERP_STATUS_TIMEOUT);
+        atomicOr(&const_cast<interp_header *>(B.fld[st[cur].fi].a.hdr)->status, INTERP_STATUS_TIMEOUT);
         // the transfer that did not arrive (the only one issued: the next slab's is
         // issued after the passes) gets a second bounded wait before the CTA's shared
         // memory is released
-        if (B.fld[MULTI ? cu.fi : 0].use_tma) mbar_wait_bounded(bar, phase ^ 1u, kTmaPolls);
+        if (B.fld[st[cur].fi].use_tma) mbar_wait_bounded(bar, phase ^ 1u, kTmaPolls);
     }
     cp_async_wait_all();
 }
 
 // ------------------------------------------------------------ host side
 constexpr int kMaxDevices = 64;
-int compress_grid[2][kMaxDevices];  // [MULTI]
-int decompress_grid[kMaxDevices], decompress_grid_multi[kMaxDevices];
+int compress_grid[2][kMaxDevices], decompress_grid[kMaxDevices];  // compression: [TMA]
 
 // Opt in to the kernel's dynamic shared memory and size the persistent grid
 // (resident CTAs per SM x SMs), once per device.
 template <typename K>
-cudaError_t prepare(K kernel, size_t smem, int *cache, int &grid)
+cudaError_t prepare(K kernel, int threads, size_t smem, int *cache, int &grid)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -1438,7 +1466,7 @@ cudaError_t prepare(K kernel, size_t smem, int *cache, int &grid)
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, NT, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
     grid = per_sm * sm_count();
@@ -1514,12 +1542,19 @@ cudaError_t launch_compress_tiles(const CompressArgs *args, int n, bool early, c
 {
     if (n < 1 || n > kMaxBatch) return cudaErrorInvalidValue;
     int grid = 0;
-    auto kernel = n > 1 ? k_compress<true> : k_compress<false>;
-    cudaError_t e = prepare(kernel, kCompressSmem, compress_grid[n > 1 ? 1 : 0], grid);
-    if (e != cudaSuccess) return e;
-    grid = scheduled_grid(grid, sched);
     thread_local CBatch B;  // large parameter block, filled on the host
     std::memset(&B, 0, sizeof(B));
+    bool tma = true;
+    for (int i = 0; i < n; ++i) {
+        const uint32_t box[3] = {XP, EY, XPL};  // planes 1..8 of a slab: must match issue_land<float, XP, XPL, 1, CNT>
+        B.fld[i].use_tma =
+            encode_tensor_map_3d(&B.map[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, args[i].x, args[i].dims, box) ? 1 : 0;
+        tma = tma && B.fld[i].use_tma;
+    }
+    auto kernel = tma ? k_compress<true> : k_compress<false>;
+    cudaError_t e = prepare(kernel, CNT, kCompressSmem, compress_grid[tma ? 1 : 0], grid);
+    if (e != cudaSuccess) return e;
+    grid = scheduled_grid(grid, sched);
     Field fs[kMaxBatch];
     for (int i = 0; i < n; ++i) fs[i] = field_of(args[i].dims);
     plan_runs(fs, n, grid, sched ? sched->run : 0);
@@ -1529,14 +1564,11 @@ cudaError_t launch_compress_tiles(const CompressArgs *args, int n, bool early, c
         B.fld[i].f = fs[i];
         B.fld[i].item0 = items;
         items += fs[i].items;
-        const uint32_t box[3] = {XP, EY, XPL};  // planes 1..8 of a slab: must match issue_land<float, XP, XPL, 1>
-        B.fld[i].use_tma =
-            encode_tensor_map_3d(&B.map[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, args[i].x, args[i].dims, box) ? 1 : 0;
     }
     B.n = n;
     B.items = items;
     if (items < grid) grid = items;
-    return launch_after(early, kernel, grid, NT, kCompressSmem, s, B);
+    return launch_after(early, kernel, grid, CNT, kCompressSmem, s, B);
 }
 
 cudaError_t launch_decompress_tiles(const DecompressArgs *args, int n, bool early, cudaStream_t s,
@@ -1544,8 +1576,7 @@ cudaError_t launch_decompress_tiles(const DecompressArgs *args, int n, bool earl
 {
     if (n < 1 || n > kMaxBatch) return cudaErrorInvalidValue;
     int grid = 0;
-    cudaError_t e = n > 1 ? prepare(k_decompress<true>, kDecompressSmem, decompress_grid_multi, grid)
-                          : prepare(k_decompress<false>, kDecompressSmem, decompress_grid, grid);
+    cudaError_t e = prepare(k_decompress, DNT, kDecompressSmem, decompress_grid, grid);
     if (e != cudaSuccess) return e;
     grid = scheduled_grid(grid, sched);
     thread_local DBatch B;
@@ -1567,7 +1598,7 @@ cudaError_t launch_decompress_tiles(const DecompressArgs *args, int n, bool earl
     B.n = n;
     B.items = items;
     if (items < grid) grid = items;
-    return launch_after(early, n > 1 ? k_decompress<true> : k_decompress<false>, grid, NT, kDecompressSmem, s, B);
+    return launch_after(early, k_decompress, grid, DNT, kDecompressSmem, s, B);
 }
 
 // ------------------------------------------------------------ tensor maps
