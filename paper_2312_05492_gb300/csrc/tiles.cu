@@ -1035,6 +1035,65 @@ __device__ __noinline__ void write_slab_rows(const CField &F, const CWrite cw, i
     }
 }
 
+// Bit j set iff the j-th of the 8 codes in w is zero (an outlier).
+__device__ __forceinline__ uint32_t zero_codes(const uint32_t (&w)[4])
+{
+    uint32_t m = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        // the top bit of each half: set iff the half is not zero (the sum cannot carry out of it)
+        const uint32_t t = ((w[j] & 0x7fff7fffu) + 0x7fff7fffu) | w[j];
+        m |= (~t & 0x80008000u) >> (15 - 2 * j);
+    }
+    return (m | (m >> 15)) & 0xffu;
+}
+
+// A slab with outliers whose rows all lie inside the field, with 16-byte aligned code rows
+// (write_slab_fast's geometry): a warp stores 8 rows of one plane per step, so its bitmap
+// words are consecutive and their outliers count towards one block of words or, where a
+// block ends between the rows, two.  The general form below, which took these slabs, spent a
+// quarter of their time on bounds, code by code tests and sums by shuffles (the kernel on
+// 1024^3 with 6% outliers: 3.64 -> 3.30 ms).
+__device__ __noinline__ void write_slab_outliers(const CField &F, int R, int WX, int z0, int y0, int x0, int col,
+                                                 int own_lo, int rows)
+{
+    const uint16_t *stage = reinterpret_cast<const uint16_t *>(g_smem + C_STAGE);
+    const Field &f = F.f;
+    constexpr int PSTEP = CNT / 4 / OY;  // planes per step
+    const int sub = threadIdx.x & 3;
+    int r = threadIdx.x >> 2;
+    const int y = r % OY;
+    int pz = own_lo + r / OY;
+    const size_t plane = (size_t)f.n[1] * f.n[2];
+    const uint16_t *sp = stage + pz * STAGE_PLANE + y * CP + 8 * sub;
+    uint16_t *gp = F.a.codes + ((size_t)(z0 + pz) * f.n[1] + y0 + y) * f.n[2] + x0 + 8 * sub;
+    uint32_t *wb = F.a.bitmap + ((size_t)col * f.n[0] + z0 + pz) * OY + y;
+    const bool anchor_row = (y & 7) == 0;
+    // word index (row-major) of the warp's first row; 32 bits: 16 points or more a word here
+    uint32_t w0 = ((uint32_t)(z0 + pz) * f.n[1] + y0 + (y & ~7)) * (uint32_t)WX + (uint32_t)x0 / 32u;
+    const uint32_t wstep = (uint32_t)PSTEP * f.n[1] * (uint32_t)WX;
+    // a warp's rows are whole planes' halves: all in or all out
+    for (; r < rows; r += CNT / 4, pz += PSTEP, sp += PSTEP * STAGE_PLANE, gp += PSTEP * plane, wb += PSTEP * OY,
+                     w0 += wstep) {
+        const uint32_t *s32 = reinterpret_cast<const uint32_t *>(sp);
+        uint32_t w[4] = {s32[0], s32[1], s32[2], s32[3]};
+        if (anchor_row && (pz & 7) == 0) w[0] = (w[0] & 0xffff0000u) | (uint32_t)R;  // anchor at x = 8*sub
+        *reinterpret_cast<uint4 *>(gp) = make_uint4(w[0], w[1], w[2], w[3]);
+        uint32_t word = zero_codes(w) << (8 * sub);
+        word |= __shfl_xor_sync(0xffffffffu, word, 1);
+        word |= __shfl_xor_sync(0xffffffffu, word, 2);
+        if (sub == 0) *wb = word;
+        const uint32_t b0 = w0 / BITMAP_BLOCK_WORDS, b1 = (w0 + 7u * WX) / BITMAP_BLOCK_WORDS;
+        const uint32_t c = sub == 0 ? (uint32_t)__popc(word) : 0u;
+        if (b0 == b1) {
+            const uint32_t all = __reduce_add_sync(0xffffffffu, c);
+            if ((threadIdx.x & 31) == 0 && all) atomicAdd(&F.a.blockcnt[b0], all);
+        } else if (c) {
+            atomicAdd(&F.a.blockcnt[(w0 + (uint32_t)(y & 7) * WX) / BITMAP_BLOCK_WORDS], c);
+        }
+    }
+}
+
 // Any other slab with 16-byte aligned code rows: codes and the exact
 // outlier-bitmap words with their block counts.  A warp takes 8 consecutive
 // rows of one plane, 4 lanes x 8 codes per row.
@@ -1183,6 +1242,8 @@ __global__ void __launch_bounds__(CNT, TMA ? kCompressCtas : kCompressCtas - 1) 
         const int planes = sl.lim[0] - sl.own_lo;
         if (!outliers && cw.code_store == 8 && sl.lim[1] == OY && sl.lim[2] == OX)
             write_slab_fast(F, cw, sl, planes * OY, stage);
+        else if (cw.code_store == 8 && sl.lim[1] == OY && sl.lim[2] == OX)
+            write_slab_outliers(F, cw.R, cw.WX, sl.g0[0], sl.g0[1], sl.g0[2], sl.col, sl.own_lo, planes * OY);
         else if (cw.code_store == 8)
             write_slab_general(F, cw, sl, planes * OY, stage);
         else

@@ -9,7 +9,7 @@ import oracle as O
 from paper_2312_05492_gb300 import fields
 from paper_2312_05492_gb300 import ginterp as G
 
-from _parity import bits
+from _parity import assert_parity, bits
 
 pytestmark = pytest.mark.gpu
 
@@ -49,3 +49,13 @@ def test_landed_in_place(offset, order):
         assert np.array_equal(bits(cf.out_val[:k].cpu().numpy()), bits(oc.out_val[:k]))
         assert np.array_equal(cf.hist.cpu().numpy().view(np.uint32), O.histogram(oc.codes, cfg.radius))
         assert np.array_equal(bits(xr.cpu().numpy()), bits(oc.xrec))
+
+
+@pytest.mark.parametrize("shape", [(10, 48, 1288), (9, 16, 32), (26, 35, 72), (17, 33, 32)])
+@pytest.mark.parametrize("eb", [1e-5, 1e-6])
+def test_outlier_words_of_whole_columns(shape, eb):
+    """Columns inside the field with outliers in most rows: words, counts (a block of words
+    that ends between a warp's rows: 41 words a row) and the list they give."""
+    x = fields.shocks(shape, 5).numpy()
+    _, _, h, _ = assert_parity(x, eb, G.Config(dim_order=(1, 0, 2), radius=64))
+    assert h.n_outliers > x.size // 64
