@@ -217,7 +217,7 @@ int compress_nd(const interp_compress_item &it, interp_stream_t stream)
     const gi::PrologueItem pro = prologue_item(it, L);
     cudaError_t e = gi::launch_prologue(&pro, 1, s);
     const gi::CompressArgs args{it.d_x, d, it.d_anchors, it.d_codes, bitmap, blockcnt, it.d_hist, c.radius,
-                                it.d_hdr, false, false, 1};
+                                it.d_hdr, false, 1};
     if (e == cudaSuccess) {
         timing_mark(0, 0, s);
         e = launch_nd_compress(c.ndim, args, early, s);
@@ -267,11 +267,11 @@ int interp_compress_batched_scheduled(const interp_compress_item *items, int n, 
         pro[i] = prologue_item(it, L[i]);
         if (is_nd(c.ndim))
             args[i] = gi::CompressArgs{it.d_x, d, it.d_anchors, it.d_codes, bitmap, blockcnt, it.d_hist, c.radius,
-                                       it.d_hdr, false, false, 1};
+                                       it.d_hdr, false, 1};
         else
             args3[n3++] = args[i] =
                 gi::CompressArgs{it.d_x, d, it.d_anchors, it.d_codes, bitmap, blockcnt, it.d_hist, c.radius,
-                                 it.d_hdr, gi::aligned16(it.d_codes) && d.nx % 8 == 0, c.domain_x == 32,
+                                 it.d_hdr, c.domain_x == 32,
                                  code_store_width(it.d_codes, d.nx)};
     }
     const bool early = small_fields(items, n);
@@ -285,8 +285,8 @@ int interp_compress_batched_scheduled(const interp_compress_item *items, int n, 
         timing_mark(0, 1, s);
     }
     if (e == cudaSuccess) {
-        // ordered compaction of every field in two launches; the tile kernels leave bin R of
-        // the histogram to the scan; 1-D / 2-D bitmaps are row-major
+        // ordered compaction of every field; the tile kernels leave bin R of the histogram to
+        // it; 1-D / 2-D bitmaps are row-major
         gi::CompactItem ci[gi::kMaxBatch];
         for (int i = 0; i < n; ++i) {
             const interp_compress_item &it = items[i];

@@ -15,16 +15,11 @@
 namespace gi {
 
 // ----------------------------------------------------------- tile geometry
-// A CTA works on a tile of TZ x TY x TX chunks of 8^3 points (Sec. IV-A),
-// staged in shared memory together with the closing faces at the far end of
-// each axis (the "borrowed" anchors and face points of the neighbouring
-// chunks, Sec. IV-C), i.e. a (8TZ+1) x (8TY+1) x (8TX+1) box.
-// A CTA marches along z through a column of 2 x 4 chunks of 8^3 points
-// (16 y x 32 x owned points), one slab of 8 planes at a time.
-#ifndef GI_TILE_ROWS
-#define GI_TILE_ROWS 16
-#endif
-constexpr int OY = GI_TILE_ROWS, OX = 32;  // owned extent of a column
+// A CTA marches along z through a column of 2 x 4 chunks of 8^3 points (Sec. IV-A;
+// 16 y x 32 x owned points), one slab of 8 planes at a time, held in shared memory together
+// with the closing faces at the far end of each axis (the "borrowed" anchors and face points
+// of the neighbouring chunks, Sec. IV-C): a box of 9 x 17 x 33 points.
+constexpr int OY = 16, OX = 32;  // owned extent of a column
 static_assert(OY % 8 == 0, "columns hold whole chunks");
 static_assert(OX == 32, "one outlier-bitmap word covers the 32 x-positions of an owned row");
 
@@ -40,10 +35,6 @@ constexpr int kMaxBatch = 16;
 // ------------------------------------------------------------- parameters
 struct Dims {
     int nz, ny, nx;
-};
-
-struct TileGrid {
-    int tz, ty, tx;  // tiles per axis
 };
 
 // ---------------------------------------------------------------- splines
@@ -214,7 +205,6 @@ struct CompressArgs {
     uint32_t *hist;  // may be null
     int radius;
     interp_header *hdr;
-    bool vec_codes;  // codes 16-byte aligned and nx % 8 == 0: 8-code vector stores
     bool xdom32;     // x-extended neighbour domain requested (cfg.domain_x == 32)
     int code_store;  // codes per store on rows of 8 codes starting at x = 8k: 8, 4 or 2
                      // (by the alignment of codes and nx), else 1

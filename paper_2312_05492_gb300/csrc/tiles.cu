@@ -11,12 +11,15 @@
 // faces are recomputed by the neighbouring column (bit-identical values).
 //
 // Persistent CTAs take work items = (column, run of slabs) round-robin and
-// march along z.  One thread issues a TMA box load of the next slab into a
-// dense staging buffer while the CTA runs the nine dependent passes (strides
-// 4, 2, 1; three axes each, a barrier between passes) on the current slab;
-// the staging buffer is then repacked into the compute box, whose odd row
-// pitch (33 floats) and plane pitch (561) make row-per-thread and
-// column-per-thread walks free of shared-memory bank conflicts.
+// march along z.  One thread issues the TMA box load of a slab (compression: its
+// values, decompression: its codes); the CTA runs the nine dependent passes
+// (strides 4, 2, 1; three axes each, a barrier between passes) on it, and the
+// next slab lands while this one is written out.
+//
+// What bounds the kernels: instructions.  A slab takes nine passes over few points each, so
+// the fixed cost of a pass (its dispatch, its barrier, the fetch of its code) counts as much
+// as its arithmetic; issue slots are 50-56% busy, HBM a third
+// (compression) and half (decompression) of its copy rate.
 //
 // Work unit inside a pass: one chunk segment, i.e. the 9 points of a line
 // along the pass axis inside one chunk; its known points (even multiples of
@@ -103,12 +106,12 @@ constexpr size_t D_LAND = 0;
 constexpr size_t D_BOX = al128(sizeof(uint16_t) * KLAND);
 constexpr size_t D_BAR = al16(D_BOX + sizeof(float) * EZ * DPLANE);
 constexpr size_t kDecompressSmem = D_BAR + 16;
-// with 16-row columns, 6 compression CTAs fit an SM: dynamic + static (< 512 B) + 1 KB reserved each
+// 6 compression CTAs fit an SM: dynamic + static (< 512 B) + 1 KB reserved each
 constexpr int kCompressCtas = 6;
-static_assert(OY != 16 || kCompressCtas * (kCompressSmem + 512 + 1024) <= 228 * 1024, "compression CTAs per SM");
+static_assert(kCompressCtas * (kCompressSmem + 512 + 1024) <= 228 * 1024, "compression CTAs per SM");
 // the smaller decompression CTA leaves room for six (at 56 registers a thread)
 constexpr int kDecompressCtas = 6;
-static_assert(OY != 16 || kDecompressCtas * (kDecompressSmem + 512 + 1024) <= 228 * 1024,
+static_assert(kDecompressCtas * (kDecompressSmem + 512 + 1024) <= 228 * 1024,
               "decompression CTAs per SM");
 
 // Nonzero iff one of the two 16-bit halves of w is zero (a borrow can only set
@@ -912,7 +915,6 @@ struct CBatch {
 // Per-field values of the compression write-out, re-read when the field changes.
 struct CWrite {
     int R, Ay, Ax, WX;
-    bool vec_codes;
     int code_store;
 };
 
@@ -923,7 +925,6 @@ __device__ __forceinline__ CWrite cwrite_of(const CField &F)
     w.Ay = (F.f.n[1] - 1) / 8 + 1;
     w.Ax = (F.f.n[2] - 1) / 8 + 1;
     w.WX = (F.f.n[2] + 31) / 32;
-    w.vec_codes = F.a.vec_codes;
     w.code_store = F.a.code_store;
     return w;
 }
@@ -957,7 +958,7 @@ __device__ __forceinline__ void write_anchors(const CField &F, const CWrite &cw,
 
 // The owned planes of a slab whose rows all lie inside the field, with 16-byte
 // aligned code rows and no outlier: staged codes -> global (8 codes per thread
-// and store, three planes per step), code R at anchors, and all-zero outlier-bitmap words.
+// and store, two planes per step), code R at anchors, and all-zero outlier-bitmap words.
 static_assert(CNT % 4 == 0 && (CNT / 4) % OY == 0, "write-out steps cover whole planes");
 __device__ __forceinline__ void write_slab_fast(const CField &F, const CWrite &cw, const Slab &sl, int rows,
                                                 const uint16_t *stage)
@@ -1053,7 +1054,7 @@ __device__ __forceinline__ uint32_t zero_codes(const uint32_t (&w)[4])
 // words are consecutive and their outliers count towards one block of words or, where a
 // block ends between the rows, two.  The general form below, which took these slabs, spent a
 // quarter of their time on bounds, code by code tests and sums by shuffles (the kernel on
-// 1024^3 with 6% outliers: 3.64 -> 3.30 ms).
+// 1024^3 with 11% outliers: 3.64 -> 3.30 ms).
 __device__ __noinline__ void write_slab_outliers(const CField &F, int R, int WX, int z0, int y0, int x0, int col,
                                                  int own_lo, int rows)
 {
