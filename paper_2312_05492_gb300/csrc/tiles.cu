@@ -35,12 +35,16 @@ namespace gi {
 namespace {
 
 // ------------------------------------------------------------ geometry
-// threads per CTA: with fewer, each warp does more of a pass per fixed cost (dispatch, index
-// set-up, barrier); compression 512^3 382 -> 361 us from 192 to 128 threads, decompression
-// is 2% slower with 128 and 13% with 256
-constexpr int CNT = 128, DNT = 192;
-template <bool COMPRESS>
-constexpr int kThreads = COMPRESS ? CNT : DNT;
+// Threads per CTA.  With fewer, each warp does more of a pass per fixed cost (dispatch, index
+// set-up, barrier): compression of 512^3 382 -> 361 us from 192 to 128 threads.  Where the
+// kernel waits more than it issues, more warps are worth more: in the general passes (the
+// x-extended domain at 384^3: 287-310 us with 128 threads, 275-289 with 192) and where a CTA
+// has a slab or two to do (64^3: 17.8 -> 14.9 us).  Rows without a tensor map like 128 too (three
+// uneven fields 525 -> 507 us).  Decompression is 2% slower with 128 threads and 13% with 256.
+constexpr int CNT = 128, CNT_WIDE = 192, DNT = 192;
+// The passes' template parameter COMPRESS: threads of the compression kernel, 0 for decompression.
+template <int COMPRESS>
+constexpr int kThreads = COMPRESS ? COMPRESS : DNT;
 constexpr int EZ = 9, EY = OY + 1, EX = OX + 1;  // slab box extents (z, y, x)
 // Floats per box row and plane.  Compression works where the TMA landed the values, so its
 // rows are whole 16-byte groups: an odd number of them, so that a warp's 16-byte reads of
@@ -62,7 +66,7 @@ constexpr uint32_t kTmaPolls = 1u << 22;         // bounded wait for one TMA box
 
 __host__ __device__ constexpr int ext_of(int a) { return a == 2 ? EX : (a == 1 ? EY : EZ); }
 __host__ __device__ constexpr int own_of(int a) { return a == 2 ? OX : (a == 1 ? OY : EZ); }
-template <bool COMPRESS>
+template <int COMPRESS>
 __host__ __device__ constexpr int bstride(int a)
 {
     return a == 2 ? 1 : (a == 1 ? (COMPRESS ? XP : DP) : (COMPRESS ? PLANE : DPLANE));
@@ -258,7 +262,7 @@ __device__ __forceinline__ void count_code(const Sink &sk, uint32_t code, uint32
 
 // INTERIOR: the slab's whole box lies inside the field and every chunk is
 // full, so no line or chunk needs the field-edge checks.
-template <bool COMPRESS, bool INTERIOR, int S, int D, bool XDOM = false>
+template <int COMPRESS, bool INTERIOR, int S, int D, bool XDOM = false>
 __device__ __forceinline__ void run_pass(float *__restrict__ box, const Sink &sk, const Slab &sl, const Field &f,
                                          const Levels &lv, int k)
 {
@@ -409,7 +413,7 @@ __device__ __forceinline__ void run_pass(float *__restrict__ box, const Sink &sk
     }
 }
 
-template <bool COMPRESS, bool INTERIOR, int S, bool XDOM>
+template <int COMPRESS, bool INTERIOR, int S, bool XDOM>
 __device__ __forceinline__ void run_level(float *box, const Sink &sk, const Slab &sl, const Field &f,
                                           const Levels &lv)
 {
@@ -423,7 +427,7 @@ __device__ __forceinline__ void run_level(float *box, const Sink &sk, const Slab
     }
 }
 
-template <bool COMPRESS, bool XDOM>
+template <int COMPRESS, bool XDOM>
 __device__ __forceinline__ void run_levels(float *box, const Sink &sk, const Slab &sl, const Field &f,
                                            const Levels &lv)
 {
@@ -485,7 +489,7 @@ struct SegOut {
     bool owned;      // the point's code is counted (compression)
 };
 
-template <bool COMPRESS>
+template <int COMPRESS>
 __device__ __forceinline__ void seg_emit(float *L, uint16_t *C, int ob, int oc, float p, const LevelQ &Lq,
                                          uint32_t cbias, float Rf, const SegOut &so)
 {
@@ -521,7 +525,7 @@ __device__ __forceinline__ float cubic_of(float m3, float m1, float p1, float p3
 // A segment of a full chunk: the fixed stencils of Fig. 3 (splines: cubic at
 // offsets 3 and 5, quadratics at 1 and 7 for stride 1; quadratics at stride 2;
 // stride 4 is always linear).
-template <bool COMPRESS, int S, int BD, int KD, int KIND>
+template <int COMPRESS, int S, int BD, int KD, int KIND>
 __device__ __forceinline__ void seg_full(float *L, uint16_t *C, const LevelQ &Lq, uint32_t cbias, float Rf,
                                          const SegOut &so)
 {
@@ -594,7 +598,7 @@ __device__ __forceinline__ void seg_full(float *L, uint16_t *C, const LevelQ &Lq
 
 // A segment of a chunk cut by the field's far edge (last in-field offset hi < 8):
 // the neighbour-count rule point by point (Sec. IV-B.1).
-template <bool COMPRESS, int S, int BD, int KD>
+template <int COMPRESS, int S, int BD, int KD>
 __device__ __forceinline__ void seg_trunc(float *L, uint16_t *C, int hi, bool spline, const LevelQ &Lq,
                                           const Cubic &cub, uint32_t cbias, float Rf, const SegOut &so)
 {
@@ -631,7 +635,7 @@ struct PassK {
 // Pass k of the level of stride S for axis order ORD.  Segments are numbered with
 // U (the faster other axis) fastest, then V, then the chunk along D; thread t
 // takes segments t, t + threads, ...  Threads without a segment skip the pass at once.
-template <bool COMPRESS, int ORD, bool CARRIED, int S, int K, int KIND>
+template <int COMPRESS, int ORD, bool CARRIED, int S, int K, int KIND>
 __device__ __forceinline__ void fast_pass(const FastCtx &c, const PassK &pk)
 {
     constexpr bool SPLINE = KIND != KIND_LINEAR;
@@ -671,7 +675,7 @@ __device__ __forceinline__ void fast_pass(const FastCtx &c, const PassK &pk)
     }
 }
 
-template <bool COMPRESS, int ORD, bool CARRIED, int S, int K>
+template <int COMPRESS, int ORD, bool CARRIED, int S, int K>
 __device__ __forceinline__ void fast_pass_any(const FastCtx &c, const PassK &pk, bool spline)
 {
     constexpr int D = ord_axis(ORD, K);
@@ -687,7 +691,7 @@ __device__ __forceinline__ void fast_pass_any(const FastCtx &c, const PassK &pk,
     __syncthreads();
 }
 
-template <bool COMPRESS, int ORD, bool CARRIED, int S>
+template <int COMPRESS, int ORD, bool CARRIED, int S>
 __device__ __forceinline__ void fast_level(const FastCtx &c, PassK pk)
 {
     constexpr int l = S == 1 ? 0 : (S == 2 ? 1 : 2);
@@ -699,7 +703,7 @@ __device__ __forceinline__ void fast_level(const FastCtx &c, PassK pk)
     fast_pass_any<COMPRESS, ORD, CARRIED, S, 2>(c, pk, spline);
 }
 
-template <bool COMPRESS, int ORD>
+template <int COMPRESS, int ORD>
 __device__ __forceinline__ void fast_slab(const FastCtx &c, const PassK &pk, bool carried)
 {
     if (carried) {
@@ -715,7 +719,7 @@ __device__ __forceinline__ void fast_slab(const FastCtx &c, const PassK &pk, boo
 
 // The nine passes of a slab in the default neighbour domain, every order.
 // rem: last in-field offset per axis from the box origin; lim: Slab::lim.
-template <bool COMPRESS>
+template <int COMPRESS>
 __device__ __forceinline__ void fast_levels(float *box, uint16_t *codes, uint32_t *hist, int rem0, int rem1,
                                             int rem2, int lim0, int lim1, int lim2, bool carried, const Levels &lv)
 {
@@ -750,7 +754,7 @@ __device__ __forceinline__ void fast_levels(float *box, uint16_t *codes, uint32_
 // the x-extended domain (an option) and radii whose bins do not fit the shared
 // histogram take the general passes.  Both are out-of-line functions, compiled
 // once for every kernel that calls them (the call happens once per slab).
-template <bool COMPRESS>
+template <int COMPRESS>
 __device__ __noinline__ void passes_fast(int code_off, int rem0, int rem1, int rem2, int lim0, int lim1, int lim2,
                                          bool carried)
 {
@@ -761,7 +765,7 @@ __device__ __noinline__ void passes_fast(int code_off, int rem0, int rem1, int r
     fast_levels<COMPRESS>(box, codes, hist, rem0, rem1, rem2, lim0, lim1, lim2, carried, g_lv);
 }
 
-template <bool COMPRESS>
+template <int COMPRESS>
 __device__ __noinline__ void passes_general(const Slab sl, const Field f, uint32_t *hist_g)
 {
     // shared-memory pointers derived from the symbol (not passed in), so that every box,
@@ -774,7 +778,7 @@ __device__ __noinline__ void passes_general(const Slab sl, const Field f, uint32
     else run_levels<COMPRESS, false>(box, sk, sl, f, g_lv);
 }
 
-template <bool COMPRESS>
+template <int COMPRESS>
 __device__ __forceinline__ void run_slab(float *box, const Sink &sk, const Slab &sl, const Field &f,
                                          const Levels &lv)
 {
@@ -930,16 +934,17 @@ __device__ __forceinline__ CWrite cwrite_of(const CField &F)
 }
 
 // Add the CTA's histogram counts of one field to its global bins and clear them.
+template <int NT>
 __device__ __forceinline__ void flush_hist(const CField &F, uint32_t *hist_s)
 {
     __syncthreads();
     const int bins = min(2 * F.a.radius, HIST_SMEM_BINS);
     if (F.a.hist)
-        for (int i = threadIdx.x; i < bins; i += CNT) {
+        for (int i = threadIdx.x; i < bins; i += NT) {
             const uint32_t h = hist_s[i];
             if (h) atomicAdd(&F.a.hist[i], h);
         }
-    for (int i = threadIdx.x; i < HIST_SMEM_BINS; i += CNT) hist_s[i] = 0u;
+    for (int i = threadIdx.x; i < HIST_SMEM_BINS; i += NT) hist_s[i] = 0u;
     __syncthreads();
 }
 
@@ -959,12 +964,13 @@ __device__ __forceinline__ void write_anchors(const CField &F, const CWrite &cw,
 // The owned planes of a slab whose rows all lie inside the field, with 16-byte
 // aligned code rows and no outlier: staged codes -> global (8 codes per thread
 // and store, two planes per step), code R at anchors, and all-zero outlier-bitmap words.
-static_assert(CNT % 4 == 0 && (CNT / 4) % OY == 0, "write-out steps cover whole planes");
+template <int NT>
 __device__ __forceinline__ void write_slab_fast(const CField &F, const CWrite &cw, const Slab &sl, int rows,
                                                 const uint16_t *stage)
 {
     const Field &f = F.f;
-    constexpr int PSTEP = CNT / 4 / OY;  // planes per step
+    static_assert(NT % 4 == 0 && (NT / 4) % OY == 0, "steps cover whole planes");
+    constexpr int PSTEP = NT / 4 / OY;  // planes per step
     const int sub = threadIdx.x & 3;
     int r = threadIdx.x >> 2;
     const int y = r % OY;
@@ -973,7 +979,7 @@ __device__ __forceinline__ void write_slab_fast(const CField &F, const CWrite &c
     const uint16_t *sp = stage + pz * STAGE_PLANE + y * CP + 8 * sub;
     uint16_t *gp = F.a.codes + ((size_t)(sl.g0[0] + pz) * f.n[1] + sl.g0[1] + y) * f.n[2] + sl.g0[2] + 8 * sub;
     const bool anchor_row = (y & 7) == 0;
-    for (; r < rows; r += CNT / 4, pz += PSTEP, sp += PSTEP * STAGE_PLANE, gp += PSTEP * plane) {
+    for (; r < rows; r += NT / 4, pz += PSTEP, sp += PSTEP * STAGE_PLANE, gp += PSTEP * plane) {
         const uint32_t *s32 = reinterpret_cast<const uint32_t *>(sp);
         uint32_t w0 = s32[0];
         const uint32_t w1 = s32[1], w2 = s32[2], w3 = s32[3];
@@ -989,6 +995,7 @@ __device__ __forceinline__ void write_slab_fast(const CField &F, const CWrite &c
 // (consecutive addresses, whatever their alignment; 4 lanes x 8 codes per row had made
 // every 2-byte store touch 32 sectors); the row's outlier word is a ballot.
 // Out of line: inlined, it made the aligned fields' loop 1% slower.
+template <int NT>
 __device__ __noinline__ void write_slab_rows(const CField &F, const CWrite cw, int z0, int y0, int x0, int col,
                                              int own_lo, int planes)
 {
@@ -1007,7 +1014,7 @@ __device__ __noinline__ void write_slab_rows(const CField &F, const CWrite cw, i
     const size_t my_block = block_of(lane < planes ? lane : 0, 0);
     const uint32_t split = __ballot_sync(0xffffffffu, lane < planes && my_block != block_of(lane, ny - 1));
     uint32_t count = 0;
-    for (int y = warp; y < ny; y += (CNT / 32)) {
+    for (int y = warp; y < ny; y += (NT / 32)) {
         const size_t grow = (size_t)(z0 + own_lo) * f.n[1] + y0 + y;
         uint16_t *gp = F.a.codes + grow * f.n[2] + x0 + lane;
         uint32_t *wb = F.a.bitmap + ((size_t)col * f.n[0] + z0 + own_lo) * OY + y;
@@ -1055,12 +1062,13 @@ __device__ __forceinline__ uint32_t zero_codes(const uint32_t (&w)[4])
 // block ends between the rows, two.  The general form below, which took these slabs, spent a
 // quarter of their time on bounds, code by code tests and sums by shuffles (the kernel on
 // 1024^3 with 11% outliers: 3.64 -> 3.30 ms).
+template <int NT>
 __device__ __noinline__ void write_slab_outliers(const CField &F, int R, int WX, int z0, int y0, int x0, int col,
                                                  int own_lo, int rows)
 {
     const uint16_t *stage = reinterpret_cast<const uint16_t *>(g_smem + C_STAGE);
     const Field &f = F.f;
-    constexpr int PSTEP = CNT / 4 / OY;  // planes per step
+    constexpr int PSTEP = NT / 4 / OY;  // planes per step
     const int sub = threadIdx.x & 3;
     int r = threadIdx.x >> 2;
     const int y = r % OY;
@@ -1074,7 +1082,7 @@ __device__ __noinline__ void write_slab_outliers(const CField &F, int R, int WX,
     uint32_t w0 = ((uint32_t)(z0 + pz) * f.n[1] + y0 + (y & ~7)) * (uint32_t)WX + (uint32_t)x0 / 32u;
     const uint32_t wstep = (uint32_t)PSTEP * f.n[1] * (uint32_t)WX;
     // a warp's rows are whole planes' halves: all in or all out
-    for (; r < rows; r += CNT / 4, pz += PSTEP, sp += PSTEP * STAGE_PLANE, gp += PSTEP * plane, wb += PSTEP * OY,
+    for (; r < rows; r += NT / 4, pz += PSTEP, sp += PSTEP * STAGE_PLANE, gp += PSTEP * plane, wb += PSTEP * OY,
                      w0 += wstep) {
         const uint32_t *s32 = reinterpret_cast<const uint32_t *>(sp);
         uint32_t w[4] = {s32[0], s32[1], s32[2], s32[3]};
@@ -1098,13 +1106,14 @@ __device__ __noinline__ void write_slab_outliers(const CField &F, int R, int WX,
 // Any other slab with 16-byte aligned code rows: codes and the exact
 // outlier-bitmap words with their block counts.  A warp takes 8 consecutive
 // rows of one plane, 4 lanes x 8 codes per row.
+template <int NT>
 __device__ __forceinline__ void write_slab_general(const CField &F, const CWrite &cw, const Slab &sl, int rows,
                                                    const uint16_t *stage)
 {
     const Field &f = F.f;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int sub = lane & 3;
-    for (int base = warp * 8; base < rows; base += (CNT / 32) * 8) {
+    for (int base = warp * 8; base < rows; base += (NT / 32) * 8) {
         const int row = base + (lane >> 2);
         const int pz = sl.own_lo + row / OY, y = row % OY;
         const int gz = sl.g0[0] + pz, gy = sl.g0[1] + y;
@@ -1157,12 +1166,13 @@ __device__ __forceinline__ void write_slab_general(const CField &F, const CWrite
     }
 }
 
-// TMA: every field's rows can be described by a tensor map.  Otherwise (copies by all
-// threads for the fields that cannot) one CTA less per SM: the shared memory of six leaves
-// next to no L1 cache, through which those copies go (449x449x235 274 -> 263 us; with TMA
-// the sixth CTA is worth 377 -> 361 us on 512^3).
-template <bool TMA>
-__global__ void __launch_bounds__(CNT, TMA ? kCompressCtas : kCompressCtas - 1) k_compress(const __grid_constant__ CBatch B)
+// TMA: every field's rows can be described by a tensor map: six CTAs of 128 threads.
+// Otherwise (copies by all threads for the fields that cannot) five: the shared memory of six
+// leaves next to no L1 cache, through which those copies go (449x449x235 274 -> 263 us; with
+// TMA the sixth CTA is worth 377 -> 361 us on 512^3).  Five of CNT_WIDE: see there.
+template <int NT, bool TMA>
+__global__ void __launch_bounds__(NT, TMA ? kCompressCtas : kCompressCtas - 1)
+    k_compress(const __grid_constant__ CBatch B)
 {
     wait_for_previous();
     unsigned char *smem = g_smem;
@@ -1181,7 +1191,7 @@ __global__ void __launch_bounds__(CNT, TMA ? kCompressCtas : kCompressCtas - 1) 
         mbar_init(bar, 1);
         fence_barrier_init();
     }
-    for (int i = threadIdx.x; i < HIST_WORDS; i += CNT) hist_s[i] = 0u;
+    for (int i = threadIdx.x; i < HIST_WORDS; i += NT) hist_s[i] = 0u;
     __syncthreads();
 
     uint32_t phase = 0;
@@ -1192,7 +1202,7 @@ __global__ void __launch_bounds__(CNT, TMA ? kCompressCtas : kCompressCtas - 1) 
     uint32_t out_seen = 0;  // outliers in the shared histogram before the current slab
     {
         const CField &F = B.fld[st[0].fi];
-        issue_land<float, XP, XPL, 1, CNT>(land, F.a.x, &B.map[st[0].fi], TMA || F.use_tma, bar, F.f, st[0].s);
+        issue_land<float, XP, XPL, 1, NT>(land, F.a.x, &B.map[st[0].fi], TMA || F.use_tma, bar, F.f, st[0].s);
     }
     for (;;) {
         const Slab &sl = st[cur].s;
@@ -1203,14 +1213,14 @@ __global__ void __launch_bounds__(CNT, TMA ? kCompressCtas : kCompressCtas - 1) 
         // the next slab (slots in turn by three: a slow thread may still be writing out the
         // previous slab)
         const int nxt = cur == 2 ? 0 : cur + 1;
-        if (threadIdx.x == CNT - 1) slab_next(st[nxt], st[cur], bv);
+        if (threadIdx.x == NT - 1) slab_next(st[nxt], st[cur], bv);
         lv_field = fi;
 
         // ---- input: plane 0 carried, or loaded directly at a run's start; planes 1..8 landed
         if (!sl.carried) {
             const int nyr = min(EY, f.n[1] - sl.g0[1]), nxc = min(EX, f.n[2] - sl.g0[2]);
             const float *src = F.a.x + ((size_t)sl.g0[0] * f.n[1] + sl.g0[1]) * f.n[2] + sl.g0[2];
-            for (int i = threadIdx.x; i < EY * EX; i += CNT) {
+            for (int i = threadIdx.x; i < EY * EX; i += NT) {
                 const int y = i / EX, xx = i - y * EX;
                 if (y < nyr && xx < nxc) box[y * XP + xx] = __ldg(src + (size_t)y * f.n[2] + xx);
             }
@@ -1221,7 +1231,7 @@ __global__ void __launch_bounds__(CNT, TMA ? kCompressCtas : kCompressCtas - 1) 
         const CWrite cw = cwrite_of(F);
         write_anchors(F, cw, sl, box);
 
-        run_slab<true>(box, Sink{stage, nullptr, hist_s, F.a.hist}, sl, f, lv);  // ends with a barrier
+        run_slab<NT>(box, Sink{stage, nullptr, hist_s, F.a.hist}, sl, f, lv);  // ends with a barrier
 
         const uint32_t out_now = hist_s[0];  // no code is counted between here and the next slab's first barrier
         const bool outliers = out_now != out_seen;
@@ -1231,26 +1241,26 @@ __global__ void __launch_bounds__(CNT, TMA ? kCompressCtas : kCompressCtas - 1) 
         // ---- plane 8 carried into plane 0 when the next slab continues this run; then the
         // next slab's input, which lands while this slab's codes are written out
         if (has_next && nx.s.carried)
-            for (int i = threadIdx.x; i < PLANE / 4; i += CNT)
+            for (int i = threadIdx.x; i < PLANE / 4; i += NT)
                 reinterpret_cast<float4 *>(box)[i] = reinterpret_cast<const float4 *>(box + 8 * PLANE)[i];
         __syncthreads();
         if (has_next) {
             const int nfi = nx.fi;
             const CField &N = B.fld[nfi];
-            issue_land<float, XP, XPL, 1, CNT>(land, N.a.x, &B.map[nfi], TMA || N.use_tma, bar, N.f, nx.s);
+            issue_land<float, XP, XPL, 1, NT>(land, N.a.x, &B.map[nfi], TMA || N.use_tma, bar, N.f, nx.s);
         }
         // ---- owned planes: codes and outlier-bitmap words
         const int planes = sl.lim[0] - sl.own_lo;
         if (!outliers && cw.code_store == 8 && sl.lim[1] == OY && sl.lim[2] == OX)
-            write_slab_fast(F, cw, sl, planes * OY, stage);
+            write_slab_fast<NT>(F, cw, sl, planes * OY, stage);
         else if (cw.code_store == 8 && sl.lim[1] == OY && sl.lim[2] == OX)
-            write_slab_outliers(F, cw.R, cw.WX, sl.g0[0], sl.g0[1], sl.g0[2], sl.col, sl.own_lo, planes * OY);
+            write_slab_outliers<NT>(F, cw.R, cw.WX, sl.g0[0], sl.g0[1], sl.g0[2], sl.col, sl.own_lo, planes * OY);
         else if (cw.code_store == 8)
-            write_slab_general(F, cw, sl, planes * OY, stage);
+            write_slab_general<NT>(F, cw, sl, planes * OY, stage);
         else
-            write_slab_rows(F, cw, sl.g0[0], sl.g0[1], sl.g0[2], sl.col, sl.own_lo, planes);
+            write_slab_rows<NT>(F, cw, sl.g0[0], sl.g0[1], sl.g0[2], sl.col, sl.own_lo, planes);
         if (!has_next || nx.fi != fi) {  // field done
-            flush_hist(F, hist_s);
+            flush_hist<NT>(F, hist_s);
             out_seen = 0;
         }
         if (!has_next) break;
@@ -1264,7 +1274,7 @@ __global__ void __launch_bounds__(CNT, TMA ? kCompressCtas : kCompressCtas - 1) 
             // CTA's shared memory is released
             if (B.fld[fi].use_tma) mbar_wait_bounded(bar, phase ^ 1u, kTmaPolls);
         }
-        flush_hist(B.fld[fi], hist_s);
+        flush_hist<NT>(B.fld[fi], hist_s);
     }
     cp_async_wait_all();
 }
@@ -1443,7 +1453,7 @@ __global__ void __launch_bounds__(DNT, kDecompressCtas) k_decompress(const __gri
         }
         if (abort_flag) break;
 
-        run_slab<false>(box, Sink{nullptr, land, nullptr, nullptr}, sl, f, lv);  // ends with a barrier
+        run_slab<0>(box, Sink{nullptr, land, nullptr, nullptr}, sl, f, lv);  // ends with a barrier
         // ---- the codes are read: the next slab's land during the write-out
         if (has_next) {
             const int nfi = nx.fi;
@@ -1511,7 +1521,7 @@ __global__ void __launch_bounds__(DNT, kDecompressCtas) k_decompress(const __gri
 
 // ------------------------------------------------------------ host side
 constexpr int kMaxDevices = 64;
-int compress_grid[2][kMaxDevices], decompress_grid[kMaxDevices];  // compression: [TMA]
+int compress_grid[3][kMaxDevices], decompress_grid[kMaxDevices];  // compression: per variant of the kernel
 
 // Opt in to the kernel's dynamic shared memory and size the persistent grid
 // (resident CTAs per SM x SMs), once per device.
@@ -1606,19 +1616,26 @@ cudaError_t launch_compress_tiles(const CompressArgs *args, int n, bool early, c
     int grid = 0;
     thread_local CBatch B;  // large parameter block, filled on the host
     std::memset(&B, 0, sizeof(B));
-    bool tma = true;
+    Field fs[kMaxBatch];
+    bool tma = true, general = false;
+    long long slabs = 0;
     for (int i = 0; i < n; ++i) {
-        const uint32_t box[3] = {XP, EY, XPL};  // planes 1..8 of a slab: must match issue_land<float, XP, XPL, 1, CNT>
+        const uint32_t box[3] = {XP, EY, XPL};  // planes 1..8 of a slab: must match issue_land<float, XP, XPL, 1, NT>
         B.fld[i].use_tma =
             encode_tensor_map_3d(&B.map[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, args[i].x, args[i].dims, box) ? 1 : 0;
         tma = tma && B.fld[i].use_tma;
+        general = general || args[i].xdom32 || 2 * args[i].radius > HIST_SMEM_BINS;
+        fs[i] = field_of(args[i].dims);
+        slabs += (long long)fs[i].cols * fs[i].slabs;
     }
-    auto kernel = tma ? k_compress<true> : k_compress<false>;
-    cudaError_t e = prepare(kernel, CNT, kCompressSmem, compress_grid[tma ? 1 : 0], grid);
+    // the wide kernel: general passes, or at most two slabs a CTA (five an SM)
+    const bool wide = general || slabs <= 2ll * (kCompressCtas - 1) * sm_count();
+    const int variant = wide ? 2 : (tma ? 1 : 0);
+    auto kernel = wide ? k_compress<CNT_WIDE, false> : (tma ? k_compress<CNT, true> : k_compress<CNT, false>);
+    const int threads = wide ? CNT_WIDE : CNT;
+    cudaError_t e = prepare(kernel, threads, kCompressSmem, compress_grid[variant], grid);
     if (e != cudaSuccess) return e;
     grid = scheduled_grid(grid, sched);
-    Field fs[kMaxBatch];
-    for (int i = 0; i < n; ++i) fs[i] = field_of(args[i].dims);
     plan_runs(fs, n, grid, sched ? sched->run : 0);
     int items = 0;
     for (int i = 0; i < n; ++i) {
@@ -1630,7 +1647,7 @@ cudaError_t launch_compress_tiles(const CompressArgs *args, int n, bool early, c
     B.n = n;
     B.items = items;
     if (items < grid) grid = items;
-    return launch_after(early, kernel, grid, CNT, kCompressSmem, s, B);
+    return launch_after(early, kernel, grid, threads, kCompressSmem, s, B);
 }
 
 cudaError_t launch_decompress_tiles(const DecompressArgs *args, int n, bool early, cudaStream_t s,
