@@ -150,7 +150,10 @@ int interp_compress(const float *d_x, const int64_t dims[3], double eb, const in
  *   dims must equal the dims the field was compressed with (the caller keeps
  *   them; they are also in the header); d_hdr, d_anchors, d_codes, d_out_idx,
  *   d_out_val as written by interp_compress, with out_capacity entries
- *   available (the first min(n_outliers, out_capacity) are scattered);
+ *   available (the first min(n_outliers, out_capacity) are scattered; where the list
+ *   was too short (INTERP_STATUS_CAPACITY), the outliers past its last index are
+ *   reconstructed as 0, and their neighbours from that).  out_capacity = 0: no list is
+ *   read, and an outlier keeps what d_xrec holds.
  *   d_xrec [N] out.  No workspace is needed. */
 int interp_decompress(const int64_t dims[3], const interp_header *d_hdr, const float *d_anchors,
                       const uint16_t *d_codes, const uint32_t *d_out_idx, const float *d_out_val,

@@ -58,6 +58,7 @@ bool cfg_ok(const interp_config *c)
 // tile-major (see tiles.cu)
 Dims to_dims(const int64_t *d) { return Dims{(int)d[0], (int)d[1], (int)d[2]}; }
 
+uint64_t points_of(const int64_t *dims) { return (uint64_t)dims[0] * dims[1] * dims[2]; }
 int64_t bitmap_words(const int64_t *dims) { return dims[0] * dims[1] * ((dims[2] + 31) / 32); }
 
 struct WsLayout {
@@ -348,7 +349,7 @@ int interp_decompress_batched_scheduled(const interp_decompress_item *items, int
         const interp_decompress_item &it = items[i];
         const Dims d = to_dims(it.dims);
         if (it.out_capacity > 0) sc[nsc++] = gi::ScatterItem{it.d_hdr, it.d_out_idx, it.d_out_val, it.out_capacity,
-                                                             it.d_xrec};
+                                                             it.d_xrec, points_of(it.dims)};
         if (is_nd(it.ndim))
             args[i] = gi::DecompressArgs{d, it.d_anchors, it.d_codes, it.d_xrec, it.d_hdr, false};
         else
@@ -404,7 +405,7 @@ int interp_decompress_nd(int32_t ndim, const int64_t dims[3], const interp_heade
     const Dims d = to_dims(dims);
     cudaError_t e = cudaSuccess;
     if (out_capacity > 0) {
-        const gi::ScatterItem sc{d_hdr, d_out_idx, d_out_val, out_capacity, d_xrec};
+        const gi::ScatterItem sc{d_hdr, d_out_idx, d_out_val, out_capacity, d_xrec, points_of(dims)};
         e = gi::launch_outlier_scatter(&sc, 1, s);
     }
     const bool early = gi::small_call((unsigned long long)dims[0] * dims[1] * dims[2]);

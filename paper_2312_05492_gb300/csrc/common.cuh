@@ -298,6 +298,7 @@ struct ScatterItem {
     const float *val;
     uint64_t capacity;
     float *xrec;
+    uint64_t points;  // of the field
 };
 cudaError_t launch_outlier_scatter(const ScatterItem *items, int n, cudaStream_t s);
 cudaError_t launch_histogram(const uint16_t *codes, uint64_t n, int radius, uint32_t *hist, cudaStream_t s);

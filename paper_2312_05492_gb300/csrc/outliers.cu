@@ -233,6 +233,7 @@ struct ScatterField {
     const float *val;
     unsigned long long capacity;
     float *xrec;
+    unsigned long long points;
 };
 
 struct ScatterBatch {
@@ -246,9 +247,14 @@ __global__ void k_outlier_scatter(const __grid_constant__ ScatterBatch B)
     const ScatterField &F = B.f[blockIdx.x / B.blocks];
     const unsigned long long b = blockIdx.x % B.blocks;
     unsigned long long n = F.hdr->n_outliers;
-    if (n > F.capacity) n = F.capacity;
     const unsigned long long step = (unsigned long long)B.blocks * blockDim.x;
     unsigned long long i = b * blockDim.x + threadIdx.x;
+    if (n > F.capacity) {
+        // a list that was too short: the outliers past its last index (it is ascending) have
+        // no value, and read as 0 and not as what xrec happened to hold
+        n = F.capacity;
+        for (unsigned long long k = F.idx[n - 1] + 1ull + i; k < F.points; k += step) F.xrec[k] = 0.0f;
+    }
     for (; i + 3 * step < n; i += 4 * step) {  // four independent pairs in flight
         uint32_t k[4];
         float v[4];
@@ -368,7 +374,8 @@ cudaError_t launch_outlier_scatter(const ScatterItem *items, int n, cudaStream_t
     ScatterBatch B;
     std::memset(&B, 0, sizeof(B));
     for (int i = 0; i < n; ++i) B.f[i] = ScatterField{items[i].hdr, items[i].idx, items[i].val,
-                                                      (unsigned long long)items[i].capacity, items[i].xrec};
+                                                      (unsigned long long)items[i].capacity, items[i].xrec,
+                                                      (unsigned long long)items[i].points};
     B.n = n;
     // a full SM of threads (the stores are scattered), but no more than the lists may need
     uint64_t most = 1;
