@@ -162,7 +162,9 @@ __device__ __forceinline__ float code_to_q(uint32_t code, uint32_t cbias)
 // set up, its CTAs waiting here, while the one before it in the stream still runs; it goes
 // on, and touches memory, only when that one is complete and its writes are visible.  Each
 // kernel lets the next one be set up as soon as it has started itself.  Only set-up
-// overlaps, never work: about 1.5 us a launch.
+// overlaps, never work: about 1.5 us a launch.  What the kernel before writes is read by
+// plain loads: it is not read-only in this kernel's lifetime, and a load that says so (__ldg,
+// const __restrict__) may be moved above the wait.
 __device__ __forceinline__ void wait_for_previous()
 {
     asm volatile("griddepcontrol.wait;\n" ::: "memory");

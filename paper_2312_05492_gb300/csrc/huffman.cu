@@ -393,12 +393,13 @@ __device__ __forceinline__ void store_group(uint16_t *dst, const unsigned char *
     }
 }
 
+// tg, symbols: written by the kernel before, which may still run when this one starts (no
+// __restrict__: see wait_for_previous).
 template <int VEC>
 __global__ void __launch_bounds__(DEC_THREADS, 2) k_huff_decode(const uint32_t *__restrict__ words,
                                                                const uint32_t *__restrict__ offsets,
-                                                               unsigned long long n, const DecodeTables *__restrict__ tg,
-                                                               const uint16_t *__restrict__ symbols, int nsym,
-                                                               int nsym_smem, uint16_t *codes,
+                                                               unsigned long long n, const DecodeTables *tg,
+                                                               const uint16_t *symbols, int nsym, int nsym_smem, uint16_t *codes,
                                                                unsigned long long nchunks, unsigned int *bad)
 {
     wait_for_previous();

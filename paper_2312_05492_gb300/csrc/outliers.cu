@@ -96,7 +96,8 @@ __device__ void outlier_scan_block(uint32_t *blockcnt, int nblk, interp_header *
 }
 
 // The outliers of bitmap block b of a field, written from position `start` of its list on.
-__device__ void outlier_write_block(const uint32_t *__restrict__ bitmap, uint32_t words, uint32_t words_per_row, int nx,
+// bitmap: by the kernel before (no __restrict__: see wait_for_previous).
+__device__ void outlier_write_block(const uint32_t *bitmap, uint32_t words, uint32_t words_per_row, int nx,
                                     int ny, int nz, const float *__restrict__ x, uint32_t *out_idx, float *out_val,
                                     unsigned long long capacity, bool row_major, uint32_t b, unsigned long long start)
 {

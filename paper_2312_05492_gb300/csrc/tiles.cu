@@ -1294,7 +1294,8 @@ struct DBatch {
 };
 
 // The outliers (code 0) among a slab's landed codes: their values, which the
-// scatter kernel put into xrec, go into the box.  A thread tests groups of 8
+// scatter kernel put into xrec (plain loads: see wait_for_previous), go into the
+// box.  A thread tests groups of 8
 // codes (one 16-byte word) for a zero code.  DENSE (fields whose outliers exceed
 // 1/64 of the points): a group with a zero fetches its 8 values with two 16-byte
 // loads; otherwise each zero code fetches its own value, which keeps the loop
@@ -1324,22 +1325,22 @@ __device__ __forceinline__ void land_outliers(float *box, const uint16_t *land, 
             const size_t g = ((size_t)(sl.g0[0] + pz) * f.n[1] + sl.g0[1] + y) * f.n[2] + sl.g0[2] + 8 * q;
             float *brow = box + row * DP + 8 * q;
             if (F.a.vec_xrec && nj == 8) {
-                const float4 a = __ldg(reinterpret_cast<const float4 *>(F.a.xrec + g));
-                const float4 b = __ldg(reinterpret_cast<const float4 *>(F.a.xrec + g) + 1);
+                const float4 a = *reinterpret_cast<const float4 *>(F.a.xrec + g);
+                const float4 b = *(reinterpret_cast<const float4 *>(F.a.xrec + g) + 1);
                 const float vals[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
                     if (((wv[j >> 1] >> (16 * (j & 1))) & 0xffffu) == 0u) brow[j] = vals[j];
             } else {
                 for (int j = 0; j < nj; ++j)
-                    if (((wv[j >> 1] >> (16 * (j & 1))) & 0xffffu) == 0u) brow[j] = __ldg(F.a.xrec + g + j);
+                    if (((wv[j >> 1] >> (16 * (j & 1))) & 0xffffu) == 0u) brow[j] = F.a.xrec[g + j];
             }
         } else {
             for (int j = 0; j < nj; ++j) {
                 if (((wv[j >> 1] >> (16 * (j & 1))) & 0xffffu) == 0u) {
                     const size_t g =
                         ((size_t)(sl.g0[0] + pz) * f.n[1] + sl.g0[1] + y) * f.n[2] + sl.g0[2] + 8 * q + j;
-                    box[row * DP + 8 * q + j] = __ldg(F.a.xrec + g);
+                    box[row * DP + 8 * q + j] = F.a.xrec[g];
                 }
             }
         }
