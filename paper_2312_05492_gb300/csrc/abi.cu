@@ -357,7 +357,7 @@ int interp_decompress_batched_scheduled(const interp_decompress_item *items, int
                                                        gi::aligned16(it.d_xrec) && d.nx % 4 == 0, it.d_out_idx,
                                                        it.out_capacity};
     }
-    const bool early = small_fields(items, n);
+    const bool early = nsc > 0 && small_fields(items, n);
     // every field's stored outlier values in one launch, then one tile launch for the 3-D
     // fields and one per 1-D / 2-D field
     cudaError_t e = nsc > 0 ? gi::launch_outlier_scatter(sc, nsc, s) : cudaSuccess;
@@ -408,7 +408,7 @@ int interp_decompress_nd(int32_t ndim, const int64_t dims[3], const interp_heade
         const gi::ScatterItem sc{d_hdr, d_out_idx, d_out_val, out_capacity, d_xrec, points_of(dims)};
         e = gi::launch_outlier_scatter(&sc, 1, s);
     }
-    const bool early = gi::small_call((unsigned long long)dims[0] * dims[1] * dims[2]);
+    const bool early = out_capacity > 0 && gi::small_call((unsigned long long)dims[0] * dims[1] * dims[2]);
     const gi::DecompressArgs args{d, d_anchors, d_codes, d_xrec, d_hdr, false};
     if (e == cudaSuccess) {
         timing_mark(1, 0, s);
