@@ -158,6 +158,13 @@ __device__ __forceinline__ float code_to_q(uint32_t code, uint32_t cbias)
     return __uint_as_float(code + cbias) - kMagic;
 }
 
+// The item after s of n in steps of `step`, n when there is none: s + step itself may not fit
+// 32 bits (rows of one point are nearly 2^32 items).
+__host__ __device__ __forceinline__ uint32_t next_item(uint32_t s, uint32_t step, uint32_t n)
+{
+    return n - s > step ? s + step : n;
+}
+
 // Programmatic dependent launch.  A kernel launched by launch_after(early = true, ..) may be
 // set up, its CTAs waiting here, while the one before it in the stream still runs; it goes
 // on, and touches memory, only when that one is complete and its writes are visible.  Each

@@ -302,8 +302,9 @@ __global__ void __launch_bounds__(32 * RC.warps, RC.ctas) k_row_compress(const C
         land_values(land, a.x, g, vec, lane);
         if (g.x0 + SEG < nx) closing = __ldg(a.x + g.base + SEG);
     }
-    for (; s < segs; s += step) {
+    for (uint32_t next; s < segs; s = next) {
         const Seg g = seg_of(s, per_row, nx);
+        next = next_item(s, step, segs);
         cp_async_wait_all();
         __syncwarp();
         Lane L;
@@ -317,8 +318,8 @@ __global__ void __launch_bounds__(32 * RC.warps, RC.ctas) k_row_compress(const C
         }
         c.closing = closing;
         __syncwarp();
-        if (s + step < segs && s + step > s) {  // the next segment lands during the levels
-            const Seg n = seg_of(s + step, per_row, nx);
+        if (next < segs) {  // the next segment lands during the levels
+            const Seg n = seg_of(next, per_row, nx);
             land_values(land, a.x, n, vec, lane);
             if (n.x0 + SEG < nx) closing = __ldg(a.x + n.base + SEG);
         }
@@ -435,8 +436,9 @@ __global__ void __launch_bounds__(32 * RD.warps, RD.ctas) k_row_decompress(const
         land_codes(land, a.codes, g, width, lane);
         anc = anchor_of(g);
     }
-    for (; s < segs; s += step) {
+    for (uint32_t next; s < segs; s = next) {
         const Seg g = seg_of(s, per_row, nx);
+        next = next_item(s, step, segs);
         cp_async_wait_all();
         __syncwarp();
         Lane L;
@@ -451,8 +453,8 @@ __global__ void __launch_bounds__(32 * RD.warps, RD.ctas) k_row_decompress(const
         c.closing = __shfl_sync(0xffffffffu, anc, 31);
         L.v[0] = anc;
         __syncwarp();
-        if (s + step < segs && s + step > s) {
-            const Seg n = seg_of(s + step, per_row, nx);
+        if (next < segs) {
+            const Seg n = seg_of(next, per_row, nx);
             land_codes(land, a.codes, n, width, lane);
             anc = anchor_of(n);
         }
