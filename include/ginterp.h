@@ -325,7 +325,7 @@ uint64_t interp_huffman_chunks(uint64_t n);
 uint64_t interp_huffman_capacity_words(uint64_t n, int32_t max_len);
 
 /* Scratch for interp_huffman_encode / interp_huffman_decode of n codes (bytes; 0 for
- * a radius outside 2..32768 or n >= 2^32). */
+ * a radius outside 2..32768 or n >= 2^32).  d_ws is 4-byte aligned. */
 size_t interp_huffman_workspace_bytes(uint64_t n, int32_t radius);
 
 /* Encode n codes (each < 2R, every one with a nonzero length in d_lengths) with the

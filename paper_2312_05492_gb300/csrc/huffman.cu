@@ -669,7 +669,9 @@ bool huffman_codebook(const uint32_t *hist, int nsym, int max_len, uint8_t *leng
 }
 
 // A status word (8 bytes) per tile of 16 chunks; the size is stated as 4 bytes per 8
-// chunks, rounded up to 256 bytes, which always holds them.
+// chunks, rounded up to 256 bytes, which always holds them.  The words start after the
+// first 256 bytes, or 4 bytes earlier when the workspace is only 4-byte aligned (the first
+// 256 bytes hold the flag and, from 128 on, the tile counter).
 size_t huffman_encode_workspace(unsigned long long n)
 {
     const unsigned long long blocks = (huffman_chunks(n) + 7) / 8;
@@ -690,9 +692,9 @@ static cudaError_t launch_encode(const uint16_t *codes, unsigned long long n, co
     if (e != cudaSuccess) return e;
     const bool vec = (reinterpret_cast<uintptr_t>(codes) & 15u) == 0;
     const unsigned long long wave = 2ull * sm_count();
+    auto *status = reinterpret_cast<unsigned long long *>(reinterpret_cast<uintptr_t>(ws + 256) & ~(uintptr_t)7);
     k_huff_encode<SMEM_TAB><<<(unsigned)std::min(tiles, wave), ENC_THREADS, smem, s>>>(
-        codes, n, lengths, codewords, nsym, vec, reinterpret_cast<unsigned long long *>(ws + 256),
-        reinterpret_cast<unsigned int *>(ws + 128), (uint32_t)tiles, offsets, words, (uint32_t)nch, capacity_words,
+        codes, n, lengths, codewords, nsym, vec, status, reinterpret_cast<unsigned int *>(ws + 128), (uint32_t)tiles, offsets, words, (uint32_t)nch, capacity_words,
         reinterpret_cast<unsigned int *>(ws));
     return cudaGetLastError();
 }
