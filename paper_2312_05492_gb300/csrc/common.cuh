@@ -178,6 +178,15 @@ __device__ __forceinline__ void wait_for_previous()
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 }
 
+// Let a kernel's launches use up to `most` bytes of dynamic shared memory: the most that any
+// call asks for, not this call's size, which another thread's call could lower before this
+// one has launched.
+template <typename K>
+inline cudaError_t allow_smem(K kernel, size_t most)
+{
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // Launch a kernel that starts with wait_for_previous().  early only after a kernel of the
 // same call (what an earlier call wrote is then complete before this kernel starts), and
 // only while that leaves room on the SMs: CTAs that wait take the place of CTAs that work (512^3

@@ -37,6 +37,7 @@ constexpr int HCHUNK = 1024;          // codes per chunk
 constexpr int HLANE = HCHUNK / 32;    // codes per lane
 constexpr int ENC_WARPS = 16;         // chunks per tile
 constexpr int ENC_THREADS = 32 * ENC_WARPS;
+constexpr int ENC_SMEM_SYMS = 16384;  // symbols of a codebook kept in shared memory
 constexpr int MAX_LEN = 24;           // longest codeword the library builds
 constexpr int LUT_BITS = 12;          // lookup window: its table (32 KB) leaves two CTAs an SM
 constexpr int LUT_SYMS = 5;           // symbols of an entry
@@ -686,7 +687,8 @@ static cudaError_t launch_encode(const uint16_t *codes, unsigned long long n, co
 {
     const unsigned long long nch = huffman_chunks(n), tiles = (nch + ENC_WARPS - 1) / ENC_WARPS;
     const size_t smem = sizeof(uint32_t) * (ENC_WARPS * MAX_WORDS + (SMEM_TAB ? (size_t)nsym : 0));
-    cudaError_t e = cudaFuncSetAttribute(k_huff_encode<SMEM_TAB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e =
+        allow_smem(k_huff_encode<SMEM_TAB>, sizeof(uint32_t) * (ENC_WARPS * MAX_WORDS + (SMEM_TAB ? ENC_SMEM_SYMS : 0)));
     // flag and tile counter (the first 256 bytes) and the status words start at zero
     if (e == cudaSuccess) e = cudaMemsetAsync(ws, 0, 256 + 8 * tiles, s);
     if (e != cudaSuccess) return e;
@@ -694,8 +696,8 @@ static cudaError_t launch_encode(const uint16_t *codes, unsigned long long n, co
     const unsigned long long wave = 2ull * sm_count();
     auto *status = reinterpret_cast<unsigned long long *>(reinterpret_cast<uintptr_t>(ws + 256) & ~(uintptr_t)7);
     k_huff_encode<SMEM_TAB><<<(unsigned)std::min(tiles, wave), ENC_THREADS, smem, s>>>(
-        codes, n, lengths, codewords, nsym, vec, status, reinterpret_cast<unsigned int *>(ws + 128), (uint32_t)tiles, offsets, words, (uint32_t)nch, capacity_words,
-        reinterpret_cast<unsigned int *>(ws));
+        codes, n, lengths, codewords, nsym, vec, status, reinterpret_cast<unsigned int *>(ws + 128), (uint32_t)tiles,
+        offsets, words, (uint32_t)nch, capacity_words, reinterpret_cast<unsigned int *>(ws));
     return cudaGetLastError();
 }
 
@@ -709,11 +711,17 @@ cudaError_t launch_huffman_encode(const uint16_t *codes, unsigned long long n, c
         const cudaError_t e = cudaMemsetAsync(w, 0, sizeof(unsigned int), s);
         return e == cudaSuccess ? cudaMemsetAsync(offsets, 0, sizeof(uint32_t), s) : e;
     }
-    // the codebook sits in shared memory up to 16384 symbols (64 KB), beyond that it is
-    // read through the cache
-    if (nsym <= 16384)
+    // the codebook sits in shared memory up to ENC_SMEM_SYMS symbols (64 KB), beyond that it
+    // is read through the cache
+    if (nsym <= ENC_SMEM_SYMS)
         return launch_encode<true>(codes, n, lengths, codewords, nsym, offsets, words, capacity_words, w, s);
     return launch_encode<false>(codes, n, lengths, codewords, nsym, offsets, words, capacity_words, w, s);
+}
+
+// Shared memory of a decoding CTA: the lookup table, a code buffer and a ring per thread, the symbols.
+static constexpr size_t decode_smem(unsigned threads, int symbols)
+{
+    return sizeof(uint2) * (1 << LUT_BITS) + 2 * (size_t)DEC_PITCH * threads + sizeof(uint16_t) * (size_t)symbols;
 }
 
 template <int VEC>
@@ -722,8 +730,7 @@ static cudaError_t launch_decode(unsigned grid, unsigned threads, size_t smem, c
                                  const uint16_t *symbols, int nsym, int nsym_smem, uint16_t *codes,
                                  unsigned long long nch, unsigned int *bad)
 {
-    const cudaError_t e =
-        cudaFuncSetAttribute(k_huff_decode<VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(k_huff_decode<VEC>, decode_smem(DEC_THREADS, SYM_SMEM));
     if (e != cudaSuccess) return e;
     // the tables kernel is one CTA
     return launch_after(true, k_huff_decode<VEC>, grid, threads, smem, s, words, offsets, n, t, symbols, nsym, nsym_smem,
@@ -746,7 +753,7 @@ cudaError_t launch_huffman_decode(const uint32_t *words, const uint32_t *offsets
     const unsigned threads = (unsigned)std::min<unsigned long long>(DEC_THREADS, std::max<unsigned long long>(128, (per + 31) / 32 * 32));
     const unsigned grid = (unsigned)((nch + threads - 1) / threads);
     const int nsym_smem = nsym <= SYM_SMEM ? nsym : 0;
-    const size_t smem = sizeof(uint2) * (1 << LUT_BITS) + 2 * (size_t)DEC_PITCH * threads + 2 * (size_t)nsym_smem;
+    const size_t smem = decode_smem(threads, nsym_smem);
     const uintptr_t a = reinterpret_cast<uintptr_t>(codes);
     if ((a & 31u) == 0)
         return launch_decode<32>(grid, threads, smem, s, words, offsets, n, t, symbols, nsym, nsym_smem, codes, nch, bad);

@@ -503,12 +503,12 @@ __global__ void __launch_bounds__(32 * RD.warps, RD.ctas) k_row_decompress(const
 uint32_t segments_per_row(Dims d) { return (uint32_t)(((long long)d.nx + SEG - 1) / SEG); }
 
 template <typename K, typename A>
-cudaError_t launch_rows(K kernel, Shape shape, const A &a, size_t smem, bool early, cudaStream_t s)
+cudaError_t launch_rows(K kernel, Shape shape, const A &a, size_t smem, size_t most, bool early, cudaStream_t s)
 {
     // segments are fewer than 2^32 (N is), and a grid of one wave takes them in turn
     const uint32_t per_row = segments_per_row(a.dims);
     const unsigned long long segs = (unsigned long long)a.dims.nz * a.dims.ny * per_row;
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(kernel, most);
     if (e != cudaSuccess) return e;
     const unsigned long long wave = (unsigned long long)sm_count() * shape.ctas;
     return launch_after(early, kernel, (unsigned)(segs < wave ? segs : wave), 32 * shape.warps, smem, s, a, per_row,
@@ -519,13 +519,15 @@ cudaError_t launch_rows(K kernel, Shape shape, const A &a, size_t smem, bool ear
 
 cudaError_t launch_row_compress(const CompressArgs &a, bool early, cudaStream_t s)
 {
-    if (2 * a.radius > R_HIST_BINS) return launch_rows(k_row_compress<ENCODE_GBINS>, RC, a, R_HIST, early, s);
-    return launch_rows(k_row_compress<ENCODE>, RC, a, R_HIST + sizeof(uint32_t) * 2 * (size_t)a.radius, early, s);
+    if (2 * a.radius > R_HIST_BINS) return launch_rows(k_row_compress<ENCODE_GBINS>, RC, a, R_HIST, R_HIST, early, s);
+    return launch_rows(k_row_compress<ENCODE>, RC, a, R_HIST + sizeof(uint32_t) * 2 * (size_t)a.radius,
+                       R_HIST + sizeof(uint32_t) * R_HIST_BINS, early, s);
 }
 
 cudaError_t launch_row_decompress(const DecompressArgs &a, bool early, cudaStream_t s)
 {
-    return launch_rows(k_row_decompress, RD, a, R_WARPS + R_WARP * RD.warps, early, s);
+    constexpr size_t smem = R_WARPS + R_WARP * RD.warps;
+    return launch_rows(k_row_decompress, RD, a, smem, smem, early, s);
 }
 
 }  // namespace gi

@@ -791,9 +791,9 @@ Plan plan_of(Dims d, unsigned long long warps)
 }
 
 template <typename K, typename Args>
-cudaError_t launch_planes(K kernel, const Args &a, size_t smem, bool early, cudaStream_t s)
+cudaError_t launch_planes(K kernel, const Args &a, size_t smem, size_t most, bool early, cudaStream_t s)
 {
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(kernel, most);
     if (e != cudaSuccess) return e;
     const uint32_t wave = (uint32_t)(sm_count() * P_CTAS);
     const Plan p = plan_of(a.dims, (unsigned long long)wave * PW);
@@ -804,13 +804,14 @@ cudaError_t launch_planes(K kernel, const Args &a, size_t smem, bool early, cuda
 
 cudaError_t launch_plane_compress(const CompressArgs &a, bool early, cudaStream_t s)
 {
-    if (2 * a.radius > P_HIST_BINS) return launch_planes(k_plane_compress<ENCODE_GBINS>, a, P_HIST, early, s);
-    return launch_planes(k_plane_compress<ENCODE>, a, P_HIST + sizeof(uint32_t) * 2 * (size_t)a.radius, early, s);
+    if (2 * a.radius > P_HIST_BINS) return launch_planes(k_plane_compress<ENCODE_GBINS>, a, P_HIST, P_HIST, early, s);
+    return launch_planes(k_plane_compress<ENCODE>, a, P_HIST + sizeof(uint32_t) * 2 * (size_t)a.radius,
+                         P_HIST + sizeof(uint32_t) * P_HIST_BINS, early, s);
 }
 
 cudaError_t launch_plane_decompress(const DecompressArgs &a, bool early, cudaStream_t s)
 {
-    return launch_planes(k_plane_decompress, a, P_HIST, early, s);
+    return launch_planes(k_plane_decompress, a, P_HIST, P_HIST, early, s);
 }
 
 }  // namespace gi

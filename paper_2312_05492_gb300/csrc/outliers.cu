@@ -391,7 +391,7 @@ cudaError_t launch_histogram(const uint16_t *codes, uint64_t n, int radius, uint
     const int bins = 2 * radius;
     const size_t smem = bins <= HIST_SMEM_MAX_BINS ? sizeof(uint32_t) * (size_t)bins : 0;
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_histogram, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(k_histogram, sizeof(uint32_t) * HIST_SMEM_MAX_BINS);
         if (e != cudaSuccess) return e;
     }
     const int vec = (reinterpret_cast<uintptr_t>(codes) % 16) == 0;

@@ -1536,7 +1536,7 @@ cudaError_t prepare(K kernel, int threads, size_t smem, int *cache, int &grid)
         grid = cache[dev];
         return cudaSuccess;
     }
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_smem(kernel, smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);

@@ -122,3 +122,18 @@ def test_data_of_the_kernel_before_is_not_declared_read_only(name, function, par
 def test_scattered_values_are_read_by_plain_loads():
     for name in ("tiles.cu", "nd1.cu", "nd2.cu"):
         assert not re.search(r"__ld\w+\([^;]*xrec", _source(name)), name
+
+
+def test_shared_memory_limits_do_not_depend_on_the_call():
+    """A limit set to one call's size could be lowered by another thread's call before the
+    first has launched: kernels' limits are set in one place, to sizes known at compile time."""
+    for name in ("tiles.cu", "nd1.cu", "nd2.cu", "huffman.cu", "outliers.cu", "profile.cu", "quality.cu"):
+        text = _source(name)
+        assert "MaxDynamicSharedMemorySize" not in text, name
+        for most in re.findall(r"allow_smem\([^,]+,\s*(.+?)\);", text, re.S):
+            assert not re.search(r"\b(radius|nsym|n|threads|bins)\b", most), (name, most)
+    for name, function in (("nd1.cu", "launch_rows"), ("nd2.cu", "launch_planes")):
+        calls = re.findall(r"return " + function + r"\((.+?)\);", _source(name), re.S)
+        assert len(calls) == 3
+        for c in calls:
+            assert "radius" not in c.split(",")[-3], c  # the limit; then early and the stream
