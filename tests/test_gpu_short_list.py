@@ -1,6 +1,6 @@
 """A field with more outliers than its list has room for: the reconstruction does not depend
-on what the output buffer held, and is the oracle's from the same short list (an outlier
-that is not listed is 0), in every geometry, alignment and call form."""
+on what the output buffer held, and is the oracle's with 0 in the place of the outliers that
+are not listed, in every geometry, alignment and call form."""
 import dataclasses
 
 import numpy as np
@@ -27,7 +27,9 @@ def _noise(shape, seed):
 
 
 def _expected(oc, cap):
-    return bits(O.decompress(dataclasses.replace(oc, out_idx=oc.out_idx[:cap], out_val=oc.out_val[:cap])))
+    val = oc.out_val.copy()
+    val[cap:] = 0
+    return bits(O.decompress(dataclasses.replace(oc, out_val=val)))
 
 
 @pytest.mark.parametrize("ndim,shape", [(3, (17, 33, 64)), (3, (9, 18, 35)), (3, (49, 49, 49)), (2, (2, 33, 72)),
