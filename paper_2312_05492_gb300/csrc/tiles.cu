@@ -45,6 +45,13 @@ constexpr int CNT = 128, CNT_WIDE = 192, DNT = 192;
 // The passes' template parameter COMPRESS: threads of the compression kernel, 0 for decompression.
 template <int COMPRESS>
 constexpr int kThreads = COMPRESS ? COMPRESS : DNT;
+// The wide kernel has 64 registers a thread.  What the slab loop derives from threadIdx.x is
+// computed where it is used there (thread_id): kept through the passes it was spilled (48 bytes
+// a thread, and the reloads miss an L1 cache that shared memory leaves little of), which cost
+// the x-extended domain at 512^3 4 - 7% (650 -> 609 us, 554 -> 515 us; orders 021 and 102).
+// The others have registers for it (449x449x235: 261 us, 277 without).
+template <int NT>
+constexpr bool kOwnIds = NT == CNT_WIDE;
 constexpr int EZ = 9, EY = OY + 1, EX = OX + 1;  // slab box extents (z, y, x)
 // Floats per box row and plane.  Compression works where the TMA landed the values, so its
 // rows are whole 16-byte groups: an odd number of them, so that a warp's 16-byte reads of
@@ -782,16 +789,18 @@ template <int COMPRESS>
 __device__ __forceinline__ void run_slab(float *box, const Sink &sk, const Slab &sl, const Field &f,
                                          const Levels &lv)
 {
-    // compression: the fixed-geometry passes keep every code's bin in shared memory
-    const bool general = lv.xdom32 || (COMPRESS && 2 * lv.R > HIST_SMEM_BINS);
-    if (general)
-        passes_general<COMPRESS>(sl, f, sk.hist_g);  // box and sink at their fixed offsets
-    else
-        passes_fast<COMPRESS>((int)((COMPRESS ? reinterpret_cast<const unsigned char *>(sk.stage)
-                                              : reinterpret_cast<const unsigned char *>(sk.cbox)) -
-                                    g_smem),
-                              f.n[0] - 1 - sl.g0[0], f.n[1] - 1 - sl.g0[1], f.n[2] - 1 - sl.g0[2], sl.lim[0],
-                              sl.lim[1], sl.lim[2], sl.carried);
+    if constexpr (COMPRESS == 0 || COMPRESS == CNT_WIDE) {  // the launch takes the wide kernel for them
+        // compression: the fixed-geometry passes keep every code's bin in shared memory
+        if (lv.xdom32 || (COMPRESS && 2 * lv.R > HIST_SMEM_BINS)) {
+            passes_general<COMPRESS>(sl, f, sk.hist_g);  // box and sink at their fixed offsets
+            return;
+        }
+    }
+    passes_fast<COMPRESS>((int)((COMPRESS ? reinterpret_cast<const unsigned char *>(sk.stage)
+                                          : reinterpret_cast<const unsigned char *>(sk.cbox)) -
+                                g_smem),
+                          f.n[0] - 1 - sl.g0[0], f.n[1] - 1 - sl.g0[1], f.n[2] - 1 - sl.g0[2], sl.lim[0],
+                          sl.lim[1], sl.lim[2], sl.carried);
 }
 
 // ------------------------------------------------------------ work list
@@ -838,11 +847,21 @@ __device__ __forceinline__ void slab_next(SlabState &nx, const SlabState &st, co
     }
 }
 
+// threadIdx.x; OWN: as a value of its own at each use, so that what a part of the slab loop
+// derives from it is computed there and not kept in registers through the passes.
+template <bool OWN>
+__device__ __forceinline__ int thread_id()
+{
+    int t = (int)threadIdx.x;
+    if constexpr (OWN) asm volatile("" : "+r"(t));
+    return t;
+}
+
 // Bring the NPL x 17 x XP (or KP) input box of a slab into shared memory:
 // one TMA box (thread 0; out-of-field elements are zero-filled), or, when the
 // field's rows cannot be described by a tensor map, 4-byte cp.async copies
 // of the in-field elements by all threads.
-template <typename T, int P, int NPL, int Z0, int NT>
+template <typename T, int P, int NPL, int Z0, int NT, bool OWN>
 __device__ __forceinline__ void issue_land(T *land, const T *__restrict__ src, const CUtensorMap *map, bool use_tma,
                                            uint64_t *bar, const Field &f, const Slab &s)
 {
@@ -855,7 +874,7 @@ __device__ __forceinline__ void issue_land(T *land, const T *__restrict__ src, c
         return;
     }
     // a warp takes whole rows, all planes of one row at a time; the closing column apart
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int tid = thread_id<OWN>(), lane = tid & 31, warp = tid >> 5;
     const int nzp = min(NPL, f.n[0] - s.g0[0] - Z0);
     const int nyr = min(EY, f.n[1] - s.g0[1]);
     const int nxc = min(EX, f.n[2] - s.g0[2]);
@@ -879,7 +898,7 @@ __device__ __forceinline__ void issue_land(T *land, const T *__restrict__ src, c
         }
     }
     if (nxc > OX)
-        for (int r = NT - 1 - (int)threadIdx.x; r < NPL * EY; r += NT) {
+        for (int r = NT - 1 - tid; r < NPL * EY; r += NT) {
             const int pz = r / EY, y = r - pz * EY;
             if (pz >= nzp || y >= nyr) continue;
             const T *one = src0 + pz * plane + (size_t)y * f.n[2] + OX;
@@ -950,10 +969,11 @@ __device__ __forceinline__ void flush_hist(const CField &F, uint32_t *hist_s)
 
 // The slab's anchors (planes 0 and 8 as far as the slab owns them), lossless.  They are
 // never modified, so they are stored while the box still holds the input.
+template <int NT>
 __device__ __forceinline__ void write_anchors(const CField &F, const CWrite &cw, const Slab &sl, const float *box)
 {
     constexpr int AY = OY / 8, AX = OX / 8;
-    const int t = threadIdx.x;
+    const int t = NT - 1 - thread_id<kOwnIds<NT>>();  // the last warp: the coarse passes keep the first ones busy
     if (t >= 2 * AY * AX) return;
     const int pz = 8 * (t / (AY * AX)), y = 8 * (t / AX % AY), x = 8 * (t % AX);
     if (pz < sl.own_lo || pz >= sl.lim[0] || y >= sl.lim[1] || x >= sl.lim[2]) return;
@@ -971,8 +991,8 @@ __device__ __forceinline__ void write_slab_fast(const CField &F, const CWrite &c
     const Field &f = F.f;
     static_assert(NT % 4 == 0 && (NT / 4) % OY == 0, "steps cover whole planes");
     constexpr int PSTEP = NT / 4 / OY;  // planes per step
-    const int sub = threadIdx.x & 3;
-    int r = threadIdx.x >> 2;
+    const int tid = thread_id<kOwnIds<NT>>(), sub = tid & 3;
+    int r = tid >> 2;
     const int y = r % OY;
     int pz = sl.own_lo + r / OY;
     const size_t plane = (size_t)f.n[1] * f.n[2];
@@ -988,7 +1008,7 @@ __device__ __forceinline__ void write_slab_fast(const CField &F, const CWrite &c
     }
     // the slab's bitmap words are contiguous (16 per plane, tile-major layout)
     uint32_t *wb = F.a.bitmap + ((size_t)sl.col * f.n[0] + sl.g0[0] + sl.own_lo) * OY;
-    if ((int)threadIdx.x < rows / 4) reinterpret_cast<uint4 *>(wb)[threadIdx.x] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid < rows / 4) reinterpret_cast<uint4 *>(wb)[tid] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 // Rows that are not 16-byte aligned: a warp stores one row per step, one code per lane
@@ -1111,7 +1131,7 @@ __device__ __forceinline__ void write_slab_general(const CField &F, const CWrite
                                                    const uint16_t *stage)
 {
     const Field &f = F.f;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int tid = thread_id<kOwnIds<NT>>(), lane = tid & 31, warp = tid >> 5;
     const int sub = lane & 3;
     for (int base = warp * 8; base < rows; base += (NT / 32) * 8) {
         const int row = base + (lane >> 2);
@@ -1202,7 +1222,7 @@ __global__ void __launch_bounds__(NT, TMA ? kCompressCtas : kCompressCtas - 1)
     uint32_t out_seen = 0;  // outliers in the shared histogram before the current slab
     {
         const CField &F = B.fld[st[0].fi];
-        issue_land<float, XP, XPL, 1, NT>(land, F.a.x, &B.map[st[0].fi], TMA || F.use_tma, bar, F.f, st[0].s);
+        issue_land<float, XP, XPL, 1, NT, kOwnIds<NT>>(land, F.a.x, &B.map[st[0].fi], TMA || F.use_tma, bar, F.f, st[0].s);
     }
     for (;;) {
         const Slab &sl = st[cur].s;
@@ -1220,7 +1240,7 @@ __global__ void __launch_bounds__(NT, TMA ? kCompressCtas : kCompressCtas - 1)
         if (!sl.carried) {
             const int nyr = min(EY, f.n[1] - sl.g0[1]), nxc = min(EX, f.n[2] - sl.g0[2]);
             const float *src = F.a.x + ((size_t)sl.g0[0] * f.n[1] + sl.g0[1]) * f.n[2] + sl.g0[2];
-            for (int i = threadIdx.x; i < EY * EX; i += NT) {
+            for (int i = thread_id<kOwnIds<NT>>(); i < EY * EX; i += NT) {
                 const int y = i / EX, xx = i - y * EX;
                 if (y < nyr && xx < nxc) box[y * XP + xx] = __ldg(src + (size_t)y * f.n[2] + xx);
             }
@@ -1229,7 +1249,7 @@ __global__ void __launch_bounds__(NT, TMA ? kCompressCtas : kCompressCtas - 1)
         __syncthreads();  // box and levels ready; the previous slab's staged codes are written out
         if (abort_flag) break;
         const CWrite cw = cwrite_of(F);
-        write_anchors(F, cw, sl, box);
+        write_anchors<NT>(F, cw, sl, box);
 
         run_slab<NT>(box, Sink{stage, nullptr, hist_s, F.a.hist}, sl, f, lv);  // ends with a barrier
 
@@ -1241,13 +1261,13 @@ __global__ void __launch_bounds__(NT, TMA ? kCompressCtas : kCompressCtas - 1)
         // ---- plane 8 carried into plane 0 when the next slab continues this run; then the
         // next slab's input, which lands while this slab's codes are written out
         if (has_next && nx.s.carried)
-            for (int i = threadIdx.x; i < PLANE / 4; i += NT)
+            for (int i = thread_id<kOwnIds<NT>>(); i < PLANE / 4; i += NT)
                 reinterpret_cast<float4 *>(box)[i] = reinterpret_cast<const float4 *>(box + 8 * PLANE)[i];
         __syncthreads();
         if (has_next) {
             const int nfi = nx.fi;
             const CField &N = B.fld[nfi];
-            issue_land<float, XP, XPL, 1, NT>(land, N.a.x, &B.map[nfi], TMA || N.use_tma, bar, N.f, nx.s);
+            issue_land<float, XP, XPL, 1, NT, kOwnIds<NT>>(land, N.a.x, &B.map[nfi], TMA || N.use_tma, bar, N.f, nx.s);
         }
         // ---- owned planes: codes and outlier-bitmap words
         const int planes = sl.lim[0] - sl.own_lo;
@@ -1415,7 +1435,7 @@ __global__ void __launch_bounds__(DNT, kDecompressCtas) k_decompress(const __gri
     bool anc_ok;
     {
         const DField &F = B.fld[st[0].fi];
-        issue_land<uint16_t, KP, EZ, 0, DNT>(land, F.a.codes, &B.map[st[0].fi], F.use_tma, bar, F.f, st[0].s);
+        issue_land<uint16_t, KP, EZ, 0, DNT, false>(land, F.a.codes, &B.map[st[0].fi], F.use_tma, bar, F.f, st[0].s);
         anc_ok = anchor_fetch(F, st[0].s, anc);
         if (threadIdx.x == DNT - 1) slab_next(st[1], st[0], bv);
         __syncthreads();
@@ -1459,7 +1479,7 @@ __global__ void __launch_bounds__(DNT, kDecompressCtas) k_decompress(const __gri
         if (has_next) {
             const int nfi = nx.fi;
             const DField &N = B.fld[nfi];
-            issue_land<uint16_t, KP, EZ, 0, DNT>(land, N.a.codes, &B.map[nfi], N.use_tma, bar, N.f, nx.s);
+            issue_land<uint16_t, KP, EZ, 0, DNT, false>(land, N.a.codes, &B.map[nfi], N.use_tma, bar, N.f, nx.s);
         }
 
         // ---- write the owned planes
@@ -1621,7 +1641,7 @@ cudaError_t launch_compress_tiles(const CompressArgs *args, int n, bool early, c
     bool tma = true, general = false;
     long long slabs = 0;
     for (int i = 0; i < n; ++i) {
-        const uint32_t box[3] = {XP, EY, XPL};  // planes 1..8 of a slab: must match issue_land<float, XP, XPL, 1, NT>
+        const uint32_t box[3] = {XP, EY, XPL};  // planes 1..8 of a slab: must match issue_land<float, XP, XPL, 1, ..>
         B.fld[i].use_tma =
             encode_tensor_map_3d(&B.map[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, args[i].x, args[i].dims, box) ? 1 : 0;
         tma = tma && B.fld[i].use_tma;
