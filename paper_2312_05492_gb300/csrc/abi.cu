@@ -97,14 +97,13 @@ double effective_alpha(const interp_config &c, double eb)
     return c.eb_mode ? alpha_of_eps(eb) : 1.0;
 }
 
-// Codes per store for rows of 8 codes starting at multiples of 8 along x: the
-// widest store whose alignment every such row start keeps.
+// Codes per store for rows of 8 codes starting at multiples of 8 along x: 8 or 4 where every
+// such row start keeps the alignment, else 1.
 int code_store_width(const void *codes, int nx)
 {
     const uintptr_t a = reinterpret_cast<uintptr_t>(codes);
     if (a % 16 == 0 && nx % 8 == 0) return 8;
     if (a % 8 == 0 && nx % 4 == 0) return 4;
-    if (a % 4 == 0 && nx % 2 == 0) return 2;
     return 1;
 }
 

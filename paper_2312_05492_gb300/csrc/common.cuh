@@ -225,8 +225,8 @@ struct CompressArgs {
     int radius;
     interp_header *hdr;
     bool xdom32;     // x-extended neighbour domain requested (cfg.domain_x == 32)
-    int code_store;  // codes per store on rows of 8 codes starting at x = 8k: 8, 4 or 2
-                     // (by the alignment of codes and nx), else 1
+    int code_store;  // codes per store on rows of 8 codes starting at x = 8k: 8 or 4 (by the
+                     // alignment of codes and nx), else 1
 };
 
 struct DecompressArgs {

@@ -1011,7 +1011,7 @@ __device__ __forceinline__ void write_slab_fast(const CField &F, const CWrite &c
     if (tid < rows / 4) reinterpret_cast<uint4 *>(wb)[tid] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-// Rows that are not 16-byte aligned: a warp stores one row per step, one code per lane
+// Rows that are not 8-byte aligned: a warp stores one row per step, one code per lane
 // (consecutive addresses, whatever their alignment; 4 lanes x 8 codes per row had made
 // every 2-byte store touch 32 sectors); the row's outlier word is a ballot.
 // Out of line: inlined, it made the aligned fields' loop 1% slower.
@@ -1123,9 +1123,9 @@ __device__ __noinline__ void write_slab_outliers(const CField &F, int R, int WX,
     }
 }
 
-// Any other slab with 16-byte aligned code rows: codes and the exact
-// outlier-bitmap words with their block counts.  A warp takes 8 consecutive
-// rows of one plane, 4 lanes x 8 codes per row.
+// Any other slab with 16-byte aligned code rows, and all with 8-byte aligned ones
+// (300x512x516: 263 us, a row a warp 334): codes and the exact outlier-bitmap words with their block counts.  A
+// warp takes 8 consecutive rows of one plane, 4 lanes x 8 codes per row.
 template <int NT>
 __device__ __forceinline__ void write_slab_general(const CField &F, const CWrite &cw, const Slab &sl, int rows,
                                                    const uint16_t *stage)
@@ -1148,8 +1148,11 @@ __device__ __forceinline__ void write_slab_general(const CField &F, const CWrite
         }
         const size_t gi = ((size_t)gz * f.n[1] + gy) * f.n[2] + gx;
         if (((pz | y) & 7) == 0) w[0] = (w[0] & 0xffff0000u) | (uint32_t)cw.R;  // anchor at x = 8*sub (Sec. IV-A)
-        if (nvalid == 8) {
+        if (nvalid == 8 && cw.code_store == 8) {
             *reinterpret_cast<uint4 *>(F.a.codes + gi) = make_uint4(w[0], w[1], w[2], w[3]);
+        } else if (nvalid == 8) {
+            reinterpret_cast<uint2 *>(F.a.codes + gi)[0] = make_uint2(w[0], w[1]);
+            reinterpret_cast<uint2 *>(F.a.codes + gi)[1] = make_uint2(w[2], w[3]);
         } else {
 #pragma unroll
             for (int j = 0; j < 8; ++j)
@@ -1275,7 +1278,7 @@ __global__ void __launch_bounds__(NT, TMA ? kCompressCtas : kCompressCtas - 1)
             write_slab_fast<NT>(F, cw, sl, planes * OY, stage);
         else if (cw.code_store == 8 && sl.lim[1] == OY && sl.lim[2] == OX)
             write_slab_outliers<NT>(F, cw.R, cw.WX, sl.g0[0], sl.g0[1], sl.g0[2], sl.col, sl.own_lo, planes * OY);
-        else if (cw.code_store == 8)
+        else if (cw.code_store >= 4)
             write_slab_general<NT>(F, cw, sl, planes * OY, stage);
         else
             write_slab_rows<NT>(F, cw, sl.g0[0], sl.g0[1], sl.g0[2], sl.col, sl.own_lo, planes);
