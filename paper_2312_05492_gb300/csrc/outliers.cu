@@ -36,9 +36,17 @@ __device__ void fill_central_bin(uint32_t *hist, int radius, unsigned long long 
 {
     __shared__ unsigned long long part[T / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned long long others = 0;
-    for (int c = threadIdx.x; c < 2 * radius; c += T)
-        if (c != radius) others += hist[c];
+    // bin R, taken off at the start
+    unsigned long long others = threadIdx.x == 0 ? 0ull - hist[radius] : 0ull;
+    // 16-byte loads, several in flight a thread: a block reads up to 65536 bins
+    const int n4 = (reinterpret_cast<uintptr_t>(hist) & 15u) == 0 ? 2 * radius / 4 : 0;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n4; i += T) {
+        const uint4 v = reinterpret_cast<const uint4 *>(hist)[i];
+        others += (unsigned long long)v.x + v.y + v.z + v.w;
+    }
+#pragma unroll 1
+    for (int c = 4 * n4 + threadIdx.x; c < 2 * radius; c += T) others += hist[c];
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) others += __shfl_xor_sync(0xffffffffu, others, off);
     __syncthreads();
