@@ -25,6 +25,12 @@ constexpr int WRITE_THREADS = 256;
 constexpr int WRITE_WARPS = WRITE_THREADS / 32;
 constexpr int WORDS_PER_THREAD = BITMAP_BLOCK_WORDS / WRITE_THREADS;  // 8
 constexpr uint32_t WRITE_LIST = 6144;  // indices expanded at a time (24 KB)
+// A block with more outliers (28% of its points) is written word by word, a warp a word and a
+// lane a point: the list is expanded by the threads whose words it holds at a time, 24 of 256
+// when every point is an outlier.  92% of 64^3 points 137 -> 38 us, of 512^3 502 -> 375 us;
+// 21% of 3 x 1001 x 1003: 80 us by the list, 98 word by word; 33% of 512^3: 212 and 237.
+constexpr uint32_t WRITE_DENSE = 3 * WRITE_LIST;
+static_assert(WRITE_LIST == 3 * BITMAP_BLOCK_WORDS, "three values of every word of a block fit the list's room");
 // up to here (a field of about 2^28 points) a CTA adds up at most 4096 counters (16 a
 // thread, from L2), which costs less than the scan's launch (5 us on 512^3 points)
 constexpr int SELF_SCAN_BLOCKS = 4096;
@@ -103,23 +109,26 @@ __device__ void outlier_scan_block(uint32_t *blockcnt, int nblk, interp_header *
     if (hist) fill_central_bin<SCAN_THREADS>(hist, radius, n);
 }
 
-// The outliers of bitmap block b of a field, written from position `start` of its list on.
-// bitmap: by the kernel before (no __restrict__: see wait_for_previous).
-__device__ void outlier_write_block(const uint32_t *bitmap, uint32_t words, uint32_t words_per_row, int nx,
-                                    int ny, int nz, const float *__restrict__ x, uint32_t *out_idx, float *out_val,
-                                    unsigned long long capacity, bool row_major, uint32_t b, unsigned long long start)
-{
-    __shared__ uint32_t warp_sum[WRITE_WARPS];
-    __shared__ uint32_t list[WRITE_LIST];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t w0 = b * (uint32_t)BITMAP_BLOCK_WORDS + (uint32_t)(threadIdx.x * WORDS_PER_THREAD);
+// Block-wide room of the write kernel: the list, and the warps' counts.
+__shared__ uint32_t w_list[WRITE_LIST];
+__shared__ uint32_t w_sum[WRITE_WARPS];
+
+// A thread's words (from w0 on), the outliers in them, those before them in the block, and the
+// block's.
+struct Words {
     uint32_t wv[WORDS_PER_THREAD];
+    uint32_t pos, total;
+};
+__device__ __forceinline__ void load_words(Words &W, const uint32_t *bitmap, uint32_t words, uint32_t words_per_row, int ny,
+                                           int nz, bool row_major, uint32_t w0)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t cnt = 0;
 #pragma unroll
     for (int k = 0; k < WORDS_PER_THREAD; ++k) {
         const uint32_t w = w0 + k;
-        wv[k] = w < words ? bitmap[row_major ? (size_t)w : tiled_word(w, words_per_row, ny, nz)] : 0u;
-        cnt += __popc(wv[k]);
+        W.wv[k] = w < words ? bitmap[row_major ? (size_t)w : tiled_word(w, words_per_row, ny, nz)] : 0u;
+        cnt += __popc(W.wv[k]);
     }
     // block exclusive scan of the threads' counts
     uint32_t incl = cnt;
@@ -128,14 +137,28 @@ __device__ void outlier_write_block(const uint32_t *bitmap, uint32_t words, uint
         const uint32_t y = __shfl_up_sync(0xffffffffu, incl, off);
         if (lane >= off) incl += y;
     }
-    if (lane == 31) warp_sum[warp] = incl;
+    if (lane == 31) w_sum[warp] = incl;
     __syncthreads();
-    uint32_t pos = incl - cnt, total = 0;
+    W.pos = incl - cnt;
+    W.total = 0;
 #pragma unroll
     for (int w = 0; w < WRITE_WARPS; ++w) {
-        if (w < warp) pos += warp_sum[w];
-        total += warp_sum[w];
+        if (w < warp) W.pos += w_sum[w];
+        W.total += w_sum[w];
     }
+}
+
+// The outliers of bitmap block b of a field, written from position `start` of its list on.
+// bitmap: by the kernel before (no __restrict__: see wait_for_previous).
+__device__ void outlier_write_block(const uint32_t *bitmap, uint32_t words, uint32_t words_per_row, int nx,
+                                    int ny, int nz, const float *__restrict__ x, uint32_t *out_idx, float *out_val,
+                                    unsigned long long capacity, bool row_major, uint32_t b, unsigned long long start)
+{
+    const uint32_t w0 = b * (uint32_t)BITMAP_BLOCK_WORDS + (uint32_t)(threadIdx.x * WORDS_PER_THREAD);
+    Words W;
+    load_words(W, bitmap, words, words_per_row, ny, nz, row_major, w0);
+    uint32_t *list = w_list, (&wv)[WORDS_PER_THREAD] = W.wv, pos = W.pos;
+    const uint32_t total = W.total;
     for (uint32_t from = 0; from < total; from += WRITE_LIST) {
         const uint32_t n = min(WRITE_LIST, total - from);
         // this thread's outliers at positions [from, from + n); their bits are cleared
@@ -184,6 +207,48 @@ struct CompactField {
     int scanned;     // blockcnt holds offsets (k_outlier_scan), not counts
 };
 
+// outlier_write_block for a block of many outliers.  Out of line: its registers are not the list's.
+__device__ __noinline__ void outlier_write_dense(const CompactField &F, uint32_t b, unsigned long long start)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t i0 = (uint32_t)(threadIdx.x * WORDS_PER_THREAD), w0 = b * (uint32_t)BITMAP_BLOCK_WORDS + i0;
+    uint32_t *bits = w_list, *at = w_list + BITMAP_BLOCK_WORDS, *first = w_list + 2 * BITMAP_BLOCK_WORDS;
+    Words W;
+    load_words(W, F.bitmap, F.words, F.words_per_row, F.ny, F.nz, F.row_major, w0);
+#pragma unroll
+    for (int k = 0; k < WORDS_PER_THREAD; ++k) {
+        const uint32_t w = w0 + k, row = w / F.words_per_row;
+        bits[i0 + k] = W.wv[k];
+        at[i0 + k] = W.pos;
+        first[i0 + k] = row * (uint32_t)F.nx + (w - row * F.words_per_row) * 32u;
+        W.pos += __popc(W.wv[k]);
+    }
+    __syncthreads();
+    const uint32_t room = (uint32_t)min((unsigned long long)W.total, F.capacity - start);
+    const float *__restrict__ x = F.x;
+    uint32_t *out_idx = F.out_idx + start;
+    float *out_val = F.out_val + start;
+    constexpr int AT_ONCE = 4;  // words of a warp whose values are on their way together
+    static_assert(BITMAP_BLOCK_WORDS % (AT_ONCE * WRITE_WARPS) == 0, "whole rounds");
+    for (int i = warp; i < BITMAP_BLOCK_WORDS; i += AT_ONCE * WRITE_WARPS) {
+        uint32_t p[AT_ONCE], idx[AT_ONCE];
+        float v[AT_ONCE];
+#pragma unroll
+        for (int j = 0; j < AT_ONCE; ++j) {
+            const uint32_t m = bits[i + j * WRITE_WARPS];
+            idx[j] = first[i + j * WRITE_WARPS] + lane;
+            p[j] = (m >> lane & 1u) ? at[i + j * WRITE_WARPS] + __popc(m & ((1u << lane) - 1u)) : room;
+            v[j] = p[j] < room ? __ldg(x + idx[j]) : 0.0f;
+        }
+#pragma unroll
+        for (int j = 0; j < AT_ONCE; ++j)
+            if (p[j] < room) {
+                out_idx[p[j]] = idx[j];
+                out_val[p[j]] = v[j];
+            }
+    }
+}
+
 struct CompactBatch {
     CompactField f[kMaxBatch];
     int n;
@@ -204,13 +269,15 @@ __global__ void __launch_bounds__(WRITE_THREADS) k_outlier_write(const __grid_co
     const CompactField &F = B.f[fi];
     const int b = (int)blockIdx.x - F.b0;
     unsigned long long start;
+    uint32_t own;
     if (F.scanned) {
         start = F.blockcnt[b];
         const unsigned long long end = b + 1 < F.nblk ? F.blockcnt[b + 1] : F.hdr->n_outliers;
-        if (end == start) return;
+        own = (uint32_t)(end - start);
+        if (own == 0) return;
     } else {
         const bool last = b == F.nblk - 1;
-        const uint32_t own = F.blockcnt[b];
+        own = F.blockcnt[b];
         if (b == 0 && F.hist) fill_central_bin<WRITE_THREADS>(F.hist, F.radius, F.n);
         if (own == 0 && !last) return;
         // the counters before this block's
@@ -231,8 +298,11 @@ __global__ void __launch_bounds__(WRITE_THREADS) k_outlier_write(const __grid_co
         if (own == 0) return;
     }
     if (start >= F.capacity) return;  // beyond the caller's capacity
-    outlier_write_block(F.bitmap, F.words, F.words_per_row, F.nx, F.ny, F.nz, F.x, F.out_idx, F.out_val, F.capacity,
-                        F.row_major, (uint32_t)b, start);
+    if (own > WRITE_DENSE)
+        outlier_write_dense(F, (uint32_t)b, start);
+    else
+        outlier_write_block(F.bitmap, F.words, F.words_per_row, F.nx, F.ny, F.nz, F.x, F.out_idx, F.out_val, F.capacity,
+                            F.row_major, (uint32_t)b, start);
 }
 
 // Outlier values of n fields into their reconstructions: `blocks` blocks per field.
