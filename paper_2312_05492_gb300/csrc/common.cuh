@@ -288,6 +288,10 @@ cudaError_t launch_compress_tiles(const CompressArgs *args, int n, bool early, c
                                   const TileSchedule *sched = nullptr);
 cudaError_t launch_decompress_tiles(const DecompressArgs *args, int n, bool early, cudaStream_t s,
                                     const TileSchedule *sched = nullptr);
+// resident CTAs per SM of the kernel that such a call takes (of args: x, dims, radius and
+// xdom32 decide it)
+cudaError_t compress_tile_ctas(const CompressArgs *args, int n, int &ctas);
+cudaError_t decompress_tile_ctas(int &ctas);
 size_t bitmap_words_tiled(Dims d);
 // the 2-D kernels (nd2.cu) and the 1-D kernels (nd1.cu)
 cudaError_t launch_plane_compress(const CompressArgs &a, bool early, cudaStream_t s);

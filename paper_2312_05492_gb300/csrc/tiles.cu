@@ -1634,13 +1634,14 @@ int scheduled_grid(int grid, const TileSchedule *sched)
     return std::max(grid, 1);
 }
 
-cudaError_t launch_compress_tiles(const CompressArgs *args, int n, bool early, cudaStream_t s, const TileSchedule *sched)
+// The compression kernel of a call: its fields' tensor maps and extents, the kernel that they
+// take, and the grid of one wave.
+struct CompressCall {
+    void (*kernel)(const CBatch);
+    int threads, grid;
+};
+static cudaError_t compress_call(const CompressArgs *args, int n, CBatch &B, Field *fs, CompressCall &call)
 {
-    if (n < 1 || n > kMaxBatch) return cudaErrorInvalidValue;
-    int grid = 0;
-    thread_local CBatch B;  // large parameter block, filled on the host
-    std::memset(&B, 0, sizeof(B));
-    Field fs[kMaxBatch];
     bool tma = true, general = false;
     long long slabs = 0;
     for (int i = 0; i < n; ++i) {
@@ -1655,11 +1656,39 @@ cudaError_t launch_compress_tiles(const CompressArgs *args, int n, bool early, c
     // the wide kernel: general passes, or at most two slabs a CTA (five an SM)
     const bool wide = general || slabs <= 2ll * (kCompressCtas - 1) * sm_count();
     const int variant = wide ? 2 : (tma ? 1 : 0);
-    auto kernel = wide ? k_compress<CNT_WIDE, false> : (tma ? k_compress<CNT, true> : k_compress<CNT, false>);
-    const int threads = wide ? CNT_WIDE : CNT;
-    cudaError_t e = prepare(kernel, threads, kCompressSmem, compress_grid[variant], grid);
+    call.kernel = wide ? k_compress<CNT_WIDE, false> : (tma ? k_compress<CNT, true> : k_compress<CNT, false>);
+    call.threads = wide ? CNT_WIDE : CNT;
+    return prepare(call.kernel, call.threads, kCompressSmem, compress_grid[variant], call.grid);
+}
+
+cudaError_t compress_tile_ctas(const CompressArgs *args, int n, int &ctas)
+{
+    thread_local CBatch B;
+    Field fs[kMaxBatch];
+    CompressCall call;
+    const cudaError_t e = compress_call(args, n, B, fs, call);
+    if (e == cudaSuccess) ctas = call.grid / sm_count();
+    return e;
+}
+
+cudaError_t decompress_tile_ctas(int &ctas)
+{
+    int grid = 0;
+    const cudaError_t e = prepare(k_decompress, DNT, kDecompressSmem, decompress_grid, grid);
+    if (e == cudaSuccess) ctas = grid / sm_count();
+    return e;
+}
+
+cudaError_t launch_compress_tiles(const CompressArgs *args, int n, bool early, cudaStream_t s, const TileSchedule *sched)
+{
+    if (n < 1 || n > kMaxBatch) return cudaErrorInvalidValue;
+    thread_local CBatch B;  // large parameter block, filled on the host
+    std::memset(&B, 0, sizeof(B));
+    Field fs[kMaxBatch];
+    CompressCall call;
+    const cudaError_t e = compress_call(args, n, B, fs, call);
     if (e != cudaSuccess) return e;
-    grid = scheduled_grid(grid, sched);
+    int grid = scheduled_grid(call.grid, sched);
     plan_runs(fs, n, grid, sched ? sched->run : 0);
     int items = 0;
     for (int i = 0; i < n; ++i) {
@@ -1671,7 +1700,7 @@ cudaError_t launch_compress_tiles(const CompressArgs *args, int n, bool early, c
     B.n = n;
     B.items = items;
     if (items < grid) grid = items;
-    return launch_after(early, kernel, grid, threads, kCompressSmem, s, B);
+    return launch_after(early, call.kernel, grid, call.threads, kCompressSmem, s, B);
 }
 
 cudaError_t launch_decompress_tiles(const DecompressArgs *args, int n, bool early, cudaStream_t s,

@@ -46,8 +46,8 @@ std::mutex g_mu;
 std::map<std::string, Picked> g_cache;
 
 // Candidate schedules: the cost model's run and fixed runs up to whole columns,
-// each with the occupancy limit and one or two CTAs per SM fewer.
-std::vector<interp_tile_schedule> candidates(const interp_compress_item *c, int n)
+// each with the occupancy limit (`limit` CTAs per SM) and one or two fewer.
+std::vector<interp_tile_schedule> candidates(const interp_compress_item *c, int n, int limit)
 {
     int max_slabs = 1;
     for (int i = 0; i < n; ++i) max_slabs = std::max(max_slabs, (int)((c[i].dims[0] - 1 + 7) / 8));
@@ -55,8 +55,10 @@ std::vector<interp_tile_schedule> candidates(const interp_compress_item *c, int 
     for (int r = 1; r < max_slabs; r *= 2) runs.push_back(r);
     runs.push_back(max_slabs);
     std::vector<interp_tile_schedule> out;
-    for (int r : runs)
-        for (int ctas : {0, 4, 3}) out.push_back(interp_tile_schedule{r, ctas});
+    for (int r : runs) {
+        out.push_back(interp_tile_schedule{r, 0});
+        for (int ctas = limit - 1; ctas >= limit - 2 && ctas > 0; --ctas) out.push_back(interp_tile_schedule{r, ctas});
+    }
     return out;
 }
 
@@ -77,13 +79,25 @@ extern "C" int interp_tune_batched(const interp_compress_item *citems, const int
             return INTERP_OK;
         }
     }
+    // the kernels' occupancy: of the 3-D fields' kernel (the schedules are its)
+    gi::CompressArgs args[gi::kMaxBatch] = {};
+    int n3 = 0, climit = 1, dlimit = 1;
+    for (int i = 0; i < n; ++i) {
+        if (citems[i].cfg.ndim == 1 || citems[i].cfg.ndim == 2) continue;
+        gi::CompressArgs &a = args[n3++];
+        a.x = citems[i].d_x;
+        a.dims = gi::Dims{(int)citems[i].dims[0], (int)citems[i].dims[1], (int)citems[i].dims[2]};
+        a.radius = citems[i].cfg.radius;
+        a.xdom32 = citems[i].cfg.domain_x == 32;
+    }
+    if (n3 > 0 && gi::compress_tile_ctas(args, n3, climit) != cudaSuccess) return INTERP_ECUDA;
+    if (n3 > 0 && gi::decompress_tile_ctas(dlimit) != cudaSuccess) return INTERP_ECUDA;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     cudaEvent_t ev[2] = {nullptr, nullptr};
     if (cudaEventCreate(&ev[0]) != cudaSuccess || cudaEventCreate(&ev[1]) != cudaSuccess) {
         if (ev[0]) cudaEventDestroy(ev[0]);
         return INTERP_ECUDA;
     }
-    const std::vector<interp_tile_schedule> cand = candidates(citems, n);
     int rc = INTERP_OK;
     // time(kind, schedule): one warm-up call, then the mean of two, in milliseconds
     auto timed = [&](bool compress, const interp_tile_schedule &sc, float &ms) -> int {
@@ -103,7 +117,7 @@ extern "C" int interp_tune_batched(const interp_compress_item *citems, const int
     };
     Picked best{};
     float best_c = 1e30f, best_d = 1e30f;
-    for (const auto &sc : cand) {
+    for (const auto &sc : candidates(citems, n, climit)) {
         float ms = 0.0f;
         rc = timed(true, sc, ms);
         if (rc != INTERP_OK) break;
@@ -113,7 +127,7 @@ extern "C" int interp_tune_batched(const interp_compress_item *citems, const int
         }
     }
     // decompression reads the codes of the last compression, identical for every schedule
-    for (const auto &sc : cand) {
+    for (const auto &sc : candidates(citems, n, dlimit)) {
         if (rc != INTERP_OK) break;
         float ms = 0.0f;
         rc = timed(false, sc, ms);
