@@ -524,7 +524,7 @@ def run_ours(args, rank, world, local):
                           "frac": round(step_gbs / peak, 4), "algorithmic_bytes_per_step": step_alg},
         "max_abs_err_over_eb": err / h.eb_abs,
         "quality": quality_summary(G, cf, x, xrec),
-        "gpu_launches": (G.launches_compress(cfg) + G.LAUNCHES_DECOMPRESS) * args.steps,
+        "gpu_launches": (G.launches_compress(cfg, x.shape) + G.LAUNCHES_DECOMPRESS) * args.steps,
         "clocks": clocks,
     }
     if not args.no_extras:
@@ -786,7 +786,8 @@ def run_batch(args, rank, world, local):
                              "speedup_vs_single": round(s_single / s_graph, 3), "bit_exact_vs_single": bool(s_exact),
                              "tile_schedule": s_sched,
                              "bound_ok": bool(s_bound)},
-            "gpu_launches": (G.launches_compress(cfgs[0]) + G.LAUNCHES_DECOMPRESS) * k}
+            "gpu_launches": (G.launches_compress(cfgs[0], max(xs, key=lambda x: x.numel()).shape)
+                             + G.LAUNCHES_DECOMPRESS) * k}
 
 
 def small_batch_fields(device):

@@ -32,10 +32,17 @@ FUNCTIONS = ("interp_anchor_count", "interp_workspace_bytes", "interp_compress",
              "interp_compress_batched_scheduled", "interp_decompress_batched_scheduled", "interp_tune_batched")
 
 # kernels each call launches, for one field or a whole batch: compress = zeroing +
-# set-up (profile, range, bounds) + tiles + outlier write (fields above about 2^28
-# points: an outlier scan too); decompress = outlier scatter + tiles
-def launches_compress(cfg: "Config") -> int:
-    return 4
+# set-up (profile, range, bounds) + tiles + outlier write, and an outlier scan for a field
+# with more than SCAN_WORDS bitmap words (32 x-positions of a row each; dims: the call's
+# largest field); decompress = outlier scatter + tiles
+SCAN_WORDS = 4096 * 2048
+
+
+def launches_compress(cfg: "Config", dims=None) -> int:
+    if dims is None:
+        return 4
+    words = int(dims[0]) * int(dims[1]) * ((int(dims[2]) + 31) // 32)
+    return 5 if words > SCAN_WORDS else 4
 
 
 LAUNCHES_DECOMPRESS = 2
