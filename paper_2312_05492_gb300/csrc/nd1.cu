@@ -16,7 +16,7 @@
 //
 // Bound by instruction issue (about 25 a point: prediction 2 .. 9, quantization 11,
 // histogram 3), then by HBM: 4N read + 2N written.
-#include "tma.cuh"
+#include "lanes.cuh"
 
 namespace gi {
 namespace {
@@ -34,8 +34,6 @@ constexpr int CHUNK = 512, CLANES = CHUNK / RUN;  // lanes per chunk
 constexpr int LEVELS = 9;
 constexpr int VP = 36;                // floats per landed run (32 and 4 of padding)
 constexpr int KP = 40;                // codes per landed run
-constexpr int R_HIST_BINS = 8192;     // bins kept in shared memory
-constexpr int R_WINDOW = 2048;        // and with more than those, the bins around R
 constexpr size_t R_V = sizeof(float) * 32 * VP, R_K = sizeof(uint16_t) * 32 * KP;
 constexpr size_t R_LQ = 0;                       // level constants
 constexpr size_t R_SPARE = R_LQ + 16 * LEVELS;   // one word per lane for updates that count nothing
@@ -46,22 +44,6 @@ static_assert(R_WARPS % 16 == 0 && R_HIST % 16 == 0, "shared layout alignment");
 
 extern __shared__ __align__(128) unsigned char r_smem[];
 
-// What a kernel does with the points: apply the stored codes; quantize and count in shared
-// or in global bins.
-enum { DECODE = 0, ENCODE = 1, ENCODE_GBINS = 2 };
-enum { K_LINEAR = 0, K_NAK = 1, K_NATURAL = 2 };
-
-// Level constants, one thread per level, with the header's own arithmetic (alpha^l by
-// repeated multiplication in double).
-__device__ void row_levels(const interp_header *h)
-{
-    const int l = threadIdx.x;
-    if (l >= LEVELS) return;
-    double apow = 1.0;
-    for (int j = 0; j < l; ++j) apow *= h->alpha;
-    const float e = (float)(h->eb_abs / apow);
-    reinterpret_cast<float4 *>(r_smem + R_LQ)[l] = make_float4(e, 2.0f * e, (float)(1.0 / (2.0 * (double)e)), 0.0f);
-}
 __device__ __forceinline__ LevelQ level_of(int l)
 {
     const float4 q = reinterpret_cast<const float4 *>(r_smem + R_LQ)[l];
@@ -75,40 +57,13 @@ struct Lane {
     uint32_t cw[RUN / 2];
 };
 
-struct Ctx {
-    uint32_t cbias, R;
+struct Ctx : Bins {
+    uint32_t cbias;
     float Rf;
-    uint32_t hist, spare;  // shared addresses of the bins (of bin win0's) and of this lane's spare word
-    uint32_t win0;         // first bin kept in shared memory
-    uint32_t *hist_g;      // more than R_HIST_BINS bins: all of them in global memory, may be null
     int lane, cl;          // lane, lane within its chunk
     float closing;         // the point after the segment (an anchor), in every lane
     int last;              // last in-field offset from the segment's start (SEG when it is whole)
 };
-
-// Count a code other than R (whose bin is filled in afterwards as N minus the others).
-// ENCODE_GBINS: more bins than shared memory keeps.  Those around R are kept there all the
-// same (nearly all codes, and few bins: in global memory their updates wait for one
-// another; 64 x 2^17 points, radius 4097, bound 1e-5: 893 -> 25 us); the others are counted in global memory.
-template <int MODE>
-__device__ __forceinline__ void count(const Ctx &c, uint32_t code, bool counts)
-{
-    const bool yes = counts && code != c.R;
-    if constexpr (MODE == ENCODE_GBINS) {
-        const uint32_t w = code - c.win0;
-        const bool in = w < (uint32_t)R_WINDOW;
-        asm volatile("red.shared.add.u32 [%0], 1;\n" ::"r"(yes && in ? c.hist + 4u * w : c.spare));
-        if (yes && !in && c.hist_g) atomicAdd(c.hist_g + code, 1u);
-    } else {
-        asm volatile("red.shared.add.u32 [%0], 1;\n" ::"r"(yes ? c.hist + 4u * code : c.spare));
-    }
-}
-
-template <int KIND>
-__device__ __forceinline__ float cubic_of(float m3, float m1, float p1, float p3)
-{
-    return KIND == K_NATURAL ? sp_cubic_nat_call(m3, m1, p1, p3) : sp_cubic_nak(m3, m1, p1, p3);
-}
 
 // Neighbour-count rule (Sec. IV-B.1).
 template <int KIND>
@@ -277,10 +232,10 @@ __global__ void __launch_bounds__(32 * RC.warps, RC.ctas) k_row_compress(const C
     wait_for_previous();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nx = a.dims.nx;
-    const int bins = MODE == ENCODE_GBINS ? R_WINDOW : 2 * a.radius;  // in shared memory
-    const int win0 = MODE == ENCODE_GBINS ? a.radius - R_WINDOW / 2 : 0;
+    const int bins = MODE == ENCODE_GBINS ? LANE_WINDOW : 2 * a.radius;  // in shared memory
+    const int win0 = MODE == ENCODE_GBINS ? a.radius - LANE_WINDOW / 2 : 0;
     uint32_t *hs = reinterpret_cast<uint32_t *>(r_smem + R_HIST);
-    row_levels(a.hdr);
+    store_levels<LEVELS>(a.hdr, reinterpret_cast<float4 *>(r_smem + R_LQ));
     for (int i = threadIdx.x; i < bins; i += 32 * RC.warps) hs[i] = 0u;
     __syncthreads();
     float *land = reinterpret_cast<float *>(r_smem + R_WARPS + R_WARP * warp);
@@ -410,7 +365,7 @@ __global__ void __launch_bounds__(32 * RD.warps, RD.ctas) k_row_decompress(const
     wait_for_previous();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nx = a.dims.nx;
-    row_levels(a.hdr);
+    store_levels<LEVELS>(a.hdr, reinterpret_cast<float4 *>(r_smem + R_LQ));
     __syncthreads();
     float *stage = reinterpret_cast<float *>(r_smem + R_WARPS + R_WARP * warp);
     uint16_t *land = reinterpret_cast<uint16_t *>(r_smem + R_WARPS + R_WARP * warp + R_V);
@@ -526,10 +481,10 @@ cudaError_t launch_rows(K kernel, Shape shape, const A &a, size_t smem, size_t m
 
 cudaError_t launch_row_compress(const CompressArgs &a, bool early, cudaStream_t s)
 {
-    constexpr size_t wide = R_HIST + sizeof(uint32_t) * R_WINDOW;
-    if (2 * a.radius > R_HIST_BINS) return launch_rows(k_row_compress<ENCODE_GBINS>, RC, a, wide, wide, early, s);
+    constexpr size_t wide = R_HIST + sizeof(uint32_t) * LANE_WINDOW;
+    if (2 * a.radius > LANE_BINS) return launch_rows(k_row_compress<ENCODE_GBINS>, RC, a, wide, wide, early, s);
     return launch_rows(k_row_compress<ENCODE>, RC, a, R_HIST + sizeof(uint32_t) * 2 * (size_t)a.radius,
-                       R_HIST + sizeof(uint32_t) * R_HIST_BINS, early, s);
+                       R_HIST + sizeof(uint32_t) * LANE_BINS, early, s);
 }
 
 cudaError_t launch_row_decompress(const DecompressArgs &a, bool early, cudaStream_t s)

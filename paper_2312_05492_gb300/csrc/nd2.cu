@@ -21,7 +21,7 @@
 //
 // The input lands in shared memory a step ahead (cp.async), 16-byte groups permuted so
 // that a warp's reads fall in distinct banks.
-#include "tma.cuh"
+#include "lanes.cuh"
 
 namespace gi {
 namespace {
@@ -32,8 +32,6 @@ constexpr int P_CTAS = 2;                 // CTAs per SM: 16 warps of 128 regist
 constexpr int A = 16;                     // chunk edge
 constexpr int SX = 64;                    // columns of a strip
 constexpr int LEVELS = 4;
-constexpr int P_HIST_BINS = 8192;         // bins kept in shared memory
-constexpr int P_WINDOW = 2048;            // and with more than those, the bins around R
 // per warp: 16 landed rows and the closing column (values, or codes in the first half
 // of the room), then a stage for rows that cannot be stored 16 bytes at a time
 constexpr size_t P_LAND = 0;
@@ -47,22 +45,7 @@ static_assert(P_WARP % 16 == 0 && P_HIST % 16 == 0, "shared layout alignment");
 
 extern __shared__ __align__(128) unsigned char p_smem[];
 
-// What a kernel does with the points: apply the stored codes; quantize and count in shared
-// or in global bins.
-enum { DECODE = 0, ENCODE = 1, ENCODE_GBINS = 2 };
-enum { K_LINEAR = 0, K_NAK = 1, K_NATURAL = 2 };
 enum { ROW0 = 0, ROW1 = 1, ROW2 = 2, ROW3 = 3 };
-
-// Level constants, one thread per level, with the header's own arithmetic.
-__device__ void plane_levels(const interp_header *h)
-{
-    const int l = threadIdx.x;
-    if (l >= LEVELS) return;
-    double apow = 1.0;
-    for (int j = 0; j < l; ++j) apow *= h->alpha;
-    const float e = (float)(h->eb_abs / apow);
-    reinterpret_cast<float4 *>(p_smem + P_LQ)[l] = make_float4(e, 2.0f * e, (float)(1.0 / (2.0 * (double)e)), 0.0f);
-}
 
 // A lane's points.  Row 0 of v is row 4 py of the chunk, but row 16 in the lanes py = 0,
 // whose row 0 (finished by the previous step) is `top`.  Column 8 is the closing column
@@ -73,42 +56,15 @@ struct Patch {
     uint32_t mc[4];
 };
 
-struct Ctx {
-    uint32_t cbias, R;
+struct Ctx : Bins {
+    uint32_t cbias;
     float Rf;
-    uint32_t hist, spare;  // shared addresses of the bins (of bin win0's) and of this lane's spare word
-    uint32_t win0;         // first bin kept in shared memory
-    uint32_t *hist_g;      // more than P_HIST_BINS bins: all of them in global memory, may be null
     int lane, px, py;
     int lx, ly;            // last in-field column from the lane's first one, and row from the
                            // chunk's first one
     bool count0;           // row 0's codes are counted (lanes py = 0: the closing row is this run's)
     LevelQ q;
 };
-
-// Count a code other than R (whose bin is filled in afterwards as N minus the others).
-// ENCODE_GBINS: more bins than shared memory keeps.  Those around R are kept there all the
-// same (nearly all codes, and few bins: in global memory their updates wait for one
-// another; 8 x 2048 x 2048 points, radius 4097: 4.49 -> 0.13 ms); the others are counted in global memory.
-template <int MODE>
-__device__ __forceinline__ void count(const Ctx &c, uint32_t code, bool counts)
-{
-    const bool yes = counts && code != c.R;
-    if constexpr (MODE == ENCODE_GBINS) {
-        const uint32_t w = code - c.win0;
-        const bool in = w < (uint32_t)P_WINDOW;
-        asm volatile("red.shared.add.u32 [%0], 1;\n" ::"r"(yes && in ? c.hist + 4u * w : c.spare));
-        if (yes && !in && c.hist_g) atomicAdd(c.hist_g + code, 1u);
-    } else {
-        asm volatile("red.shared.add.u32 [%0], 1;\n" ::"r"(yes ? c.hist + 4u * code : c.spare));
-    }
-}
-
-template <int KIND>
-__device__ __forceinline__ float cubic_of(float m3, float m1, float p1, float p3)
-{
-    return KIND == K_NATURAL ? sp_cubic_nat_call(m3, m1, p1, p3) : sp_cubic_nak(m3, m1, p1, p3);
-}
 
 // Neighbour-count rule (Sec. IV-B.1).  MAYBE3: bit 0 / 1 set if x_{n-3s} / x_{n+3s} may
 // lie in the chunk at all (a stencil that cannot occur is not evaluated).
@@ -431,10 +387,10 @@ __global__ void __launch_bounds__(P_THREADS, P_CTAS) k_plane_compress(const Comp
     wait_for_previous();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const Dims d = a.dims;
-    const int bins = MODE == ENCODE_GBINS ? P_WINDOW : 2 * a.radius;  // in shared memory
-    const int win0 = MODE == ENCODE_GBINS ? a.radius - P_WINDOW / 2 : 0;
+    const int bins = MODE == ENCODE_GBINS ? LANE_WINDOW : 2 * a.radius;  // in shared memory
+    const int win0 = MODE == ENCODE_GBINS ? a.radius - LANE_WINDOW / 2 : 0;
     uint32_t *hs = reinterpret_cast<uint32_t *>(p_smem + P_HIST);
-    plane_levels(a.hdr);
+    store_levels<LEVELS>(a.hdr, reinterpret_cast<float4 *>(p_smem + P_LQ));
     for (int i = threadIdx.x; i < bins; i += P_THREADS) hs[i] = 0u;
     __syncthreads();
     unsigned char *land = p_smem + P_WARP * warp;
@@ -610,7 +566,7 @@ __global__ void __launch_bounds__(P_THREADS, P_CTAS) k_plane_decompress(const De
     wait_for_previous();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const Dims d = a.dims;
-    plane_levels(a.hdr);
+    store_levels<LEVELS>(a.hdr, reinterpret_cast<float4 *>(p_smem + P_LQ));
     __syncthreads();
     unsigned char *land = p_smem + P_WARP * warp;
     float *stage = reinterpret_cast<float *>(land + P_STAGE);
@@ -810,10 +766,10 @@ cudaError_t launch_planes(K kernel, const Args &a, size_t smem, size_t most, boo
 
 cudaError_t launch_plane_compress(const CompressArgs &a, bool early, cudaStream_t s)
 {
-    constexpr size_t wide = P_HIST + sizeof(uint32_t) * P_WINDOW;
-    if (2 * a.radius > P_HIST_BINS) return launch_planes(k_plane_compress<ENCODE_GBINS>, a, wide, wide, early, s);
+    constexpr size_t wide = P_HIST + sizeof(uint32_t) * LANE_WINDOW;
+    if (2 * a.radius > LANE_BINS) return launch_planes(k_plane_compress<ENCODE_GBINS>, a, wide, wide, early, s);
     return launch_planes(k_plane_compress<ENCODE>, a, P_HIST + sizeof(uint32_t) * 2 * (size_t)a.radius,
-                         P_HIST + sizeof(uint32_t) * P_HIST_BINS, early, s);
+                         P_HIST + sizeof(uint32_t) * LANE_BINS, early, s);
 }
 
 cudaError_t launch_plane_decompress(const DecompressArgs &a, bool early, cudaStream_t s)

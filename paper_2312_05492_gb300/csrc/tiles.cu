@@ -61,10 +61,8 @@ constexpr int EZ = 9, EY = OY + 1, EX = OX + 1;  // slab box extents (z, y, x)
 constexpr int XP = OX + 4, PLANE = EY * XP;
 constexpr int DP = EX, DPLANE = EY * DP;
 constexpr int CP = OX + 2;                       // u16 pitch of code rows (17 words, odd)
-constexpr int CBOX_PLANE = EY * CP;              // code box (compression staging, decompression input):
-constexpr int CBOX = EZ * CBOX_PLANE;            // every row and column of the slab box
-constexpr int STAGE_PLANE = CBOX_PLANE;
-constexpr int STAGE = CBOX;
+constexpr int STAGE_PLANE = EY * CP;             // compression's staged codes: every row and column
+constexpr int STAGE = EZ * STAGE_PLANE;          // of the slab box
 constexpr int XPL = 8;                           // landed input planes: 1..8 of a slab (plane 0 is
                                                  // carried, or loaded directly at a run's start)
 constexpr int KP = 40;                           // codes per landed row (x 0..39)
@@ -78,8 +76,7 @@ __host__ __device__ constexpr int bstride(int a)
 {
     return a == 2 ? 1 : (a == 1 ? (COMPRESS ? XP : DP) : (COMPRESS ? PLANE : DPLANE));
 }
-__host__ __device__ constexpr int sstride(int a) { return a == 2 ? 1 : (a == 1 ? CP : STAGE_PLANE); }
-__host__ __device__ constexpr int cstride(int a) { return a == 2 ? 1 : (a == 1 ? CP : CBOX_PLANE); }
+__host__ __device__ constexpr int cstride(int a) { return a == 2 ? 1 : (a == 1 ? CP : STAGE_PLANE); }
 // decompression reads the codes where the TMA landed them: rows of KP codes, planes of EY rows
 __host__ __device__ constexpr int lstride(int a) { return a == 2 ? 1 : (a == 1 ? KP : EY * KP); }
 static_assert((KP * 2) % 16 == 0, "landed code rows stay 16-byte aligned");
@@ -277,7 +274,7 @@ __device__ __forceinline__ void run_pass(float *__restrict__ box, const Sink &sk
     constexpr int EU = ext_of(U), EV = ext_of(V);
     constexpr int NC = chunks_of(D);
     constexpr int BD = bstride<COMPRESS>(D), BU = bstride<COMPRESS>(U), BV = bstride<COMPRESS>(V);
-    constexpr int SD = sstride(D), SU = sstride(U), SV = sstride(V);
+    constexpr int SD = cstride(D), SU = cstride(U), SV = cstride(V);
     constexpr int KD = lstride(D), KU = lstride(U), KV = lstride(V);
     constexpr int l = S == 1 ? 0 : (S == 2 ? 1 : 2);
     if ((int)threadIdx.x >= lv.nseg[sl.carried ? 1 : 0][l][k]) return;  // no segment for this thread
@@ -1594,18 +1591,14 @@ void plan_runs(Field *fs, int n, int grid, int forced = 0)
     int best_run = max_slabs;
     double best = 1e300;
     for (int run = 1; run <= max_slabs; ++run) {
-        long long items = 0, work = 0;
-        for (int i = 0; i < n; ++i) {
-            items += (long long)fs[i].cols * ((fs[i].slabs + run - 1) / run);
-            work += (long long)fs[i].cols * fs[i].slabs;
-        }
+        long long items = 0;
+        for (int i = 0; i < n; ++i) items += (long long)fs[i].cols * ((fs[i].slabs + run - 1) / run);
         const long long per_cta = (items + grid - 1) / grid;
         // the busiest CTA's items, each the run length plus the cost of a run start
         // (plane 0 loaded and computed, the transfers not yet overlapped: about two
         // slabs), and the run length once more for the CTAs that idle while the last
         // items finish; fitted to 512^3 timings of runs 1 .. 64 (best: 8)
         const double cost = (double)per_cta * (run + 2.0) + 1.0 * run;
-        (void)work;
         if (cost <= best + 1e-9) {  // ties: the longer run (fewer run starts)
             best = cost;
             best_run = run;
