@@ -156,7 +156,8 @@ struct BitRun {
     }
 };
 
-// SMEM_TAB: the codebook (length << 24 | codeword) in shared memory.
+// SMEM_TAB: the codebook (length << 24 | codeword) in shared memory; otherwise a code's entry
+// is put together from global memory.
 template <bool SMEM_TAB>
 __global__ void __launch_bounds__(ENC_THREADS, 2) k_huff_encode(const uint16_t *__restrict__ codes, unsigned long long n,
                                                                const uint8_t *__restrict__ lengths,
@@ -170,7 +171,7 @@ __global__ void __launch_bounds__(ENC_THREADS, 2) k_huff_encode(const uint16_t *
     __shared__ uint32_t warp_words[ENC_WARPS];
     __shared__ uint32_t tile_s, base_s;
     uint32_t *tab = enc_sm + ENC_WARPS * MAX_WORDS;
-    bool longest16 = true, packed = SMEM_TAB;
+    bool longest16 = true, packed = true;
     {
         int l16 = 0, l24 = 0;
         for (int i = threadIdx.x; i < nsym; i += ENC_THREADS) {
@@ -199,7 +200,10 @@ __global__ void __launch_bounds__(ENC_THREADS, 2) k_huff_encode(const uint16_t *
             const int cnt = lane_codes(codes, n, i0, vec, w);
             if (packed) {
 #pragma unroll
-                for (int j = 0; j < HLANE; ++j) e[j] = tab[code_at(w, j)];
+                for (int j = 0; j < HLANE; ++j) {
+                    const uint32_t c = code_at(w, j);
+                    e[j] = SMEM_TAB ? tab[c] : ((uint32_t)__ldg(lengths + c) << 24) | __ldg(codewords + c);
+                }
                 if (cnt < HLANE)
 #pragma unroll
                     for (int j = 0; j < HLANE; ++j) e[j] = j < cnt ? e[j] : 0u;
