@@ -49,8 +49,9 @@ constexpr int DEC_PITCH = 80;   // bytes of a thread's code buffer (35 codes and
                                 // may overwrite) and of its ring of stream words; an odd number of
                                 // 16-byte units: a warp's accesses spread over the banks
 constexpr int DEC_RING = 16;    // words of the ring, four 16-byte blocks
-constexpr int SYM_SMEM = 8192;  // canonical symbol list kept in shared memory up to this many symbols
-constexpr int DEC_THREADS = 448;  // two CTAs an SM hold one field of 512^3 codes in one wave
+constexpr int SYM_SMEM = 4096;  // canonical symbol list kept in shared memory up to this many symbols
+constexpr int DEC_THREADS = 448;  // two CTAs fit an SM, with SYM_SMEM symbols too (480, which fit with
+                                  // 2800, decode 512^3 codes no faster: 247 us, 248)
 static_assert(2 * (DEC_GROUP - 1 + DEC_STEPS * LUT_SYMS + LUT_SYMS - 1) <= DEC_PITCH, "a round fits the buffer");
 static_assert(4 * DEC_RING <= DEC_PITCH && 31 + DEC_STEPS * MAX_LEN < 32 * 4, "a round takes at most 3 words");
 
@@ -404,8 +405,9 @@ template <int VEC>
 __global__ void __launch_bounds__(DEC_THREADS, 2) k_huff_decode(const uint32_t *__restrict__ words,
                                                                const uint32_t *__restrict__ offsets,
                                                                unsigned long long n, const DecodeTables *tg,
-                                                               const uint16_t *symbols, int nsym, int nsym_smem, uint16_t *codes,
-                                                               unsigned long long nchunks, unsigned int *bad)
+                                                               const uint16_t *symbols, int nsym, int nsym_smem,
+                                                               uint16_t *codes, unsigned long long nchunks,
+                                                               unsigned per, unsigned int *bad)
 {
     wait_for_previous();
     __shared__ DecodeTables t;
@@ -414,13 +416,13 @@ __global__ void __launch_bounds__(DEC_THREADS, 2) k_huff_decode(const uint32_t *
     uint2 *lut = reinterpret_cast<uint2 *>(dec_sm);
     unsigned char *bufs = dec_sm + sizeof(uint2) * (1 << LUT_BITS);
     unsigned char *buf = bufs + DEC_PITCH * threadIdx.x;
-    uint32_t *ring = reinterpret_cast<uint32_t *>(bufs + DEC_PITCH * (blockDim.x + threadIdx.x));
-    uint16_t *sym_s = reinterpret_cast<uint16_t *>(bufs + 2 * DEC_PITCH * blockDim.x);
+    uint32_t *ring = reinterpret_cast<uint32_t *>(bufs + DEC_PITCH * (DEC_THREADS + threadIdx.x));
+    uint16_t *sym_s = reinterpret_cast<uint16_t *>(bufs + 2 * DEC_PITCH * DEC_THREADS);
     {
         const uint32_t *src = reinterpret_cast<const uint32_t *>(tg);
         uint32_t *dst = reinterpret_cast<uint32_t *>(&t);
-        for (int i = threadIdx.x; i < (int)(sizeof(DecodeTables) / 4); i += blockDim.x) dst[i] = src[i];
-        for (int i = threadIdx.x; i < nsym_smem; i += blockDim.x) sym_s[i] = symbols[i];
+        for (int i = threadIdx.x; i < (int)(sizeof(DecodeTables) / 4); i += DEC_THREADS) dst[i] = src[i];
+        for (int i = threadIdx.x; i < nsym_smem; i += DEC_THREADS) sym_s[i] = symbols[i];
     }
     __syncthreads();
     const uint16_t *sym_tab = nsym_smem ? sym_s : symbols;
@@ -432,7 +434,7 @@ __global__ void __launch_bounds__(DEC_THREADS, 2) k_huff_decode(const uint32_t *
     }
     // one-codeword table (symbol << 8 | length, 0: longer than the window) in the buffers' room
     uint32_t *lut1 = reinterpret_cast<uint32_t *>(bufs);
-    for (int v = threadIdx.x; v < (1 << LUT_BITS); v += blockDim.x) {
+    for (int v = threadIdx.x; v < (1 << LUT_BITS); v += DEC_THREADS) {
         uint32_t e = 0;
         for (int l = 1; l <= min(maxl, LUT_BITS); ++l) {
             const uint32_t c = (uint32_t)v >> (LUT_BITS - l);
@@ -447,7 +449,7 @@ __global__ void __launch_bounds__(DEC_THREADS, 2) k_huff_decode(const uint32_t *
     // lookup table: word x and the low byte of y the symbols - R, then the bits taken by all
     // of them (y bits 8-11) and their number (y bits 12-14).  Number 0 and some bits: one
     // codeword whose symbol (word x) is no byte from R; number 0 and no bits: a longer codeword.
-    for (int v = threadIdx.x; v < (1 << LUT_BITS); v += blockDim.x) {
+    for (int v = threadIdx.x; v < (1 << LUT_BITS); v += DEC_THREADS) {
         unsigned long long e = 0;
         uint32_t used = 0, k = 0;
         while (k < (uint32_t)LUT_SYMS) {
@@ -470,8 +472,8 @@ __global__ void __launch_bounds__(DEC_THREADS, 2) k_huff_decode(const uint32_t *
     }
     __syncthreads();
 
-    const unsigned long long chunk = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool live = chunk < nchunks;
+    const unsigned long long chunk = (unsigned long long)blockIdx.x * per + threadIdx.x;
+    const bool live = threadIdx.x < per && chunk < nchunks;
     // The chunk's words arrive in 16-byte blocks through the ring, asynchronously and two
     // rounds ahead.  Word q counts from the block that holds the chunk's first word; words
     // before rbeg or from rend on are not the chunk's (past its end it reads zeros).
@@ -723,22 +725,24 @@ cudaError_t launch_huffman_encode(const uint16_t *codes, unsigned long long n, c
 }
 
 // Shared memory of a decoding CTA: the lookup table, a code buffer and a ring per thread, the symbols.
-static constexpr size_t decode_smem(unsigned threads, int symbols)
+static constexpr size_t decode_smem(int symbols)
 {
-    return sizeof(uint2) * (1 << LUT_BITS) + 2 * (size_t)DEC_PITCH * threads + sizeof(uint16_t) * (size_t)symbols;
+    return sizeof(uint2) * (1 << LUT_BITS) + 2 * (size_t)DEC_PITCH * DEC_THREADS + sizeof(uint16_t) * (size_t)symbols;
 }
+static_assert(2 * (decode_smem(SYM_SMEM) + 1024 + 1024) <= 228 * 1024, "two decoding CTAs fit an SM");
 
 template <int VEC>
-static cudaError_t launch_decode(unsigned grid, unsigned threads, size_t smem, cudaStream_t s, const uint32_t *words,
+static cudaError_t launch_decode(unsigned grid, unsigned per, cudaStream_t s, const uint32_t *words,
                                  const uint32_t *offsets, unsigned long long n, const DecodeTables *t,
-                                 const uint16_t *symbols, int nsym, int nsym_smem, uint16_t *codes,
-                                 unsigned long long nch, unsigned int *bad)
+                                 const uint16_t *symbols, int nsym, uint16_t *codes, unsigned long long nch,
+                                 unsigned int *bad)
 {
-    const cudaError_t e = allow_smem(k_huff_decode<VEC>, decode_smem(DEC_THREADS, SYM_SMEM));
+    const int nsym_smem = nsym <= SYM_SMEM ? nsym : 0;
+    const cudaError_t e = allow_smem(k_huff_decode<VEC>, decode_smem(SYM_SMEM));
     if (e != cudaSuccess) return e;
     // the tables kernel is one CTA
-    return launch_after(true, k_huff_decode<VEC>, grid, threads, smem, s, words, offsets, n, t, symbols, nsym, nsym_smem,
-                        codes, nch, bad);
+    return launch_after(true, k_huff_decode<VEC>, grid, DEC_THREADS, decode_smem(nsym_smem), s, words, offsets, n, t,
+                        symbols, nsym, nsym_smem, codes, nch, per, bad);
 }
 
 cudaError_t launch_huffman_decode(const uint32_t *words, const uint32_t *offsets, unsigned long long n,
@@ -752,18 +756,14 @@ cudaError_t launch_huffman_decode(const uint32_t *words, const uint32_t *offsets
     if (e != cudaSuccess) return e;
     const unsigned long long nch = huffman_chunks(n);
     if (nch == 0) return cudaSuccess;
-    // few chunks spread over the SMs: at least 128 threads (they share the table's building)
-    const unsigned long long per = (nch + 2ull * sm_count() - 1) / (2ull * sm_count());
-    const unsigned threads = (unsigned)std::min<unsigned long long>(DEC_THREADS, std::max<unsigned long long>(128, (per + 31) / 32 * 32));
-    const unsigned grid = (unsigned)((nch + threads - 1) / threads);
-    const int nsym_smem = nsym <= SYM_SMEM ? nsym : 0;
-    const size_t smem = decode_smem(threads, nsym_smem);
+    // few chunks spread over the SMs, a warp of them a CTA or more; all of its threads build the table
+    const unsigned long long share = (nch + 2ull * sm_count() - 1) / (2ull * sm_count());
+    const unsigned per = (unsigned)std::min<unsigned long long>(DEC_THREADS, (share + 31) / 32 * 32);
+    const unsigned grid = (unsigned)((nch + per - 1) / per);
     const uintptr_t a = reinterpret_cast<uintptr_t>(codes);
-    if ((a & 31u) == 0)
-        return launch_decode<32>(grid, threads, smem, s, words, offsets, n, t, symbols, nsym, nsym_smem, codes, nch, bad);
-    if ((a & 15u) == 0)
-        return launch_decode<16>(grid, threads, smem, s, words, offsets, n, t, symbols, nsym, nsym_smem, codes, nch, bad);
-    return launch_decode<2>(grid, threads, smem, s, words, offsets, n, t, symbols, nsym, nsym_smem, codes, nch, bad);
+    if ((a & 31u) == 0) return launch_decode<32>(grid, per, s, words, offsets, n, t, symbols, nsym, codes, nch, bad);
+    if ((a & 15u) == 0) return launch_decode<16>(grid, per, s, words, offsets, n, t, symbols, nsym, codes, nch, bad);
+    return launch_decode<2>(grid, per, s, words, offsets, n, t, symbols, nsym, codes, nch, bad);
 }
 
 }  // namespace gi
