@@ -16,7 +16,7 @@
 // taken earlier, so they run or are done), and writes its words out coalesced.  The codes
 // are read once; as sizes, scan and write passes they were read twice.
 // Decoding: one thread per chunk, reading its words in order.  The next 12 bits index a
-// lookup table with the whole codewords they contain (up to five symbols, as signed bytes
+// lookup table with the whole codewords they contain (up to five symbols, as bytes of 256
 // around the central code R, and the bits they take); other codewords take the canonical
 // rule (per length, the first codeword and the first symbol index).  Every thread does
 // DEC_STEPS lookups a round whatever they yield, so the lanes of a warp stay together;
@@ -368,29 +368,21 @@ struct LongCodes {
     int n;
 };
 
-// Byte permutation with sign replication (selector bit 3), which __byte_perm masks off.
-__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t sel)
-{
-    uint32_t r;
-    asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r) : "r"(a), "r"(sel));
-    return r;
-}
-
 // One group of DEC_GROUP codes from shared to global memory.  VEC: bytes the destination is
 // aligned to (32, 16 or 2).
 template <int VEC>
 __device__ __forceinline__ void store_group(uint16_t *dst, const unsigned char *src)
 {
     const uint4 a = reinterpret_cast<const uint4 *>(src)[0], b = reinterpret_cast<const uint4 *>(src)[1];
+    const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
     if (VEC == 32) {
-        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(dst), "r"(a.x), "r"(a.y),
-                     "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(dst), "r"(w[0]), "r"(w[1]),
+                     "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
                      : "memory");
     } else if (VEC == 16) {
-        reinterpret_cast<uint4 *>(dst)[0] = a;
-        reinterpret_cast<uint4 *>(dst)[1] = b;
+        reinterpret_cast<uint4 *>(dst)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+        reinterpret_cast<uint4 *>(dst)[1] = make_uint4(w[4], w[5], w[6], w[7]);
     } else {
-        const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             dst[2 * k] = (uint16_t)(w[k] & 0xffffu);
@@ -412,6 +404,7 @@ __global__ void __launch_bounds__(DEC_THREADS, 2) k_huff_decode(const uint32_t *
     wait_for_previous();
     __shared__ DecodeTables t;
     __shared__ LongCodes lc;
+    __shared__ uint32_t taken;  // symbols of all entries of the lookup table
     extern __shared__ __align__(16) unsigned char dec_sm[];
     uint2 *lut = reinterpret_cast<uint2 *>(dec_sm);
     unsigned char *bufs = dec_sm + sizeof(uint2) * (1 << LUT_BITS);
@@ -426,7 +419,9 @@ __global__ void __launch_bounds__(DEC_THREADS, 2) k_huff_decode(const uint32_t *
     }
     __syncthreads();
     const uint16_t *sym_tab = nsym_smem ? sym_s : symbols;
-    const int R = nsym / 2, maxl = t.max_len;
+    const int maxl = t.max_len;
+    // symbols are bytes from here on in the lookup table: 128 on either side of R
+    const int base = max(nsym / 2 - 128, 0);
     if (threadIdx.x == 0) {
         lc.n = 0;
         for (int l = LUT_BITS + 1; l <= maxl; ++l)
@@ -446,31 +441,42 @@ __global__ void __launch_bounds__(DEC_THREADS, 2) k_huff_decode(const uint32_t *
         lut1[v] = e;
     }
     __syncthreads();
-    // lookup table: word x and the low byte of y the symbols - R, then the bits taken by all
+    if (threadIdx.x == 0) taken = 0u;
+    __syncthreads();
+    // lookup table: word x and the low byte of y the symbols - base, then the bits taken by all
     // of them (y bits 8-11) and their number (y bits 12-14).  Number 0 and some bits: one
-    // codeword whose symbol (word x) is no byte from R; number 0 and no bits: a longer codeword.
+    // codeword whose symbol (word x) is no byte from base; number 0 and no bits: a longer codeword.
+    uint32_t symbols_here = 0;
     for (int v = threadIdx.x; v < (1 << LUT_BITS); v += DEC_THREADS) {
         unsigned long long e = 0;
         uint32_t used = 0, k = 0;
         while (k < (uint32_t)LUT_SYMS) {
             const uint32_t e1 = lut1[((uint32_t)v << used) & ((1u << LUT_BITS) - 1u)];  // then zeros
             const uint32_t len = e1 & 0xffu;
-            const int delta = (int)(e1 >> 8) - R;
+            const int delta = (int)(e1 >> 8) - base;
             if (!e1 || used + len > (uint32_t)LUT_BITS) break;  // not a whole codeword of the window
-            if (delta < -128 || delta > 127) {
+            if (delta < 0 || delta > 255) {
                 if (k == 0) {
                     e = e1 >> 8;
                     used = len;
                 }
                 break;
             }
-            e |= (unsigned long long)((uint32_t)delta & 0xffu) << (8 * k);
+            e |= (unsigned long long)delta << (8 * k);
             used += len;
             ++k;
         }
         lut[v] = make_uint2((uint32_t)e, (uint32_t)(e >> 32) | (used << 8) | (k << 12));
+        symbols_here += k;
     }
+    atomicAdd(&taken, symbols_here);
     __syncthreads();
+    // A stream's bits are close to random, so this is what a lookup yields on average.  Wide
+    // codes: an entry's symbols past its number are not stored (a warp's stores meet in the
+    // banks: 2^27 codes of 7 bits 461 -> 319 us); narrow ones: all five are, in two whole words
+    // and a half, the rest to be overwritten by the next (2.6 bits: 174 us by halves, 150; by
+    // tested halves 168, and 262 against 248 where chunks differ).
+    const bool wide = taken < 5u << (LUT_BITS - 1);  // 2.5 symbols
 
     const unsigned long long chunk = (unsigned long long)blockIdx.x * per + threadIdx.x;
     const bool live = threadIdx.x < per && chunk < nchunks;
@@ -512,7 +518,7 @@ __global__ void __launch_bounds__(DEC_THREADS, 2) k_huff_decode(const uint32_t *
     int left = live ? (int)min((unsigned long long)HCHUNK, n - chunk * HCHUNK) : 0;  // codes not yet stored
     uint16_t *dst = codes + chunk * HCHUNK;
     int have = 0;         // codes in the buffer
-    const uint32_t rr = (uint32_t)R | ((uint32_t)R << 16);
+    const uint32_t base2 = (uint32_t)base | ((uint32_t)base << 16);
     while (!__all_sync(0xffffffffu, left == 0)) {
         fetch();
         cp_async_wait_pending<2>();  // what was asked for two rounds ago is there: 5 words or more
@@ -522,14 +528,23 @@ __global__ void __launch_bounds__(DEC_THREADS, 2) k_huff_decode(const uint32_t *
             const uint2 e = lut[top >> (32 - LUT_BITS)];
             uint16_t *row = reinterpret_cast<uint16_t *>(buf) + have;
             uint32_t len = (e.y >> 8) & 0xfu, k = e.y >> 12;
-            // bytes to signed halves, plus R; symbols past the entry's number are overwritten next
-            const uint32_t s01 = __vadd2(prmt(e.x, 0x9180), rr), s23 = __vadd2(prmt(e.x, 0xb3a2), rr);
-            const uint32_t s4 = prmt(e.y, 0x9180) + (uint32_t)R;
-            row[0] = (uint16_t)s01;
-            row[1] = (uint16_t)(s01 >> 16);
-            row[2] = (uint16_t)s23;
-            row[3] = (uint16_t)(s23 >> 16);
-            row[4] = (uint16_t)s4;
+            // bytes to halves, plus base (no sum leaves its half)
+            const uint32_t s01 = __byte_perm(e.x, 0, 0x4140) + base2, s23 = __byte_perm(e.x, 0, 0x4342) + base2;
+            const uint32_t s4 = (e.y & 0xffu) + (uint32_t)base;
+            if (!wide) {
+                // two whole words and the half before or after them
+                const uint32_t odd = (uint32_t)have & 1u;
+                uint32_t *pair = reinterpret_cast<uint32_t *>(row + odd);
+                pair[0] = __funnelshift_r(s01, s23, 16 * odd);
+                pair[1] = __funnelshift_r(s23, s4, 16 * odd);
+                row[odd ? 0 : 4] = (uint16_t)(odd ? s01 : s4);
+            } else {
+                row[0] = (uint16_t)s01;
+                if (k > 1) row[1] = (uint16_t)(s01 >> 16);
+                if (k > 2) row[2] = (uint16_t)s23;
+                if (k > 3) row[3] = (uint16_t)(s23 >> 16);
+                if (k > 4) row[4] = (uint16_t)s4;
+            }
             if (k == 0) {
                 uint32_t sym = e.x;
                 if (len == 0) {  // longer than the window: the canonical rule, length by length
