@@ -248,13 +248,25 @@ __global__ void __launch_bounds__(EQ_THREADS, 2) k_quality(const uint32_t *__res
         done = n4 * 4;
     }
     int pending = 0;
-    for (unsigned long long i = done + tid; i < n; i += nth) {
-        err_point(s, __ldg(x + i), __ldg(xr + i));
-        ++points;
-        if (++pending == 64) {
+    unsigned long long i = done + tid;
+    for (; i < n && i + 3 * nth < n; i += 4 * nth) {  // eight loads in flight
+        float a[4], b[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            a[j] = __ldcs(x + i + j * nth);
+            b[j] = __ldcs(xr + i + j * nth);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) err_point(s, a[j], b[j]);
+        points += 4;
+        if (++pending == 16) {
             err_flush(s);
             pending = 0;
         }
+    }
+    for (; i < n; i += nth) {  // three at most
+        err_point(s, __ldg(x + i), __ldg(xr + i));
+        ++points;
     }
     err_flush(s);
     __shared__ bool last;
