@@ -283,7 +283,7 @@ typedef struct {
     int32_t max_abs_q;    /* largest |code - R| among kept points (code != 0) */
     int32_t reserved;
     double entropy_bits;  /* -sum_c p_c log2 p_c, p_c = hist[c] / n */
-    double sse;           /* sum of (x - x')^2 over finite x, in double (NaN without x) */
+    double sse;           /* sum of (x - x')^2 over finite x, to double rounding (NaN without x) */
     double max_abs_err;   /* max |x - x'| over finite x */
     double vmin, vmax;    /* finite value range of x */
     double psnr_db;       /* 20 log10(vmax - vmin) - 10 log10(sse / n_finite); +Inf if sse = 0 */
@@ -294,8 +294,9 @@ size_t interp_quality_workspace_bytes(void);
 
 /* Fill *d_out (device) from d_hist (2R uint32) and, when both are non-NULL, from
  * d_x and d_xrec (N floats each).  Stream-ordered; d_ws holds at least
- * interp_quality_workspace_bytes() bytes.  The error sums are accumulated in double
- * in a fixed order for a given device, so they match a float64 sum to rounding. */
+ * interp_quality_workspace_bytes() bytes.  The error sums hold what sums in double hold
+ * (short chains of floats, added up in double) in a fixed order for a given device, so
+ * they match a float64 sum to rounding. */
 int interp_quality_report(const uint32_t *d_hist, int32_t radius, const float *d_x, const float *d_xrec,
                           uint64_t n, interp_quality *d_out, void *d_ws, size_t ws_bytes, interp_stream_t stream);
 

@@ -16,10 +16,10 @@
 // (strides 4, 2, 1; three axes each, a barrier between passes) on it, and the
 // next slab lands while this one is written out.
 //
-// What bounds the kernels: instructions.  A slab takes nine passes over few points each, so
-// the fixed cost of a pass (its dispatch, its barrier, the fetch of its code) counts as much
-// as its arithmetic; issue slots are 50-56% busy, HBM a third
-// (compression) and half (decompression) of its copy rate.
+// What bounds the kernels: a slab takes nine passes over few points each, so the fixed cost of
+// a pass (its dispatch, its barrier, the fetch of its code) counts as much as its arithmetic.
+// Issue slots are 48% busy in compression and 54% in decompression; of the stalls, barriers
+// and instruction fetch are 39% and 46%.  HBM runs at 34% and 48% of its copy rate (512^3).
 //
 // Work unit inside a pass: one chunk segment, i.e. the 9 points of a line
 // along the pass axis inside one chunk; its known points (even multiples of
@@ -36,10 +36,10 @@ namespace {
 
 // ------------------------------------------------------------ geometry
 // Threads per CTA.  With fewer, each warp does more of a pass per fixed cost (dispatch, index
-// set-up, barrier): compression of 512^3 382 -> 361 us from 192 to 128 threads.  Where the
-// kernel waits more than it issues, more warps are worth more: in the general passes (the
-// x-extended domain at 384^3: 287-310 us with 128 threads, 275-289 with 192) and where a CTA
-// has a slab or two to do (64^3: 17.8 -> 14.9 us).  Rows without a tensor map like 128 too (three
+// set-up, barrier): compression of 512^3 382 -> 361 us from 192 to 128 threads (350 now).  Where
+// the kernel waits more than it issues, more warps are worth more: in the general passes (the
+// x-extended domain at 384^3: 287-310 us with 128 threads, 275-289 with 192, 257-273 since
+// those no longer spill) and where a CTA has a slab or two to do (64^3: 17.8 -> 14.9 us).  Rows without a tensor map like 128 too (three
 // uneven fields 525 -> 507 us).  Decompression is 2% slower with 128 threads and 13% with 256.
 constexpr int CNT = 128, CNT_WIDE = 192, DNT = 192;
 // The passes' template parameter COMPRESS: threads of the compression kernel, 0 for decompression.
